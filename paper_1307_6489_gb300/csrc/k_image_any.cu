@@ -1,0 +1,68 @@
+// The image chain on contiguous bundles (as k_image_lean.cu) for launches with a
+// camera whose sample count or window has no specialised search (ANY = true).
+#include "k_image_chain.cuh"
+
+namespace rta {
+
+constexpr size_t SMEM_PER_SM = size_t(227) * 1024;
+
+// FILT: the form with the digital filter (LEAN = false, FILT = true).
+template <int IW, int PPT, int MB, bool NB, bool FILT = false>
+static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
+                               int* occ) {
+    auto kern = k_image_chain<IW, PPT, MB, NB, false, !FILT, FILT, true>;
+    // the dynamic shared-memory opt-in is per device; remember the largest size set
+    static size_t attr_bytes[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || attr_bytes[dev] < smem) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_bytes[dev] = smem;
+    }
+    if (occupancy_only) {
+        *occ = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, IW * 32 + 64, smem);
+    }
+    kern<<<grid, IW * 32 + 64, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+// The same tile variants as the other window modes (kVariants in k_image.cu).
+cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
+                                      bool occ_only, int* occ) {
+    // variant 4 is variant 0's tile in the 64 registers that let three CTAs share an SM; where
+    // shared memory holds fewer, its spills buy nothing (4096 pixels x 128 samples: 516 us, and
+    // 478 with variant 0's 88 registers)
+    if (v == 4 && 3 * smem > SMEM_PER_SM) v = 0;
+    if (a.pp.nbpeak) {
+        switch (v) {
+        case 0: return launch_any<8, 1, 2, true>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_any<4, 2, 2, true>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_any<8, 2, 2, true>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_any<4, 1, 2, true>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_any<8, 1, 3, true>(a, grid, smem, s, occ_only, occ);
+        default: return cudaErrorInvalidValue;
+        }
+    }
+    if (a.pp.filter) {
+        switch (v) {
+        case 0: return launch_any<8, 1, 2, false, true>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_any<4, 2, 2, false, true>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_any<8, 2, 2, false, true>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_any<4, 1, 2, false, true>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_any<8, 1, 3, false, true>(a, grid, smem, s, occ_only, occ);
+        default: return cudaErrorInvalidValue;
+        }
+    }
+    switch (v) {
+    case 0: return launch_any<8, 1, 2, false>(a, grid, smem, s, occ_only, occ);
+    case 1: return launch_any<4, 2, 2, false>(a, grid, smem, s, occ_only, occ);
+    case 2: return launch_any<8, 2, 2, false>(a, grid, smem, s, occ_only, occ);
+    case 3: return launch_any<4, 1, 2, false>(a, grid, smem, s, occ_only, occ);
+    case 4: return launch_any<8, 1, 3, false>(a, grid, smem, s, occ_only, occ);   // registers for three CTAs per SM
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace rta

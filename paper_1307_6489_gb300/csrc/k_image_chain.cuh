@@ -206,7 +206,7 @@ __device__ __forceinline__ uint32_t spread_even(uint32_t v) {
     return v;
 }
 
-__device__ __forceinline__ int best_key_generic(const uint16_t* row, int S, int W) {
+__device__ __forceinline__ int best_key_serial(const uint16_t* row, int S, int W) {
     int s = 0;
     for (int k = 0; k < W; ++k) s += row[k];
     int key = s * 128 + 127;
@@ -217,12 +217,164 @@ __device__ __forceinline__ int best_key_generic(const uint16_t* row, int S, int 
     return key;
 }
 
+// Eight words at v into u[at..at + 7]; wide: v is 16-byte aligned.
+template <int AT>
+__device__ __forceinline__ void load_words8(const uint32_t* v, bool wide, uint32_t (&u)[16]) {
+    if (wide) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint4 q = reinterpret_cast<const uint4*>(v)[k];
+            u[AT + 4 * k] = q.x; u[AT + 4 * k + 1] = q.y; u[AT + 4 * k + 2] = q.z; u[AT + 4 * k + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) u[AT + k] = v[k];
+    }
+}
+
+// The W-sample sums of the sixteen windows that start in the words u[0..7], two per word
+// (low half: the window of the word's low sample). Sums of 2, 4, 8 and 16 samples are built by
+// doubling and the bits of W pick the ones a window is made of, longest last: every shift is
+// then a whole number of words known at compile time although W is not. Halves stay below
+// 16 * 4096 = 2^16, so plain 32-bit adds carry nothing from one half into the other.
+__device__ __forceinline__ void window_words(const uint32_t (&u)[16], int W, uint32_t (&r)[8]) {
+    uint32_t p[15], t[15];
+#pragma unroll
+    for (int j = 0; j < 15; ++j) {
+        p[j] = u[j] + __byte_perm(u[j], u[j + 1], 0x5432);      // 2 samples
+        t[j] = (W & 1) ? u[j] : 0u;
+    }
+    if (W & 2) {
+#pragma unroll
+        for (int j = 0; j < 14; ++j) t[j] = p[j] + t[j + 1];
+    }
+    if (W > 3) {
+#pragma unroll
+        for (int j = 0; j < 14; ++j) p[j] += p[j + 1];          // 4 samples
+        if (W & 4) {
+#pragma unroll
+            for (int j = 0; j < 12; ++j) t[j] = p[j] + t[j + 2];
+        }
+        if (W > 7) {
+#pragma unroll
+            for (int j = 0; j < 12; ++j) p[j] += p[j + 2];      // 8 samples
+            if (W == 16) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) t[j] = p[j] + p[j + 4];
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) t[j] = p[j] + t[j + 4];
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) r[j] = t[j];
+}
+
+// The search for any sample count and any window of up to 16 samples (the cameras and windows
+// without a specialised one), eight words of window starts at a time. As in max_window6_packed,
+// samples must be below 4096 (checked), and rows that start on an odd 16-bit position are read
+// from the word below. Words read past the row's end stay inside the stage (its calibration
+// rows follow) and their windows are dropped.
+// Bound: issue slots. The serial search it replaces (two 16-bit shared loads per window start,
+// all lanes of a 256-byte row stride in one bank) took 3,583 us for 1,000 images of 4096 pixels
+// x 128 samples, W = 16; this one 478 us, of which the HBM read is 155.
+struct PackedRow {
+    const uint32_t* v;
+    int W, odd, n_pos, n_row;    // n_pos: half-word positions of window starts; n_row: words of the row
+    bool wide;
+
+    __device__ __forceinline__ PackedRow(const uint16_t* row, int S, int W_) : W(W_) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(row);
+        v = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
+        odd = (a & 2u) ? 1 : 0;
+        wide = (S & 7) == 0;     // rows of whole 16-byte pieces
+        n_pos = S - W + 1 + odd;
+        n_row = (S + odd + 1) >> 1;
+    }
+    __device__ __forceinline__ int blocks() const { return (n_pos + 15) >> 4; }
+
+    // window sums of block j0 / 8 from its words u, invalid windows as 0
+    __device__ __forceinline__ void sums(int j0, const uint32_t (&u)[16], uint32_t (&r)[8]) const {
+        window_words(u, W, r);
+        if (odd && j0 == 0) r[0] &= 0xFFFF0000u;     // the half-word before the row
+        if (2 * (j0 + 8) > n_pos) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int left = n_pos - 2 * (j0 + k);
+                r[k] = left >= 2 ? r[k] : left == 1 ? r[k] & 0xFFFFu : 0u;
+            }
+        }
+    }
+
+    // Largest sum of the blocks [b0, b1) and the first of them that holds it; any: the OR of
+    // their words (all blocks' together cover the row: a window is at most 16 samples).
+    __device__ __forceinline__ void best_of(int b0, int b1, int& best, int& best_b, uint32_t& any) const {
+        best = 0;
+        best_b = b0;
+        any = 0;
+        if (b0 >= b1) return;
+        uint32_t u[16];
+        load_words8<0>(v + 8 * b0, wide, u);
+#pragma unroll 1
+        for (int b = b0;;) {
+            const int j0 = 8 * b;
+            load_words8<8>(v + j0 + 8, wide, u);
+            if (j0 + 16 <= n_row) {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) any |= u[k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < 16; ++k) any |= j0 + k < n_row ? u[k] : 0u;
+            }
+            uint32_t r[8];
+            sums(j0, u, r);
+            const uint32_t m = __vimax3_u16x2(__vimax3_u16x2(r[0], r[1], r[2]), __vimax3_u16x2(r[3], r[4], r[5]),
+                                              __vmaxu2(r[6], r[7]));
+            const int mb = int(max(m >> 16, m & 0xFFFFu));
+            if (mb > best) {
+                best = mb;
+                best_b = b;
+            }
+            if (++b == b1) break;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) u[k] = u[k + 8];
+        }
+    }
+
+    // first window start of block b whose sum is `best`
+    __device__ __forceinline__ int start_in(int b, int best) const {
+        uint32_t u[16], r[8];
+        load_words8<0>(v + 8 * b, wide, u);
+        load_words8<8>(v + 8 * b + 8, wide, u);
+        sums(8 * b, u, r);
+        int pos = 0;
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+            const int p = 2 * (8 * b + k);
+            if (int(r[k] >> 16) == best && p + 1 < n_pos) pos = p + 1;
+            if (int(r[k] & 0xFFFFu) == best && p < n_pos && p >= odd) pos = p;
+        }
+        return pos - odd;
+    }
+};
+
+__device__ __forceinline__ int best_key_generic(const uint16_t* row, int S, int W) {
+    const PackedRow pr(row, S, W);
+    int best, b;
+    uint32_t any;
+    pr.best_of(0, pr.blocks(), best, b, any);
+    if (any & 0xF000F000u) return best_key_serial(row, S, W);
+    return best * 128 + (127 - pr.start_in(b, best));
+}
+
 // Window start and integer sum of one pixel whose S samples start at `row`
 // (shared memory), for the cameras without a specialised search.
+template <bool ANY>
 __device__ __forceinline__ void window_sum(const uint16_t* row, int S, const ProcParams& pp, int& sum, int& st) {
     const int W = pp.W;
-    if (pp.sliding) {
-        const int key = best_key_generic(row, S, W);
+    if (ANY && pp.sliding) {
+        const int key = best_key_serial(row, S, W);
         sum = key >> 7;
         st = 127 - (key & 127);
     } else {
@@ -323,7 +475,8 @@ __device__ __forceinline__ bool any_neighbour(const int4 nbr, int K, int P, cons
 
 // Tailcut cleaning on the bitmaps: core = hi (with a hi neighbour if asked),
 // mask = core | (lo with a core neighbour). Needs hi and lo filled.
-template <class Bar>
+// CLEAR: hi and lo are left zero, for the next image.
+template <bool CLEAR = false, class Bar>
 __device__ __forceinline__ void clean_bits(const DevCam& C, const ProcParams& pp, const ImgBits& b, int tid,
                                            int nthr, Bar bar) {
     const int nw = words_of(C.P);
@@ -343,7 +496,9 @@ __device__ __forceinline__ void clean_bits(const DevCam& C, const ProcParams& pp
     for (int w = tid; w < nw; w += nthr) {
         const uint32_t cb = b.core[w];
         uint32_t mb = cb;
-        for (uint32_t m = b.lo[w] & ~cb; m; m &= m - 1) {
+        const uint32_t lb = b.lo[w];
+        if (CLEAR) b.hi[w] = b.lo[w] = 0u;     // the core bits are formed: nobody else reads them
+        for (uint32_t m = lb & ~cb; m; m &= m - 1) {
             const int bit = __ffs(m) - 1;
             if (any_neighbour(__ldg(C.nb + (w * 32 + bit)), C.K, C.P, b.core)) mb |= 1u << bit;
         }
@@ -467,7 +622,7 @@ __device__ __forceinline__ void write_bad_row(rta_hillas_t* out) {
 // searches in flight. Integrated images go through two shared-memory slots (q, t
 // and the hi/lo bitmaps of one image each): the integrators fill one slot while
 // the tail warp cleans and parameterises the other.
-constexpr int NSLOT = 2;
+constexpr int NSLOT = 2;      // (the kernel's opening writes both by name)
 enum { SLOT_END = 1 };
 
 struct SlotHdr {
@@ -504,8 +659,22 @@ __host__ __device__ __forceinline__ size_t slot_bytes(int max_P) {
 // Pixels of camera S per stage: a multiple of 32 (chunks start on bitmap words)
 // that fits the stage's waveform area with 16 bytes of slack for the unaligned
 // row loads of odd sample counts.
+// Rows of 64, 96, 128 ... bytes put eight neighbouring rows on the same shared-memory banks
+// (two to eight of them; 128-bit loads are served eight lanes at a time). The kernel without a
+// specialised search stages such a chunk as SKEW_BLOCKS runs of consecutive pixels, SKEW_PAD
+// bytes between them, and gives neighbouring threads pixels of different runs: eight lanes then
+// cover all 32 banks. (16-sample rows, two to a bank, stay as they are: their runs are too short
+// to be worth eight copies.)
+constexpr int SKEW_BLOCKS = 8, SKEW_PAD = 16;
+__host__ __device__ __forceinline__ bool skewed_rows(int S) { return S >= 32 && S % 16 == 0; }
+
+// Long rows are searched by two threads each, which keeps every integrator warp busy on the
+// smaller chunks that the same stages then hold.
+__host__ __device__ __forceinline__ bool split_rows(int S) { return S >= 64; }
+
 __host__ __device__ __forceinline__ int chunk_pixels(int chunk, int stage_wave_bytes, int S) {
-    const int cp = ((stage_wave_bytes - 16) / (2 * S)) & ~31;
+    const int slack = skewed_rows(S) ? 16 + (SKEW_BLOCKS - 1) * SKEW_PAD : 16;
+    const int cp = ((stage_wave_bytes - slack) / (2 * S)) & ~31;
     return cp < chunk ? cp : chunk;
 }
 
@@ -641,7 +810,10 @@ __device__ __forceinline__ void nb_pixel(const ChainArgs& a, const ProcParams& p
 // compile-time for the specialised sliding-window cameras (the camera is the
 // same for the whole chunk, so the dispatch happens once per chunk); S == 0 is
 // the generic path with run-time S and W.
-template <int S, int W, int IT, int PPT, bool NO_INTEG, bool NO_FILTER>
+// ANY: the generic path (S == 0) searches sliding windows; without it only the fixed window is
+// left there. SKEW: chunks of skewed_rows cameras are laid out in SKEW_BLOCKS runs, and
+// split_rows cameras take two threads a pixel.
+template <int S, int W, int IT, int PPT, bool NO_INTEG, bool NO_FILTER, bool ANY = false, bool SKEW = false>
 __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
                                                 const unsigned char* buf, const int32_t* cp16, const float* cscale,
                                                 const SlotView& v, int ct, int lane, const int* wts) {
@@ -698,10 +870,21 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
     } else {
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
-            const int c = ct + k * IT;    // pixel within the chunk
+            int c = ct + k * IT;          // pixel within the chunk
+            const unsigned char* at = buf;
+            const bool skew = SKEW && skewed_rows(Sr);
+            const bool split = SKEW && split_rows(Sr);
+            const int half = split ? lane >> 4 : 0;
+            if (split) c = (c >> 5) * 16 + (lane & 15);
+            if (skew) {
+                const int rb = (h.npix + SKEW_BLOCKS - 1) / SKEW_BLOCKS, b = c % SKEW_BLOCKS;
+                at += b * (rb * 2 * Sr + SKEW_PAD) - b * rb * 2 * Sr;
+                c = c / SKEW_BLOCKS < rb ? b * rb + c / SKEW_BLOCKS : h.npix;
+            }
             bool hi = false, lo = false;
+            const unsigned here = split ? __ballot_sync(0xffffffffu, c < h.npix) : 0u;   // both lanes of a pixel or none
             if (c < h.npix) {
-                const uint16_t* row = reinterpret_cast<const uint16_t*>(buf) + size_t(c) * Sr;
+                const uint16_t* row = reinterpret_cast<const uint16_t*>(at) + size_t(c) * Sr;
                 int sum = 0, wst = 0;
                 bool done = false;
                 if constexpr (S != 0 && W == 6) {
@@ -729,16 +912,60 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                     sum = key >> 7;
                     wst = 127 - (key & 127);
                 } else {
-                    window_sum(row, h.S, pp, sum, wst);
+                    bool found = false;
+                    if (ANY && pp.sliding) {
+                        // as above: below t_lo the maximum alone is the pixel's result
+                        const PackedRow pr(row, h.S, Wr);
+                        int b0 = 0, b1 = pr.blocks(), blk;
+                        if (split) {
+                            const int mid = (b1 + 1) >> 1;
+                            if (half) b0 = mid;
+                            else b1 = mid;
+                        }
+                        uint32_t any;
+                        pr.best_of(b0, b1, sum, blk, any);
+                        if (split) {              // the lower half's lane takes the pixel
+                            const int s2 = __shfl_xor_sync(here, sum, 16), blk2 = __shfl_xor_sync(here, blk, 16);
+                            any |= __shfl_xor_sync(here, any, 16);
+                            if (s2 > sum) {
+                                sum = s2;
+                                blk = blk2;
+                            }
+                            done = half != 0;
+                        }
+                        if (!done && !(any & 0xF000F000u)) {
+                            found = true;
+                            if (!integ && !filt) {
+                                const float q0 = __fmul_rn(__int2float_rn(16 * sum - Wr * cp16[c]), cscale[c]);
+                                if (q0 < pp.t_lo) {
+                                    v.q[h.base + c] = q0;
+                                    done = true;
+                                }
+                            }
+                            if (!done) wst = pr.start_in(blk, sum);
+                        }
+                    }
+                    if (!done && !found) window_sum<ANY>(row, h.S, pp, sum, wst);
                 }
                 if (!done) emit(c, sum, wst, row, hi, lo);
             }
-            if (!integ) {
-                const uint32_t bh = __ballot_sync(0xffffffffu, hi), bl = __ballot_sync(0xffffffffu, lo);
-                const int word = (h.base + c) >> 5;
-                if (lane == 0 && word < ((h.base + h.npix + 31) >> 5)) {      // only the chunk's own words
-                    v.hi[word] = bh;
-                    v.lo[word] = bl;
+            // the slot's bitmaps are zero until here (the tail warp clears them), and most words stay so
+            if (skew || split) {                     // neighbouring threads' pixels are not neighbours
+                if (lo) {
+                    const int p = h.base + c;
+                    const uint32_t bit = 1u << (p & 31);
+                    atomicOr(&v.lo[p >> 5], bit);
+                    if (hi) atomicOr(&v.hi[p >> 5], bit);
+                }
+            } else if (!integ) {
+                const uint32_t bl = __ballot_sync(0xffffffffu, lo);
+                if (bl) {
+                    const uint32_t bh = __ballot_sync(0xffffffffu, hi);
+                    const int word = (h.base + ct - lane + k * IT) >> 5;
+                    if (lane == 0) {
+                        v.hi[word] = bh;
+                        v.lo[word] = bl;
+                    }
                 }
             }
         }
@@ -787,11 +1014,16 @@ static __device__ __forceinline__ int stream_chunk_copy(const ChainArgs& a, cons
 // integrate-only outputs. Each combination is a separate instantiation, so that
 // every kernel carries only the code of the calls it serves (branches left in,
 // even untaken, cost the hot loop instruction-cache misses and scheduling).
-template <int IW, int PPT, int MB, bool NB, bool STREAM = false, bool LEAN = false, bool FILT = false>
+// ANY: the sliding search that takes any sample count and window width; without it the kernel
+// has only the specialised ones (and the fixed window), for launches all of whose cameras have one (its code and
+// registers, left in, cost those launches 11 % on the 10,000-event bundle, 926 against 834 us).
+template <int IW, int PPT, int MB, bool NB, bool STREAM = false, bool LEAN = false, bool FILT = false,
+          bool ANY = true>
 __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArgs a) {
     static_assert(!(LEAN && FILT) && !(NB && FILT), "the filter form is of the flat-window chain");
     constexpr bool NO_INTEG = LEAN || STREAM || FILT;     // STREAM: never integrate-only
     const bool integ = !NO_INTEG && a.integrate_only;
+    constexpr bool SKEW = ANY && !NB && !STREAM;
     constexpr int IT = IW * 32;          // integrator threads
     constexpr int CHUNK = IT * PPT;      // largest chunk in pixels
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -843,6 +1075,8 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
         sm.abort = 0;
         fence_mbar_init();
     }
+    if (!NB && !integ)
+        for (int w = tid; w < 2 * maxw; w += IT + 64) slot_view(0).hi[w] = slot_view(1).hi[w] = 0u;   // hi and lo
     if (tid == 0) {
 #pragma unroll
         for (int k = 0; k < RTA_MAX_W; ++k) sm.wts[k] = a.pp.wts[k];   // constant indices: no copy of the parameters
@@ -954,7 +1188,7 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
                 if (++stage == NST) { stage = 0; phase ^= 1u; }
                 continue;
             }
-            const int CP = chunk_pixels(CHUNK, a.stage_wave_bytes, S);
+            const int CP = chunk_pixels(SKEW && split_rows(S) ? CHUNK / 2 : CHUNK, a.stage_wave_bytes, S);
             const uint16_t* src = a.wave + woff;
             int cur_seg = 0;
             for (int base = 0; base < P; base += CP) {
@@ -984,6 +1218,11 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
                 const uint64_t pol = NB ? pol_keep : pol_stream;
                 if (stream_mode) {
                     cur_seg = stream_chunk_copy(a, rec, cur_seg, base, npix, S, buf, &sm.full[stage], pol);
+                } else if (SKEW && skewed_rows(S)) {
+                    const int rb = (npix + SKEW_BLOCKS - 1) / SKEW_BLOCKS;
+                    for (int r0 = 0, at = 0; r0 < npix; r0 += rb, at += rb * 2 * S + SKEW_PAD)
+                        bulk_g2s(buf + at, src + size_t(base + r0) * S, uint32_t(min(rb, npix - r0)) * uint32_t(S) * 2u,
+                                 &sm.full[stage], pol);
                 } else {
                     bulk_g2s(buf, src + size_t(base) * S, wbytes, &sm.full[stage], pol);
                 }
@@ -1029,7 +1268,7 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
             const SlotView v = slot_view(slot);
             const DevCam C = a.arr.cams[sh.cam];
             const ImgBits ib = {v.hi, v.lo, core, maskb};
-            clean_bits(C, pp, ib, lane, 32, WarpBar());
+            clean_bits<!NB>(C, pp, ib, lane, 32, WarpBar());
             if constexpr (!NO_INTEG) {
                 if (a.mask_out) write_mask(a, C, maskb, sh.img, lane);
             }
@@ -1092,7 +1331,7 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
                 nb_keys_chunk<30, 6, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             else if (pp.W == 6 && h.S == 25)
                 nb_keys_chunk<25, 6, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
-            else
+            else if constexpr (ANY)
                 nb_keys_chunk<0, 0, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
@@ -1125,7 +1364,7 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
             else if (pp.sliding && pp.W == 5 && h.S == 16)
                 integrate_chunk<16, 5, IT, PPT, NO_INTEG, LEAN>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else
-                integrate_chunk<0, 0, IT, PPT, NO_INTEG, LEAN>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<0, 0, IT, PPT, NO_INTEG, LEAN, ANY, SKEW>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
             if (++stage == NST) { stage = 0; phase ^= 1u; }

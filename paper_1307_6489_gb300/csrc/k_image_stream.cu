@@ -7,10 +7,10 @@
 
 namespace rta {
 
-template <int IW, int PPT, int MB, bool LEAN>
+template <int IW, int PPT, int MB, bool LEAN, bool ANY>
 static cudaError_t launch_stream(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                  int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, false, true, LEAN>;
+    auto kern = k_image_chain<IW, PPT, MB, false, true, LEAN, false, ANY>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;
@@ -29,26 +29,33 @@ static cudaError_t launch_stream(const ChainArgs& a, int grid, size_t smem, cuda
 }
 
 // The same tile variants as the other window modes (kVariants in k_image.cu).
-cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
-                                        bool occ_only, int* occ) {
+template <bool ANY>
+static cudaError_t dispatch_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
+                                   int* occ) {
     if (!a.pp.filter && !occ_only) {
         switch (v) {
-        case 0: return launch_stream<8, 1, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_stream<4, 2, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_stream<8, 2, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_stream<4, 1, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_stream<8, 1, 3, true>(a, grid, smem, s, occ_only, occ);
+        case 0: return launch_stream<8, 1, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_stream<4, 2, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_stream<8, 2, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_stream<4, 1, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_stream<8, 1, 3, true, ANY>(a, grid, smem, s, occ_only, occ);
         default: return cudaErrorInvalidValue;
         }
     }
     switch (v) {
-    case 0: return launch_stream<8, 1, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 1: return launch_stream<4, 2, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 2: return launch_stream<8, 2, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 3: return launch_stream<4, 1, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 4: return launch_stream<8, 1, 3, false>(a, grid, smem, s, occ_only, occ);
+    case 0: return launch_stream<8, 1, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
+    case 1: return launch_stream<4, 2, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
+    case 2: return launch_stream<8, 2, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
+    case 3: return launch_stream<4, 1, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
+    case 4: return launch_stream<8, 1, 3, false, ANY>(a, grid, smem, s, occ_only, occ);
     default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
+                                        bool occ_only, int* occ) {
+    return a.any_window ? dispatch_stream<true>(v, a, grid, smem, s, occ_only, occ)
+                        : dispatch_stream<false>(v, a, grid, smem, s, occ_only, occ);
 }
 
 }  // namespace rta

@@ -274,6 +274,12 @@ int chain_launch_config(rta_ctx* c, int64_t n_img, int* grid, size_t* smem, int*
     return config_launch(c, cfg_of(c, kind), n_img, grid, smem, swb, kind);
 }
 
+int needs_any_window(const rta_ctx* c, const rta::ProcParams& pp) {
+    for (int t = 0; t < c->n_tel; ++t)
+        if (!rta::window_specialised(pp, c->cams[c->tel_cam[t]].S)) return 1;
+    return 0;
+}
+
 int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t* d_wave_off, const int32_t* d_img_tel,
               const int64_t* d_pix_off, int64_t n_img, const rta::ProcParams& pp, float* d_q, float* d_t,
               int64_t n_q, rta_hillas_t* d_out, int integrate_only, cudaStream_t s, unsigned int* counter,
@@ -306,6 +312,7 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
     const ChainCfg cfg = cfg_of(c, kind);
     a.nstage = std::max(2, std::min(cfg.nstage, 8));
     a.integrate_only = integrate_only;
+    a.any_window = needs_any_window(c, pp);
     a.n_img_dev = d_n_img;
     a.seg = d_seg;
     a.img_seg = d_img_seg;
@@ -1029,12 +1036,53 @@ int rta_selftest_wait_timeout(rta_ctx* c, int timeout_ms, uint64_t* waited_ns, v
     return RTA_OK;
 }
 
+// exec[k]: the pass captured with the image kernel that carries the search for any window
+// (k = 1) or only the specialised ones (k = 0). A camera registered after the capture may need
+// the other one, which is then captured at the launch.
 struct rta_graph {
     rta_ctx* ctx = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraph_t graph[2] = {};
+    cudaGraphExec_t exec[2] = {};
     unsigned int* counter = nullptr;
+    const uint16_t* d_wave;
+    int64_t n_wave;
+    const int64_t* d_wave_off;
+    const int32_t* d_img_tel;
+    const int64_t* d_n_img;
+    int64_t max_img;
+    const int32_t* d_evt_off;
+    const int64_t* d_n_evt;
+    int64_t max_evt;
+    rta::ProcParams pp;
+    rta_hillas_t* d_hillas;
+    rta_stereo_t* d_stereo;
 };
+
+static int graph_capture(rta_graph* g, int k) {
+    cudaStream_t s = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return fail(RTA_E_CUDA, "stream creation failed");
+    int rc = RTA_OK;
+    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        rc = run_chain(g->ctx, g->d_wave, g->n_wave, g->d_wave_off, g->d_img_tel, nullptr, g->max_img, g->pp, nullptr,
+                       nullptr, 0, g->d_hillas, 0, s, g->counter, g->d_n_img);
+        if (!rc)
+            rc = run_stereo(g->ctx, g->d_hillas, g->d_img_tel, g->max_img, g->d_evt_off, g->max_evt, g->d_stereo, s,
+                            g->d_n_img, g->d_n_evt);
+        cudaError_t e2 = cudaStreamEndCapture(s, &g->graph[k]);
+        if (!rc && e2 != cudaSuccess) rc = fail(RTA_E_CUDA, "capture failed: %s", cudaGetErrorString(e2));
+    } else {
+        rc = fail(RTA_E_CUDA, "cudaStreamBeginCapture: %s", cudaGetErrorString(e));
+    }
+    if (!rc && cudaGraphInstantiate(&g->exec[k], g->graph[k], 0) != cudaSuccess)
+        rc = fail(RTA_E_CUDA, "graph instantiation failed");
+    cudaStreamDestroy(s);
+    if (rc && g->graph[k]) {
+        cudaGraphDestroy(g->graph[k]);
+        g->graph[k] = nullptr;
+    }
+    return rc;
+}
 
 int rta_graph_create(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t* d_wave_off,
                      const int32_t* d_img_tel, const int64_t* d_n_img, int64_t max_img, const int32_t* d_evt_off,
@@ -1052,26 +1100,19 @@ int rta_graph_create(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const i
     rta_graph* g = new rta_graph();
     g->ctx = c;
     g->counter = take_counter(c);
-    cudaStream_t s = nullptr;
-    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) {
-        delete g;
-        return fail(RTA_E_CUDA, "stream creation failed");
-    }
-    const rta::ProcParams pp = make_pp(c, window_mode, start, W, core_needs_neighbour, t_hi, t_lo);
-    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        rc = run_chain(c, d_wave, n_wave, d_wave_off, d_img_tel, nullptr, max_img, pp, nullptr, nullptr, 0, d_hillas, 0,
-                       s, g->counter, d_n_img);
-        if (!rc) rc = run_stereo(c, d_hillas, d_img_tel, max_img, d_evt_off, max_evt, d_stereo, s, d_n_img, d_n_evt);
-        cudaError_t e2 = cudaStreamEndCapture(s, &g->graph);
-        if (!rc && e2 != cudaSuccess) rc = fail(RTA_E_CUDA, "capture failed: %s", cudaGetErrorString(e2));
-    } else {
-        rc = fail(RTA_E_CUDA, "cudaStreamBeginCapture: %s", cudaGetErrorString(e));
-    }
-    if (!rc && cudaGraphInstantiate(&g->exec, g->graph, 0) != cudaSuccess) rc = fail(RTA_E_CUDA, "graph instantiation failed");
-    cudaStreamDestroy(s);
-    if (rc) {
-        if (g->graph) cudaGraphDestroy(g->graph);
+    g->d_wave = d_wave;
+    g->n_wave = n_wave;
+    g->d_wave_off = d_wave_off;
+    g->d_img_tel = d_img_tel;
+    g->d_n_img = d_n_img;
+    g->max_img = max_img;
+    g->d_evt_off = d_evt_off;
+    g->d_n_evt = d_n_evt;
+    g->max_evt = max_evt;
+    g->pp = make_pp(c, window_mode, start, W, core_needs_neighbour, t_hi, t_lo);
+    g->d_hillas = d_hillas;
+    g->d_stereo = d_stereo;
+    if ((rc = graph_capture(g, needs_any_window(c, g->pp)))) {
         delete g;
         return rc;
     }
@@ -1083,15 +1124,19 @@ int rta_graph_launch(rta_graph* g, void* stream) {
     if (!g) return fail(RTA_E_INVALID, "graph is NULL");
     int rc = check_ctx(g->ctx);
     if (rc) return rc;
-    CUDA_TRY(cudaGraphLaunch(g->exec, (cudaStream_t)stream));
+    const int k = needs_any_window(g->ctx, g->pp);
+    if (!g->exec[k] && (rc = graph_capture(g, k))) return rc;
+    CUDA_TRY(cudaGraphLaunch(g->exec[k], (cudaStream_t)stream));
     return RTA_OK;
 }
 
 int rta_graph_destroy(rta_graph* g) {
     if (!g) return RTA_OK;
     cudaSetDevice(g->ctx->device);
-    if (g->exec) cudaGraphExecDestroy(g->exec);
-    if (g->graph) cudaGraphDestroy(g->graph);
+    for (int k = 0; k < 2; ++k) {
+        if (g->exec[k]) cudaGraphExecDestroy(g->exec[k]);
+        if (g->graph[k]) cudaGraphDestroy(g->graph[k]);
+    }
     delete g;
     return RTA_OK;
 }

@@ -25,6 +25,7 @@ struct ChainArgs {
     int stage_wave_bytes;    // multiple of 128
     int nstage;
     int integrate_only;
+    int any_window;          // some camera has no specialised window search (window_specialised)
     // a byte-stream bundle (rta_ingest's directory): wave is the stream, wave_off unused;
     // smeta: one prepared record per image (k_stream_meta)
     const rta_segment_t* seg;
@@ -32,6 +33,13 @@ struct ChainArgs {
     int64_t n_seg;
     const struct StreamImg* smeta;
 };
+
+// Whether the fused kernel has a search compiled for S samples and windows of W (the fixed
+// window needs none): launches all of whose cameras have one run the instantiations that carry
+// no other.
+inline bool window_specialised(const ProcParams& pp, int S) {
+    return !pp.sliding || ((pp.W == 6 && (S == 40 || S == 30 || S == 25)) || (pp.W == 5 && S == 16 && !pp.nbpeak));
+}
 
 // One image of a byte stream as the image kernel's producer needs it: checked
 // once (its segments tile the camera's pixels with 16-byte-aligned runs inside
@@ -106,6 +114,8 @@ cudaError_t dispatch_image_chain_nb(int v, const ChainArgs& a, int grid, size_t 
                                     int* occ);
 cudaError_t dispatch_image_chain_lean(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                       bool occ_only, int* occ);
+cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
+                                     bool occ_only, int* occ);
 cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                         bool occ_only, int* occ);
 int chain_variant_min_blocks(int v);

@@ -157,6 +157,80 @@ def test_generic_paths_and_largest_camera(kind, P, S, W, sliding):
     ctx.close()
 
 
+@pytest.mark.parametrize("kind,P,S,W", [
+    ("hex", 72, 1, 1), ("hex", 72, 2, 2), ("hex", 40, 16, 16), ("hex", 40, 17, 16), ("grid", 64, 31, 3),
+    ("hex", 331, 32, 8), ("square", 1030, 48, 5), ("hex", 152, 63, 9), ("square", 257, 64, 16), ("hex", 1855, 40, 7),
+    ("hex", 1000, 65, 2), ("square", 516, 96, 15), ("hex", 130, 100, 12), ("square", 1030, 112, 6),
+    ("hex", 264, 127, 16), ("square", 2049, 128, 4)])
+def test_any_camera_and_window(kind, P, S, W):
+    """The sliding search for cameras and windows without a specialised one: sample counts around
+    a word, a block of starts and the split of long rows, odd rows, rows that share banks, pixel
+    counts that leave a ragged last chunk, samples from 0 to 12 bits and beyond. Charges bit for
+    bit through the integrate-only call; the chain's decisions exact, its rows and the byte-wise
+    masks within the usual rules; the same through every tile shape."""
+    rng = np.random.default_rng(1000 * S + W)
+    xy, nb = synth.lattice(kind, P, 0.1)
+    n_img = 5
+    wave = rng.integers(380, 421, (n_img, P, S)).astype(np.uint16)
+    for i in range(n_img):                          # a bright blob, flat rows, rows of full scale
+        d = ((xy - xy[rng.integers(P)]) ** 2).sum(1)
+        amp = (np.array([60, 900, 3500, 60000, 200])[i] * np.exp(-d / 0.02)).astype(np.int64)
+        k0 = rng.integers(0, S)
+        wave[i, :, k0] = np.minimum(wave[i, :, k0] + amp, 65535)
+    wave[0, : P // 4] = 400                          # ties: the first window
+    wave[1, P // 2] = 4095
+    wave[2, P // 3, S // 2:] = 4096
+    wave[3, P - 1] = 65535
+    wave[4, 0] = 0
+    p16 = np.full(P, 16 * 400, np.int32)
+    scale = (1 / (16 * 8.0 * rng.uniform(0.9, 1.1, P))).astype(np.float32)
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), p16, scale)
+    d_wave = torch.from_numpy(wave.reshape(-1).view(np.int16)).cuda()
+    off = torch.arange(n_img, dtype=torch.int64, device="cuda") * (P * S)
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    pix = torch.arange(n_img, dtype=torch.int64, device="cuda") * P
+    q = torch.zeros(n_img * P, dtype=torch.float32, device="cuda")
+    t = torch.zeros_like(q)
+    hi, lo = 10.0, 5.0
+    mode = rta.RTA_WINDOW_SLIDING
+    ref_q, rows, masks = [], [], []
+    for i in range(n_img):
+        qr, tr, _, _ = oracle.integrate(wave[i], p16, scale, True, 0, W)
+        m = oracle.clean(qr, nb, hi, lo, 1)
+        ref_q.append((qr, tr))
+        masks.append(m)
+        rows.append(oracle.hillas(xy, qr, tr, m))
+    ctx.calibrate_integrate(d_wave, off, tel, pix, mode, 0, W, q, t)
+    qg, tg = q.cpu().numpy().reshape(n_img, P), t.cpu().numpy().reshape(n_img, P)
+    for i, (qr, tr) in enumerate(ref_q):
+        np.testing.assert_array_equal(qg[i].view(np.uint32), qr.view(np.uint32))
+        assert np.max(np.abs(tg[i] - tr)) <= T_ABS
+    first = None
+    for variant, stages in ((4, 2), (0, 3), (1, 2), (2, 2), (3, 4)):
+        try:
+            ctx.set_chain_config(variant, stages, 0)
+        except rta.RtaError:
+            continue                                 # no room for this camera
+        out = torch.zeros(n_img * 16, dtype=torch.float32, device="cuda")
+        mask = torch.full((n_img * P,), 7, dtype=torch.uint8, device="cuda")
+        ctx.image_chain(d_wave, off, tel, mode, 0, W, hi, lo, 1, out)
+        with_mask = torch.zeros_like(out)
+        ctx.image_chain_masks(d_wave, off, tel, pix, mode, 0, W, hi, lo, 1, mask, with_mask)
+        assert ctx.check() == 0
+        g = hillas_rows(out, n_img)
+        np.testing.assert_array_equal(g["n_pix"], np.array(rows)[:, oracle.H["n_pix"]].astype(np.int32))
+        np.testing.assert_array_equal(mask.cpu().numpy().reshape(n_img, P), np.array(masks))
+        raw = out.cpu().numpy().view(np.uint32)
+        np.testing.assert_array_equal(raw, with_mask.cpu().numpy().view(np.uint32))
+        if first is None:
+            first = raw
+            compare_hillas(g, np.array(rows), f"{kind}{P}x{S} W={W}")
+        np.testing.assert_array_equal(raw, first)
+    ctx.close()
+
+
 def test_argument_checks(arr):
     wl, ctx = arr
     dev = Dev(wl)
