@@ -58,6 +58,7 @@ struct FeatArgs {
     uint8_t* used;           // [n_img]
     float2* base;            // [n_evt]
     int32_t* n_used;         // [n_evt], -1 = malformed event
+    __nv_bfloat16* zero;     // a training step's dZ2, cleared on the way (images of no event stay zero); nullable
 };
 
 // Epilogues: ReLU(D + bias) as BF16; D where mask > 0 (the ReLU derivative) as
@@ -66,7 +67,7 @@ struct FeatArgs {
 enum { EPI_BIAS_RELU_BF16 = 0, EPI_MASK_BF16 = 1, EPI_F32_SPLIT = 2, EPI_BF16 = 3, EPI_F32_BIAS = 4 };
 
 // D[M x N] = op(A) op(B): A stored [M x K] (K-major) or [K x M] (MN-major), B
-// stored [N x K] (K-major) or [K x N] (MN-major); 16 <= N <= 256, N % 16 == 0;
+// stored [N x K] (K-major) or [K x N] (MN-major); N is 16, 64, 128, 192 or 256;
 // MN-major row counts and K-major K are multiples of 8; leading dimensions
 // and bases 16-byte aligned.
 struct GemmArgs {
@@ -95,29 +96,19 @@ struct PoolArgs {
     __nv_bfloat16* dZ2;
 };
 
-struct HeadArgs {
-    int64_t n_evt;
-    const int64_t* n_evt_dev;
-    const __nv_bfloat16* G;    // [n_evt x 256]
-    const __nv_bfloat16* V2b;  // [256 x 4]
-    const float* c2;
-    float* Y;                  // [n_evt x 4]
-    const float* dY;
-    __nv_bfloat16* dG;
-    float* dV2;
-    float* dc2;
-};
-
+// Loss terms, dL/dy and dL/dG of a training step.
 struct LossArgs {
     int64_t n_evt;
-    const int64_t* n_evt_dev;
-    const float* Y;
+    const float* Y;            // [n_evt x 4]
+    const __nv_bfloat16* G;    // [n_evt x 256]
+    const __nv_bfloat16* V2b;  // [256 x 4]
     const float2* base;
     const float* logE;
     const float2* src;
     const uint8_t* is_gamma;
     float* lterm;
     float* dY;
+    __nv_bfloat16* dG;
 };
 
 struct OutArgs {
@@ -140,29 +131,53 @@ struct InferArgs {
     OutArgs o;
 };
 
-struct AdamArgs {
-    int64_t n;
-    float* p;
-    float* m;
-    float* v;
-    const float* g;
-    __nv_bfloat16* pb;
+// The step's gradients (from the partial sums of the split weight gradients and the output layer's
+// inputs; those of b1, b2 and c1 are in g), its loss and one Adam step.
+struct UpdateArgs {
+    const float *w1, *w2, *v1;                  // [splits][K x N] partial sums
+    int n_w1, n_w2, n_v1;
+    const __nv_bfloat16* G;                     // [n_evt x 256]
+    const float *dY, *lterm;
+    int64_t n_evt;
+    float* d_loss;             // nullable
+    float* g;
+    int apply;                 // also take the Adam step
+    float *p, *m, *v;
+    __nv_bfloat16 *pb, *pk;
     float lr, b1, b2, eps, bc1, bc2;
 };
 
 cudaError_t launch_features(const FeatArgs& a, int grid, cudaStream_t s);
-// Tensor-core GEMM (tcgen05): a_mn / b_mn give the operands' storage order;
-// splits > 1 divides K (EPI_F32_SPLIT; gemm_tc_splits gives the number of
-// partial sums actually written).
-cudaError_t launch_gemm(const GemmArgs& g, bool a_mn, bool b_mn, int splits, int n_sm, cudaStream_t s);
+// A training step's kernels are launched as programmatic dependents of one another: each
+// signals at once, and waits (grid_dependency_wait) before it reads anything.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
+// Tensor-core GEMM (tcgen05) of a forward layer: A K-major, B MN-major, one split.
+cudaError_t launch_gemm(const GemmArgs& g, int n_sm, cudaStream_t s);
+// Partial sums that `splits` K-ranges of a weight gradient come to (the reduction is cut into
+// ranges of whole 64-row units).
 int gemm_tc_splits(int64_t K, int splits);
+// The backward pass of a layer in one launch: its weight gradient w (A and B MN-major, split), its
+// bias gradient (the columns of w's B, into bias) and, when x is not NULL, its input gradient
+// (both operands K-major).
+cudaError_t launch_gemm_backward(const GemmArgs& w, int splits, float* bias, const GemmArgs* x, int n_sm,
+                                 cudaStream_t s);
 cudaError_t launch_pool(const PoolArgs& a, int grid, bool bwd, cudaStream_t s);
-cudaError_t launch_head_bwd(const HeadArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_loss(const LossArgs& a, int grid, float* d_loss, cudaStream_t s);
-cudaError_t launch_colsum(const __nv_bfloat16* Xb, const float* Xf, const int64_t* rows_dev, int64_t rows, int cols,
-                          float* out, cudaStream_t s);
-cudaError_t launch_reduce_splits(const float* ws, int splits, int64_t n, float* out, cudaStream_t s);
-cudaError_t launch_adam(const AdamArgs& a, cudaStream_t s);
+cudaError_t launch_loss(const LossArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_update(const UpdateArgs& a, cudaStream_t s);
 // The whole inference in one persistent launch (one CTA per SM, n_sm of them at
 // most, each with an equal share of the image rows; programmatic dependent
 // launch), geometric fallback included.

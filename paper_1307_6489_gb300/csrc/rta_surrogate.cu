@@ -31,7 +31,11 @@ int sfail(int code, const char* fmt, ...) {
         if (e_ != cudaSuccess) return sfail(RTA_E_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
 
-constexpr int64_t SPLIT_WS = int64_t(1) << 20;   // floats of split-K partial sums
+// Partial sums of a training step's split weight gradients (floats).
+constexpr int MAX_SPLITS_V1 = 16, MAX_SPLITS_W2 = 64, MAX_SPLITS_W1 = 512;
+constexpr int64_t WS_V1 = 0, WS_W2 = WS_V1 + int64_t(MAX_SPLITS_V1) * SUR_G * SUR_G,
+                  WS_W1 = WS_W2 + int64_t(MAX_SPLITS_W2) * SUR_H * SUR_H,
+                  SPLIT_WS = WS_W1 + int64_t(MAX_SPLITS_W1) * SUR_XPAD * SUR_H;
 
 }  // namespace
 
@@ -101,10 +105,9 @@ int reserve(rta_model* md, int64_t n_img, int64_t n_evt) {
 
 int blocks_for(int64_t n, int per) { return int(std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 65535))); }
 
-// D = op(A) op(B) on the tensor cores. ta: A stored [K x M]; tb: B stored [N x K].
-int gemm(rta_model* md, const __nv_bfloat16* A, int64_t lda, bool ta, const __nv_bfloat16* B, int64_t ldb, bool tb,
-         int64_t M, int64_t N, int64_t K, int epi, const float* bias, const __nv_bfloat16* mask, int64_t ldmask,
-         __nv_bfloat16* Cb, float* Cf, int64_t ldc, int splits, cudaStream_t s, int n_store = 0) {
+rta::GemmArgs gemm_args(rta_model* md, const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb, int64_t M,
+                        int64_t N, int64_t K, int epi, const float* bias, const __nv_bfloat16* mask, int64_t ldmask,
+                        __nv_bfloat16* Cb, float* Cf, int64_t ldc, int n_store = 0) {
     rta::GemmArgs g;
     g.A = A;
     g.B = B;
@@ -122,24 +125,32 @@ int gemm(rta_model* md, const __nv_bfloat16* A, int64_t lda, bool ta, const __nv
     g.Cb = Cb;
     g.Cf = Cf;
     g.status = rta::surrogate_ctx_status(md->ctx);
-    S_TRY(rta::launch_gemm(g, ta, !tb, splits, md->n_sm, s));
+    return g;
+}
+
+// D = A B + bias of a forward layer: A stored [M x K], B stored [K x N].
+int layer(rta_model* md, const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb, int64_t M, int64_t N,
+          int64_t K, int epi, const float* bias, __nv_bfloat16* Cb, float* Cf, int64_t ldc, cudaStream_t s,
+          int n_store = 0) {
+    S_TRY(rta::launch_gemm(gemm_args(md, A, lda, B, ldb, M, N, K, epi, bias, nullptr, 0, Cb, Cf, ldc, n_store), md->n_sm,
+                           s));
     return RTA_OK;
 }
 
-// Weight gradient [M x N] = A^T B with the reduction split into K-ranges whose
-// partial sums are added in a fixed order.
-int weight_grad(rta_model* md, const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb, int64_t M,
-                int64_t N, int64_t K, float* out, cudaStream_t s) {
+// Partial sums of the weight gradient [M x N] = A^T B, the reduction split into K-ranges; the
+// number of ranges in *used (k_update adds them in order).
+int weight_splits(const rta_model* md, int64_t M, int64_t K, int max_splits, int* used) {
     const int64_t tiles = (M + 127) / 128;
-    // about one work item per SM, each at least 8 chunks (512 rows) of the reduction
+    // each range at least 8 chunks (512 rows) of the reduction
     int64_t splits = std::max<int64_t>(1, std::min<int64_t>(md->n_sm / tiles, (K + 511) / 512));
-    splits = std::min<int64_t>(splits, SPLIT_WS / (M * N));
-    const int used = rta::gemm_tc_splits(K, int(splits));
-    int rc = gemm(md, A, lda, true, B, ldb, false, M, N, K, rta::EPI_F32_SPLIT, nullptr, nullptr, 0, nullptr,
-                  md->split_ws, N, int(splits), s);
-    if (rc) return rc;
-    S_TRY(rta::launch_reduce_splits(md->split_ws, used, M * N, out, s));
-    return RTA_OK;
+    splits = std::min<int64_t>(splits, max_splits);
+    *used = rta::gemm_tc_splits(K, int(splits));
+    return int(splits);
+}
+
+rta::GemmArgs weight_grad(rta_model* md, const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb,
+                          int64_t M, int64_t N, int64_t K, float* part) {
+    return gemm_args(md, A, lda, B, ldb, M, N, K, rta::EPI_F32_SPLIT, nullptr, nullptr, 0, nullptr, part, N);
 }
 
 // Argument checks of a batch; with_workspace: also grow the layer-by-layer
@@ -155,8 +166,9 @@ int check_batch(rta_model* md, const rta_hillas_t* d_h, const int32_t* d_img_tel
     return with_workspace ? reserve(md, std::max<int64_t>(n_img, 1), std::max<int64_t>(n_evt, 1)) : RTA_OK;
 }
 
+// train: the step's dZ2 is cleared on the way.
 int forward(rta_model* md, const rta_hillas_t* d_h, const int32_t* d_img_tel, int64_t n_img, const int32_t* d_evt_off,
-            int64_t n_evt, cudaStream_t s) {
+            int64_t n_evt, bool train, cudaStream_t s) {
     rta::FeatArgs f;
     f.h = d_h;
     f.img_tel = d_img_tel;
@@ -172,15 +184,16 @@ int forward(rta_model* md, const rta_hillas_t* d_h, const int32_t* d_img_tel, in
     f.used = md->used;
     f.base = md->base;
     f.n_used = md->n_used;
+    f.zero = train ? md->dZ2 : nullptr;
     if (n_img > 0) S_TRY(cudaMemsetAsync(md->X, 0, sizeof(__nv_bfloat16) * n_img * SUR_XPAD, s));
     S_TRY(rta::launch_features(f, blocks_for(n_evt, 256 / rta::SUR_EVT_LANES), s));
     const __nv_bfloat16* pb = md->pb;
     if (n_img > 0) {
-        if ((rc = gemm(md, md->X, SUR_XPAD, false, pb + rta::OFF_W1, SUR_H, false, n_img, SUR_H, SUR_XPAD,
-                       rta::EPI_BIAS_RELU_BF16, md->p + rta::OFF_B1, nullptr, 0, md->H1, nullptr, SUR_H, 1, s)))
+        if ((rc = layer(md, md->X, SUR_XPAD, pb + rta::OFF_W1, SUR_H, n_img, SUR_H, SUR_XPAD, rta::EPI_BIAS_RELU_BF16,
+                        md->p + rta::OFF_B1, md->H1, nullptr, SUR_H, s)))
             return rc;
-        if ((rc = gemm(md, md->H1, SUR_H, false, pb + rta::OFF_W2, SUR_H, false, n_img, SUR_H, SUR_H,
-                       rta::EPI_BIAS_RELU_BF16, md->p + rta::OFF_B2, nullptr, 0, md->H2, nullptr, SUR_H, 1, s)))
+        if ((rc = layer(md, md->H1, SUR_H, pb + rta::OFF_W2, SUR_H, n_img, SUR_H, SUR_H, rta::EPI_BIAS_RELU_BF16,
+                        md->p + rta::OFF_B2, md->H2, nullptr, SUR_H, s)))
             return rc;
     }
     rta::PoolArgs pa = {};
@@ -190,13 +203,13 @@ int forward(rta_model* md, const rta_hillas_t* d_h, const int32_t* d_img_tel, in
     pa.n_used = md->n_used;
     pa.H2 = md->H2;
     pa.P = md->P;
-    S_TRY(rta::launch_pool(pa, blocks_for(n_evt, 1), false, s));
-    if ((rc = gemm(md, md->P, SUR_G, false, pb + rta::OFF_V1, SUR_G, false, n_evt, SUR_G, SUR_G, rta::EPI_BIAS_RELU_BF16,
-                   md->p + rta::OFF_C1, nullptr, 0, md->G, nullptr, SUR_G, 1, s)))
+    S_TRY(rta::launch_pool(pa, blocks_for(n_evt, 8), false, s));
+    if ((rc = layer(md, md->P, SUR_G, pb + rta::OFF_V1, SUR_G, n_evt, SUR_G, SUR_G, rta::EPI_BIAS_RELU_BF16,
+                    md->p + rta::OFF_C1, md->G, nullptr, SUR_G, s)))
         return rc;
     // output layer: Y = G V2 + c2 (V2 widened to 16 zero columns; 4 stored)
-    if ((rc = gemm(md, md->G, SUR_G, false, md->pk + rta::PK_V2P, 16, false, n_evt, 16, SUR_G, rta::EPI_F32_BIAS,
-                   md->p + rta::OFF_C2, nullptr, 0, nullptr, md->Y, 4, 1, s, 4)))
+    if ((rc = layer(md, md->G, SUR_G, md->pk + rta::PK_V2P, 16, n_evt, 16, SUR_G, rta::EPI_F32_BIAS, md->p + rta::OFF_C2,
+                    nullptr, md->Y, 4, s, 4)))
         return rc;
     return RTA_OK;
 }
@@ -438,7 +451,7 @@ int rta_surrogate_forward(rta_model* md, const rta_hillas_t* d_h, const int32_t*
     if (rc) return rc;
     if (n_evt == 0) return RTA_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    if ((rc = forward(md, d_h, d_img_tel, n_img, d_evt_off, n_evt, s))) return rc;
+    if ((rc = forward(md, d_h, d_img_tel, n_img, d_evt_off, n_evt, false, s))) return rc;
     if (d_y) S_TRY(cudaMemcpyAsync(d_y, md->Y, sizeof(float) * 4 * n_evt, cudaMemcpyDeviceToDevice, s));
     if (d_base) S_TRY(cudaMemcpyAsync(d_base, md->base, sizeof(float2) * n_evt, cudaMemcpyDeviceToDevice, s));
     return RTA_OK;
@@ -453,33 +466,31 @@ int rta_surrogate_train_step(rta_model* md, const rta_hillas_t* d_h, const int32
     if (!d_log_energy || !d_src_xy || !d_is_gamma) return sfail(RTA_E_INVALID, "NULL label pointer");
     if (!(lr >= 0.f)) return sfail(RTA_E_INVALID, "learning rate must be >= 0");
     cudaStream_t s = (cudaStream_t)stream;
-    if ((rc = forward(md, d_h, d_img_tel, n_img, d_evt_off, n_evt, s))) return rc;
+    if ((rc = forward(md, d_h, d_img_tel, n_img, d_evt_off, n_evt, true, s))) return rc;
     rta::LossArgs la = {};
     la.n_evt = n_evt;
     la.Y = md->Y;
+    la.G = md->G;
+    la.V2b = md->pb + rta::OFF_V2;
     la.base = md->base;
     la.logE = d_log_energy;
     la.src = reinterpret_cast<const float2*>(d_src_xy);
     la.is_gamma = d_is_gamma;
     la.lterm = md->lterm;
     la.dY = md->dY;
-    S_TRY(rta::launch_loss(la, blocks_for(n_evt, 256), d_loss, s));
-    // output layer
-    rta::HeadArgs ha = {};
-    ha.n_evt = n_evt;
-    ha.G = md->G;
-    ha.V2b = md->pb + rta::OFF_V2;
-    ha.dY = md->dY;
-    ha.dG = md->dG;
-    ha.dV2 = md->g + rta::OFF_V2;
-    ha.dc2 = md->g + rta::OFF_C2;
-    S_TRY(rta::launch_head_bwd(ha, blocks_for(n_evt * SUR_G, 256), s));
-    // event network
-    if ((rc = weight_grad(md, md->P, SUR_G, md->dG, SUR_G, SUR_G, SUR_G, n_evt, md->g + rta::OFF_V1, s))) return rc;
-    S_TRY(rta::launch_colsum(md->dG, nullptr, nullptr, n_evt, SUR_G, md->g + rta::OFF_C1, s));
-    if ((rc = gemm(md, md->dG, SUR_G, false, md->pb + rta::OFF_V1, SUR_G, true, n_evt, SUR_G, SUR_G, rta::EPI_BF16, nullptr,
-                   nullptr, 0, md->dP, nullptr, SUR_G, 1, s)))
-        return rc;
+    la.dG = md->dG;
+    S_TRY(rta::launch_loss(la, blocks_for(n_evt, 8), s));
+    rta::UpdateArgs u = {};
+    u.w1 = md->split_ws + WS_W1;
+    u.w2 = md->split_ws + WS_W2;
+    u.v1 = md->split_ws + WS_V1;
+    // event network: V1's gradient and dP
+    int splits = weight_splits(md, SUR_G, n_evt, MAX_SPLITS_V1, &u.n_v1);
+    rta::GemmArgs x = gemm_args(md, md->dG, SUR_G, md->pb + rta::OFF_V1, SUR_G, n_evt, SUR_G, SUR_G, rta::EPI_BF16,
+                                nullptr, nullptr, 0, md->dP, nullptr, SUR_G);
+    S_TRY(rta::launch_gemm_backward(
+        weight_grad(md, md->P, SUR_G, md->dG, SUR_G, SUR_G, SUR_G, n_evt, md->split_ws + WS_V1), splits,
+        md->g + rta::OFF_C1, &x, md->n_sm, s));
     // pooling
     rta::PoolArgs pa = {};
     pa.evt_off = d_evt_off;
@@ -489,40 +500,44 @@ int rta_surrogate_train_step(rta_model* md, const rta_hillas_t* d_h, const int32
     pa.H2 = md->H2;
     pa.dP = md->dP;
     pa.dZ2 = md->dZ2;
-    if (n_img > 0) S_TRY(cudaMemsetAsync(md->dZ2, 0, sizeof(__nv_bfloat16) * n_img * SUR_H, s));
-    S_TRY(rta::launch_pool(pa, blocks_for(n_evt, 1), true, s));
-    // per-telescope network
+    S_TRY(rta::launch_pool(pa, blocks_for(n_evt, 8), true, s));
+    // per-telescope network: W2's gradient and dZ1, then W1's (no image: no partial sums, zero gradients)
     if (n_img > 0) {
-        if ((rc = weight_grad(md, md->H1, SUR_H, md->dZ2, SUR_H, SUR_H, SUR_H, n_img, md->g + rta::OFF_W2, s)))
-            return rc;
-        S_TRY(rta::launch_colsum(md->dZ2, nullptr, nullptr, n_img, SUR_H, md->g + rta::OFF_B2, s));
-        if ((rc = gemm(md, md->dZ2, SUR_H, false, md->pb + rta::OFF_W2, SUR_H, true, n_img, SUR_H, SUR_H,
-                       rta::EPI_MASK_BF16, nullptr, md->H1, SUR_H, md->dZ1, nullptr, SUR_H, 1, s)))
-            return rc;
-        if ((rc = weight_grad(md, md->X, SUR_XPAD, md->dZ1, SUR_H, SUR_XPAD, SUR_H, n_img, md->g + rta::OFF_W1, s)))
-            return rc;
-        S_TRY(rta::launch_colsum(md->dZ1, nullptr, nullptr, n_img, SUR_H, md->g + rta::OFF_B1, s));
+        splits = weight_splits(md, SUR_H, n_img, MAX_SPLITS_W2, &u.n_w2);
+        x = gemm_args(md, md->dZ2, SUR_H, md->pb + rta::OFF_W2, SUR_H, n_img, SUR_H, SUR_H, rta::EPI_MASK_BF16, nullptr,
+                      md->H1, SUR_H, md->dZ1, nullptr, SUR_H);
+        S_TRY(rta::launch_gemm_backward(
+            weight_grad(md, md->H1, SUR_H, md->dZ2, SUR_H, SUR_H, SUR_H, n_img, md->split_ws + WS_W2), splits,
+            md->g + rta::OFF_B2, &x, md->n_sm, s));
+        splits = weight_splits(md, SUR_XPAD, n_img, MAX_SPLITS_W1, &u.n_w1);
+        S_TRY(rta::launch_gemm_backward(
+            weight_grad(md, md->X, SUR_XPAD, md->dZ1, SUR_H, SUR_XPAD, SUR_H, n_img, md->split_ws + WS_W1), splits,
+            md->g + rta::OFF_B1, nullptr, md->n_sm, s));
     } else {
         S_TRY(cudaMemsetAsync(md->g, 0, sizeof(float) * rta::OFF_V1, s));
     }
+    u.G = md->G;
+    u.dY = md->dY;
+    u.lterm = md->lterm;
+    u.n_evt = n_evt;
+    u.d_loss = d_loss;
+    u.g = md->g;
+    u.apply = apply_update != 0;
+    u.p = md->p;
+    u.m = md->m;
+    u.v = md->v;
+    u.pb = md->pb;
+    u.pk = md->pk;
+    u.lr = lr;
+    u.b1 = 0.9f;
+    u.b2 = 0.999f;
+    u.eps = 1e-8f;
     if (apply_update) {
         ++md->step;
-        rta::AdamArgs ad;
-        ad.n = rta::N_PARAM_INTERNAL;
-        ad.p = md->p;
-        ad.m = md->m;
-        ad.v = md->v;
-        ad.g = md->g;
-        ad.pb = md->pb;
-        ad.lr = lr;
-        ad.b1 = 0.9f;
-        ad.b2 = 0.999f;
-        ad.eps = 1e-8f;
-        ad.bc1 = float(1.0 - pow(0.9, double(md->step)));
-        ad.bc2 = float(1.0 - pow(0.999, double(md->step)));
-        S_TRY(rta::launch_adam(ad, s));
-        S_TRY(rta::launch_pack_tc(md->pb, md->pk, s));
+        u.bc1 = float(1.0 - pow(0.9, double(md->step)));
+        u.bc2 = float(1.0 - pow(0.999, double(md->step)));
     }
+    S_TRY(rta::launch_update(u, s));
     return RTA_OK;
 }
 

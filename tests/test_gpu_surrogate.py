@@ -119,6 +119,51 @@ def test_gradients_match_the_oracle(which, request):
         assert cos >= G_COS and rel <= G_REL, k
 
 
+def stored_gradients(p, X, used, off, logE, ddir, gam):
+    """The oracle's chain rule in FP64 with every activation and activation gradient rounded to
+    BF16 where the library stores it; (loss, gradients)."""
+    bf, n = mlp.bf16_round, len(off) - 1
+    evt = np.repeat(np.arange(n), np.diff(off))
+    cnt = np.maximum(1.0, np.bincount(evt, weights=used, minlength=n))
+    h1 = bf(mlp.relu(X @ p["W1"] + p["b1"]))
+    h2 = bf(mlp.relu(h1 @ p["W2"] + p["b2"]))
+    total = np.zeros((n, h2.shape[1]))
+    np.add.at(total, evt, h2 * used[:, None])
+    pool = bf(np.concatenate([total / mlp.POOL_DIV, total / cnt[:, None]], 1))
+    G = bf(mlp.relu(pool @ p["V1"] + p["c1"]))
+    L, dy = mlp.loss(G @ p["V2"] + p["c2"], logE, ddir, gam)
+    dG = bf((dy @ p["V2"].T) * (G > 0))
+    dP = bf(dG @ p["V1"].T)
+    H = h2.shape[1]
+    dZ2 = bf(used[:, None] * (dP[:, :H] / mlp.POOL_DIV + dP[:, H:] / cnt[:, None])[evt] * (h2 > 0))
+    dZ1 = bf((dZ2 @ p["W2"].T) * (h1 > 0))
+    return L, dict(V2=G.T @ dy, c2=dy.sum(0), V1=pool.T @ dG, c1=dG.sum(0), W2=h1.T @ dZ2, b2=dZ2.sum(0), W1=X.T @ dZ1,
+                   b1=dZ1.sum(0))
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 17, 33, 129])
+def test_gradients_of_small_batches_match_the_oracle(setup, n):
+    """Batches of one event to a few tiles: reductions shorter than a chunk, ragged row tiles, bias
+    sums of a part of a stage, events per warp and block that do not divide. Both sides round to
+    BF16 at the same places, so what is left are FP32 sums (1e-6) and the roundings they tip over
+    (one in 2,000 values by 2^-8, 1e-4 of a norm per layer): 2e-3."""
+    s = setup
+    wl, d = s["wl"], s["d"]
+    off = wl.evt_off[: n + 1]
+    n_img = int(off[-1])
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    rta.rta_surrogate_train_step(s["model"], d["h"].data_ptr(), d["img_tel"].data_ptr(), n_img,
+                                 d["evt_off"].data_ptr(), n, d["logE"].data_ptr(), d["src"].data_ptr(),
+                                 d["gam"].data_ptr(), 1e-3, 0, loss.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    g = rta.unpack_params(rta.rta_surrogate_get_params(s["model"], 1))
+    L_ref, g_ref = stored_gradients(s["p"], mlp.bf16_round(s["X"][:n_img]), s["used"][:n_img].astype(np.float64), off,
+                                    np.log10(wl.truth[:n, 0]), wl.truth[:n, 1:3] - s["base"][:n], wl.truth[:n, 5] == 0)
+    assert float(loss.item()) == pytest.approx(L_ref, rel=2e-3)
+    for k in g_ref:
+        a, r = g[k].reshape(-1).astype(np.float64), g_ref[k].reshape(-1)
+        assert np.linalg.norm(a - r) <= 2e-3 * np.linalg.norm(r), k
+
+
 def test_adam_step_moves_each_weight_by_lr_against_its_gradient(setup):
     s = setup
     wl, d = s["wl"], s["d"]
