@@ -14,9 +14,9 @@
 //
 // Checks: every packet gets the oracle's checks in the oracle's order (framing,
 // fixed header fields, camera, segment order, CRC, capacity); the fault reported
-// is the one of the earliest packet. The CRC (optional) is computed per packet
-// by a warp: each lane four pieces, four bytes per step with four lookup
-// tables, and the pieces combined in GF(2)[x] modulo the generator.
+// is the one of the earliest packet. The CRC (optional) is computed by warps,
+// each up to 32 KiB of a packet, folded in registers, and the parts combined in
+// GF(2)[x] modulo the generator.
 #include <algorithm>
 
 #include "rta_launch.cuh"
@@ -261,6 +261,8 @@ __global__ void __launch_bounds__(256) k_pkt_check(const IngestArgs a) {
         // the stream may not end inside an image (only when the walk reached the end)
         if (!err && k == a.hdr->n_pk - 1 && !a.hdr->walk_err && f.first + f.n < f.P) err = RTA_STREAM_SEGMENT;
         a.pk_err[k] = err;
+        a.pk_len[k] = f.length;
+        a.pk_crc[k] = 0u;
         a.pk_scan[k] = (uint64_t(f.first == 0) << 32) | uint64_t(new_event);
     }
 }
@@ -268,134 +270,134 @@ __global__ void __launch_bounds__(256) k_pkt_check(const IngestArgs a) {
 // ---------------------------------------------------------------- CRC
 namespace {
 
-// Product of two polynomials of degree < 16 modulo x^16 + x^12 + x^5 + 1.
-__device__ __forceinline__ uint32_t gf_mulmod(uint32_t x, uint32_t y) {
+// Product of two polynomials of degree < 16 (degree < 31): a multiply by one bit of x is a shift
+// of y or nothing.
+__device__ __forceinline__ uint32_t gf_mul(uint32_t x, uint32_t y) {
     uint32_t p = 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-        if ((y >> i) & 1u) p ^= x << i;
+    for (int i = 0; i < 16; ++i) p ^= (x & (1u << i)) * y;
+    return p;
+}
+
+// A polynomial of degree < 31 modulo x^16 + x^12 + x^5 + 1: the part at x^16 and above, taken
+// down three times.
+__device__ __forceinline__ uint32_t gf_mod(uint32_t p) {
 #pragma unroll
-    for (int i = 30; i >= 16; --i)
-        if ((p >> i) & 1u) p ^= 0x11021u << (i - 16);
-    return p & 0xFFFFu;
-}
-
-__device__ __forceinline__ uint32_t gf_pow(uint32_t b, int e) {
-    uint32_t r = 1;
-    while (e) {
-        if (e & 1) r = gf_mulmod(r, b);
-        b = gf_mulmod(b, b);
-        e >>= 1;
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t t = p >> 16;
+        p = (p & 0xFFFFu) ^ t ^ (t << 5) ^ (t << 12);
     }
-    return r;
+    return p;
 }
 
-constexpr int CRC_X16 = RTA_PKT_MAX_BYTES / 16 + 1;
-constexpr int CRC_THREADS = 1024;                 // one CTA per SM (the lane tables fill most of its shared memory)
-constexpr int CRC_STRIDE_WORDS = 32;             // a lane's 16-byte words are this far apart
-constexpr size_t CRC_LANE_TABLE_BYTES = size_t(6) * 256 * 32 * 4;
-constexpr size_t CRC_SMEM_BYTES =
-    CRC_LANE_TABLE_BYTES + 2 * (size_t(6) * 256 + CRC_X16 + 64 + CRC_X16 / 64 + 1);
-static_assert(CRC_SMEM_BYTES <= 227 * 1024, "shared memory per CTA");
+// x^(128 k) modulo the generator, k < 256: a register carried over k 16-byte words of zeros.
+struct CrcPowers {
+    uint16_t x[256];
+    constexpr CrcPowers() : x() {
+        uint32_t r = 1;
+        for (int k = 0; k < 256; ++k) {
+            x[k] = uint16_t(r);
+            for (int i = 0; i < 128; ++i) r = (r & 0x8000u) ? ((r << 1) ^ 0x11021u) : (r << 1);
+        }
+    }
+};
+__device__ constexpr CrcPowers kCrcPowers{};
+
+constexpr int CRC_THREADS = 256;
+constexpr int CRC_BLOCK = 4096;                   // bytes a warp takes per step
+constexpr int CRC_UNIT = 8;                       // steps of a work unit at most
+static_assert(CRC_UNIT <= 8, "the folded words' top byte");
+constexpr int CRC_UNITS = (RTA_PKT_MAX_BYTES / CRC_BLOCK + CRC_UNIT - 1) / CRC_UNIT;   // units of the longest packet
 
 }  // namespace
 
-// One warp per packet. For a correct packet, running the CRC register over all
-// L bytes -- the CRC field included, most significant byte first -- ends at 0
-// (the register after the message equals the field, and two bytes equal to the
-// register clear it). The register is linear in the message, so the packet's
-// 16-byte words can be taken in any grouping: lane l takes words l, l + 32, ...
-// (the warp reads 512 contiguous bytes a step), forms each word's CRC from a zero
-// register (four bytes a step through four lookup tables) and folds it into its
-// own register, which is carried over the 512-byte stride between its words by
-// two more tables (multiplication by x^4096 modulo the generator). At the end
-// each lane's register is carried to the packet's end by x^(8 k), k the bytes
-// after its last word, from a table over multiples of 16 bytes; the preset
-// register 0xFFFF is carried likewise; the XOR of all of it must be 0. Every
-// lane has its own copy of the tables in shared memory, so a warp's lookups hit
-// 32 different banks.
-__global__ void __launch_bounds__(CRC_THREADS, 1) k_pkt_crc(const IngestArgs a) {
-    extern __shared__ __align__(16) unsigned char crc_smem[];
-    uint16_t* T = reinterpret_cast<uint16_t*>(crc_smem + CRC_LANE_TABLE_BYTES); // [6][256]
-    uint16_t* X16 = T + 6 * 256;                                                // x^(128 k) mod G
-    uint16_t* A = X16 + CRC_X16;
-    uint16_t* B = A + 64;
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        uint32_t r = uint32_t(i) << 8;
-        for (int k = 0; k < 8; ++k) r = (r & 0x8000u) ? ((r << 1) ^ 0x1021u) : (r << 1);
-        T[i] = uint16_t(r);
-    }
-    const uint32_t x128 = gf_pow(2u, 128);          // x^128 = 16 zero bytes
-    if (threadIdx.x < 64) A[threadIdx.x] = uint16_t(gf_pow(x128, threadIdx.x));
-    if (threadIdx.x < CRC_X16 / 64 + 1) B[threadIdx.x] = uint16_t(gf_pow(gf_pow(x128, 64), threadIdx.x));
-    __syncthreads();
-    const uint32_t K = gf_pow(2u, 8 * 16 * CRC_STRIDE_WORDS);     // one lane's stride: 32 words
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        // T[k][x]: byte x followed by k zero bytes, register starting at zero
-        uint32_t r = T[i];
-        for (int k = 1; k < 4; ++k) {
-            r = ((r << 8) & 0xFFFFu) ^ T[(r >> 8) & 0xFFu];
-            T[k * 256 + i] = uint16_t(r);
-        }
-        // register (x : 0) and (0 : x) carried over one lane stride of zero bytes
-        T[4 * 256 + i] = uint16_t(gf_mulmod(uint32_t(i) << 8, K));
-        T[5 * 256 + i] = uint16_t(gf_mulmod(uint32_t(i), K));
-    }
-    for (int k = threadIdx.x; k < CRC_X16; k += blockDim.x) X16[k] = uint16_t(gf_mulmod(A[k & 63], B[k >> 6]));
-    __syncthreads();
-    // one copy of the six tables per lane: entry (k, x) of lane l at byte
-    // 65536 (k >> 1) + 256 x + 128 (k & 1) + 4 l, so that every lookup of a warp hits
-    // 32 different banks and a lookup's offset is one byte permute of the index
-    // byte and 4 l (the table's constant part goes into the load's immediate)
-    for (int w = threadIdx.x; w < 6 * 256 * 32; w += blockDim.x) {
-        const int k = w >> 13, x = (w >> 5) & 255, l = w & 31;
-        *reinterpret_cast<uint32_t*>(crc_smem + 65536 * (k >> 1) + 256 * x + 128 * (k & 1) + 4 * l) = T[k * 256 + x];
-    }
-    __syncthreads();
+// For a correct packet, running the CRC register over all L bytes -- the CRC field included,
+// most significant byte first -- ends at 0 (the register after the message equals the field,
+// and two bytes equal to the register clear it). The register is linear in the message, so the
+// packet's 16-byte words can be taken in any grouping, and zeros in front of the message do not
+// count: the packet is cut into 4096-byte blocks from its end, the first one padded in front.
+// A warp step takes a block, eight words a lane (l, l + 32, ...: coalesced). The same word of the
+// next block follows 8 * 4096 bits later, and since x has order 32767 modulo the generator,
+// x^32768 is x: a lane's words of successive blocks fold into one polynomial, R <- R x + word, a
+// funnel shift and an XOR per 32 bits. At the end of a unit (up to CRC_UNIT blocks) the folded
+// words' registers come from byte-parallel arithmetic -- a 32-bit register holds the same byte of
+// four of them, and a byte step is nine shifts and three-input logic operations for all four
+//   t = hi ^ d; t ^= t >> 4;  hi = lo ^ t << 4 ^ t >> 3;  lo = t ^ t << 5   (per byte, truncated)
+// -- each is carried to the end of its block by x^(128 k), the warp's sum over the blocks that
+// follow by a power of x below 16, and XORed into the packet's register; the preset 0xFFFF is
+// the first two bytes inverted. 0 must be left.
+// Bound: memory. A 0.5 GB stream takes 87 us, 5.9 TB/s (225 us with four lookup tables
+// per lane in shared memory, a packet to a warp: 9,900 packets on 4,864 warps, three rounds; 107
+// with every word's register formed in byte-parallel arithmetic: integer issue).
+__global__ void __launch_bounds__(CRC_THREADS, 3) k_pkt_crc(const IngestArgs a) {
     const int lane = threadIdx.x & 31;
-    const uint32_t l4 = uint32_t(lane) * 4u;
-    // entry of table k at the index in byte j of v (byte permute: l4 in byte 0, the
-    // index byte in byte 1, zeros above)
-    auto look = [&](int k, uint32_t v, int j) {
-        const uint32_t off = __byte_perm(v, l4, 0x7604u | (uint32_t(j) << 4));
-        return *reinterpret_cast<const uint32_t*>(crc_smem + off + 65536 * (k >> 1) + 128 * (k & 1));
-    };
-    const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
     const int64_t n = a.hdr->n_pk < a.seg_cap + 1 ? a.hdr->n_pk : a.seg_cap + 1;
-    for (int64_t k = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); k < n; k += warps) {
-        const int64_t pos = a.pk_off[k];
-        const uint4* p = reinterpret_cast<const uint4*>(a.stream + pos);
-        PktFields f;
-        pkt_check(a.stream, pos, a.n_bytes, a.arr, f);
-        const int L = f.length;                           // multiple of 16
-        const int words = L >> 4;
-        // lane l takes words l, l + 32, ...: one coalesced 512-byte load per warp and
-        // step, issued one step ahead. Its register r covers its words with zeros
-        // between them: r <- r x^(8 * 512) + CRC_0(word), the word's own CRC from a
-        // zero register.
-        uint32_t r = 0;
-        int w = lane;
-        uint4 qn = w < words ? __ldg(p + w) : make_uint4(0, 0, 0, 0);
-        int last = -1;
-        for (; w < words; w += CRC_STRIDE_WORDS) {
-            const uint4 q = qn;
-            if (w + CRC_STRIDE_WORDS < words) qn = __ldg(p + w + CRC_STRIDE_WORDS);
-            const uint32_t ws[4] = {q.x, q.y, q.z, q.w};
-            uint32_t c = 0;
+    const int64_t tickets = n * CRC_UNITS;
+    unsigned long long ticket = 0;               // lane 0's, asked for a unit ahead
+    if (lane == 0) ticket = atomicAdd(&a.hdr->crc_ticket, 1ull);
+    for (;;) {
+        const int64_t unit = int64_t(__shfl_sync(0xffffffffu, ticket, 0));
+        if (unit >= tickets) break;
+        if (lane == 0) ticket = atomicAdd(&a.hdr->crc_ticket, 1ull);
+        const int64_t k = unit / CRC_UNITS;
+        const int part = int(unit % CRC_UNITS);
+        const int L = a.pk_len[k], words = L >> 4;               // L is a multiple of 16
+        const int blocks = (words + 255) >> 8, pad = blocks * 256 - words;
+        const int b0 = part * CRC_UNIT, b1 = min(blocks, b0 + CRC_UNIT);
+        if (b0 >= b1) continue;
+        const uint4* p = reinterpret_cast<const uint4*>(a.stream + a.pk_off[k]);
+        uint32_t R[8][5] = {};                    // most significant word first
+#pragma unroll 1
+        for (int b = b0; b < b1; ++b) {
+            const int w0 = b * 256 + lane - pad;
+            uint4 q[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) q[j] = w0 + 32 * j >= 0 ? __ldg(p + w0 + 32 * j) : make_uint4(0u, 0u, 0u, 0u);
+            if (b == 0) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (w0 + 32 * j == 0) q[j].x ^= 0xFFFFu;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                R[j][0] = __funnelshift_l(R[j][1], R[j][0], 1);
+                R[j][1] = __funnelshift_l(R[j][2], R[j][1], 1) ^ __byte_perm(q[j].x, 0u, 0x0123);
+                R[j][2] = __funnelshift_l(R[j][3], R[j][2], 1) ^ __byte_perm(q[j].y, 0u, 0x0123);
+                R[j][3] = __funnelshift_l(R[j][4], R[j][3], 1) ^ __byte_perm(q[j].z, 0u, 0x0123);
+                R[j][4] = (R[j][4] << 1) ^ __byte_perm(q[j].w, 0u, 0x0123);
+            }
+        }
+        uint32_t v = 0;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            uint32_t hi = 0u, lo = 0u;
+            auto byte_step = [&](uint32_t d) {
+                uint32_t t = hi ^ d;
+                t ^= (t >> 4) & 0x0F0F0F0Fu;
+                hi = lo ^ ((t << 4) & 0xF0F0F0F0u) ^ ((t >> 3) & 0x1F1F1F1Fu);
+                lo = t ^ ((t << 5) & 0xE0E0E0E0u);
+            };
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                const uint32_t A = R[4 * g][k], B = R[4 * g + 1][k], C = R[4 * g + 2][k], D = R[4 * g + 3][k];
+                const uint32_t ab0 = __byte_perm(A, B, 0x5140), cd0 = __byte_perm(C, D, 0x5140);
+                if (k > 0) {                      // the first word holds at most CRC_UNIT - 1 bits
+                    const uint32_t ab1 = __byte_perm(A, B, 0x7362), cd1 = __byte_perm(C, D, 0x7362);
+                    byte_step(__byte_perm(ab1, cd1, 0x7632));
+                    byte_step(__byte_perm(ab1, cd1, 0x5410));
+                    byte_step(__byte_perm(ab0, cd0, 0x7632));
+                }
+                byte_step(__byte_perm(ab0, cd0, 0x5410));
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const uint32_t x = ws[j];
-                const uint32_t u = c ^ __byte_perm(x, 0u, 0x4401u);     // register ^ (b0 : b1)
-                c = look(3, u, 1) ^ look(2, u, 0) ^ look(1, x, 2) ^ look(0, x, 3);
+                const uint32_t r = __byte_perm(lo, hi, 0x0040u | uint32_t(j * 0x11)) & 0xFFFFu;
+                v ^= gf_mul(r, kCrcPowers.x[255 - lane - 32 * (4 * g + j)]);
             }
-            r = look(4, r, 1) ^ look(5, r, 0) ^ c;
-            last = w;
         }
-        // carried to the packet's end; the preset register 0xFFFF likewise
-        uint32_t v = last >= 0 ? gf_mulmod(r, X16[words - 1 - last]) : 0u;
-        if (lane == 0) v ^= gf_mulmod(0xFFFFu, X16[words]);
+#pragma unroll
         for (int o = 16; o; o >>= 1) v ^= __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0 && v != 0 && a.pk_err[k] == 0) a.pk_err[k] = RTA_STREAM_CRC;
+        if (lane == 0) atomicXor(a.pk_crc + k, gf_mod(gf_mul(gf_mod(v), 1u << (blocks - b1))));
     }
 }
 
@@ -472,6 +474,7 @@ __global__ void __launch_bounds__(1024) k_pkt_final(const IngestArgs a) {
     a.pk_scan[k] = incl;
     const int64_t img = int64_t(incl >> 32) - 1, evt = int64_t(incl & 0xFFFFFFFFull) - 1;
     int err = a.pk_err[k];
+    if (!err && a.pk_crc[k] != 0u) err = RTA_STREAM_CRC;
     if (!err && (k >= a.seg_cap || img >= a.img_cap || evt >= a.evt_cap)) err = RTA_STREAM_CAPACITY;
     a.pk_err[k] = err;
     if (err) atomicMin(reinterpret_cast<unsigned long long*>(&a.hdr->first_bad_pk), (unsigned long long)k);
@@ -598,18 +601,9 @@ cudaError_t launch_ingest(const IngestArgs& a, int verify_crc, int n_sm, cudaStr
     const int g = int(std::min<int64_t>((max_pk + 255) / 256, int64_t(n_sm) * 8));
     k_pkt_check<<<g, 256, 0, s>>>(a);
     if (verify_crc) {
-        // the dynamic shared-memory opt-in is per device
-        static bool attr_set[64] = {};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-            if ((e = cudaFuncSetAttribute(k_pkt_crc, cudaFuncAttributeMaxDynamicSharedMemorySize, int(CRC_SMEM_BYTES))) !=
-                cudaSuccess)
-                return e;
-            if (dev >= 0 && dev < 64) attr_set[dev] = true;
-        }
+        // three CTAs an SM; warps take units as they finish others
         const int64_t wpb = CRC_THREADS / 32;
-        k_pkt_crc<<<int(std::min<int64_t>((max_pk + wpb - 1) / wpb, int64_t(n_sm))), CRC_THREADS, CRC_SMEM_BYTES, s>>>(a);
+        k_pkt_crc<<<int(std::min<int64_t>((max_pk * CRC_UNITS + wpb - 1) / wpb, int64_t(n_sm) * 3)), CRC_THREADS, 0, s>>>(a);
     }
     k_pkt_scan_local<<<unsigned(n_blk), 1024, 0, s>>>(a);
     k_pkt_scan_blocks<<<1, 1024, 0, s>>>(a, n_blk);

@@ -1289,7 +1289,7 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
     const size_t b_err = up(sizeof(int) * size_t(max_pk));
     const size_t b_scan = up(sizeof(unsigned long long) * size_t(max_pk));
     const size_t b_blk = up(sizeof(unsigned long long) * size_t(n_blk));
-    const size_t need = b_chunks + b_hdr + b_off + b_err + b_scan + b_blk;
+    const size_t need = b_chunks + b_hdr + b_off + 3 * b_err + b_scan + b_blk;
     if (need > c->ingest_bytes) {
         CUDA_TRY(cudaStreamSynchronize(s));
         cudaFree(c->d_ingest);
@@ -1308,8 +1308,10 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
     a.hdr = reinterpret_cast<rta::IngHdr*>(w + b_chunks);
     a.pk_off = reinterpret_cast<int64_t*>(w + b_chunks + b_hdr);
     a.pk_err = reinterpret_cast<int*>(w + b_chunks + b_hdr + b_off);
-    a.pk_scan = reinterpret_cast<unsigned long long*>(w + b_chunks + b_hdr + b_off + b_err);
-    a.blk_sum = reinterpret_cast<unsigned long long*>(w + b_chunks + b_hdr + b_off + b_err + b_scan);
+    a.pk_len = reinterpret_cast<int*>(w + b_chunks + b_hdr + b_off + b_err);
+    a.pk_crc = reinterpret_cast<unsigned int*>(w + b_chunks + b_hdr + b_off + 2 * b_err);
+    a.pk_scan = reinterpret_cast<unsigned long long*>(w + b_chunks + b_hdr + b_off + 3 * b_err);
+    a.blk_sum = reinterpret_cast<unsigned long long*>(w + b_chunks + b_hdr + b_off + 3 * b_err + b_scan);
     a.seg = d_seg;
     a.seg_cap = seg_cap;
     a.img_seg = d_img_seg;

@@ -164,6 +164,7 @@ struct IngHdr {
     long long n_pk;          // packets on the chain (before a framing fault)
     long long first_bad_pk;  // earliest packet with a fault
     long long walk_err_pos;
+    unsigned long long crc_ticket;   // next unit of the CRC check
     int walk_err;
     int error;
 };
@@ -176,6 +177,8 @@ struct IngestArgs {
     IngHdr* hdr;
     int64_t* pk_off;             // seg_cap + 1
     int* pk_err;
+    int* pk_len;                 // bytes of each packet
+    unsigned int* pk_crc;        // CRC register after the whole packet (0: correct, or not checked)
     unsigned long long* pk_scan;
     unsigned long long* blk_sum;
     rta_segment_t* seg;
