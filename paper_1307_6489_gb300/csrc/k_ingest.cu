@@ -4,10 +4,11 @@
 // the image kernel reads each chunk of pixels from the segment that holds it.
 //
 // Framing: packets follow one another and only a walk from byte 0 knows where
-// they start. The stream is cut into 1 MiB pieces. Each piece looks for its
-// first valid packet (16-byte aligned positions, a header whose fields hold and
-// whose successor's header holds too; 256 positions per round) and walks from
-// there to the end of the piece. The walks must join up: piece b's first packet
+// they start. The stream is cut into pieces (128 KiB to 1 MiB). Each piece looks
+// for its first valid packet (16-byte aligned positions, a header whose fields
+// hold and whose successor's header holds too; 1,024 positions per round) and walks
+// from there to the end of the piece, keeping the first 32 packets' positions.
+// The walks must join up: piece b's first packet
 // is where piece b-1's walk ended. Where they do not (a fault, or a payload that
 // happens to look like a header) a single thread walks on from the last joined
 // position, and the piece counts are redone from that walk.
@@ -25,8 +26,9 @@ namespace rta {
 
 namespace {
 
-constexpr int64_t ING_CHUNK = int64_t(1) << 20;
 constexpr int ING_SCAN_THREADS = 256;
+constexpr int ING_SCAN_UNROLL = 4;                // positions a thread looks at per round
+constexpr int ING_JOIN_SMEM = 4096;               // pieces whose counts the join keeps in shared memory
 
 struct PktFields {
     int apid, seq_flags, length, first, n, P, S;
@@ -51,10 +53,10 @@ __device__ __forceinline__ uint32_t be32(const uint4& a, const uint4& b, int i) 
 
 // The oracle's framing, header and camera checks of the packet at pos (16-byte
 // aligned), in its order; fills f when the header could be read.
-__device__ int pkt_check(const uint8_t* s, int64_t pos, int64_t n_bytes, const DevArray& arr, PktFields& f) {
-    if (n_bytes - pos < 48) return RTA_STREAM_FRAMING;
-    const uint4* h = reinterpret_cast<const uint4*>(s + pos);
-    const uint4 a = __ldg(h), b = __ldg(h + 1);
+// pkt_check: the packet at pos; header_check: the same from the header's 32 bytes, once at least
+// 48 bytes are known to be left.
+__device__ int header_check(const uint4& a, const uint4& b, int64_t pos, int64_t n_bytes, const DevArray& arr,
+                            PktFields& f) {
     const uint32_t w0 = be16(a, b, 0), w1 = be16(a, b, 2);
     f.apid = int(w0 & 0x7FFu);
     f.seq_flags = int(w1 >> 14);
@@ -81,6 +83,19 @@ __device__ int pkt_check(const uint8_t* s, int64_t pos, int64_t n_bytes, const D
     return RTA_STREAM_OK;
 }
 
+__device__ int pkt_check(const uint8_t* s, int64_t pos, int64_t n_bytes, const DevArray& arr, PktFields& f) {
+    if (n_bytes - pos < 48) return RTA_STREAM_FRAMING;
+    const uint4* h = reinterpret_cast<const uint4*>(s + pos);
+    return header_check(__ldg(h), __ldg(h + 1), pos, n_bytes, arr, f);
+}
+
+// The fixed fields in a header's first 16 bytes: version, type and secondary-header bits, PUS
+// version, service and subservice. What fails here fails pkt_check.
+__device__ __forceinline__ bool header_like(const uint4& a) {
+    return (a.x & 0xF8u) == 0x08u && (a.y >> 16) == ((uint32_t(RTA_PKT_SERVICE) << 8) | 0x10u) &&
+           (a.z & 0xFFu) == RTA_PKT_SUBSERVICE;
+}
+
 // A position where a packet can start: its checks hold and so do its successor's.
 __device__ __forceinline__ bool plausible_start(const uint8_t* s, int64_t pos, int64_t n_bytes, const DevArray& arr) {
     PktFields f, g;
@@ -91,64 +106,105 @@ __device__ __forceinline__ bool plausible_start(const uint8_t* s, int64_t pos, i
 
 }  // namespace
 
-__global__ void k_ingest_init(const IngestArgs a) { a.hdr->first_bad_pk = LLONG_MAX; }
+// The last block of a kernel to finish goes on with what needs all of them (no block waits).
+__device__ __forceinline__ bool last_block(unsigned int* done) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    __threadfence();
+    return last != 0;
+}
 
 // ---------------------------------------------------------------- framing
-// One block per piece: its first plausible packet start, then the walk.
+// The walk of one piece (one thread) from ch.first; returns the fault that ends it, at ch.end.
+__device__ int walk_piece(const IngestArgs& a, int64_t b, IngChunk& ch) {
+    const int64_t c1 = (b + 1) * a.chunk_bytes < a.n_bytes ? (b + 1) * a.chunk_bytes : a.n_bytes;
+    int64_t pos = ch.first;
+    int code = RTA_STREAM_OK;
+    ch.count = 0;
+    ch.last = -1;
+    auto fetch = [&](int64_t at, uint4& a0, uint4& a1) {
+        if (at < 0 || at >= c1 || a.n_bytes - at < 48) return;
+        const uint4* h = reinterpret_cast<const uint4*>(a.stream + at);
+        a0 = __ldg(h);
+        a1 = __ldg(h + 1);
+    };
+    uint4 h0 = make_uint4(0u, 0u, 0u, 0u), h1 = h0;
+    fetch(pos, h0, h1);
+    while (pos < c1) {
+        if (a.n_bytes - pos < 48) {
+            code = RTA_STREAM_FRAMING;
+            break;
+        }
+        // the next header is on its way (from the length alone) while this one is checked
+        const uint4 g0 = h0, g1 = h1;
+        const int64_t nx = pos + int(be16(g0, g1, 4)) + 7;
+        if ((nx & 15) == 0) fetch(nx, h0, h1);
+        PktFields f;
+        if ((code = header_check(g0, g1, pos, a.n_bytes, a.arr, f)) != RTA_STREAM_OK) break;
+        if (ch.count < ING_SLOTS) a.chunk_pos[b * ING_SLOTS + ch.count] = pos;
+        ch.last = pos;
+        ++ch.count;
+        pos += f.length;                          // = nx
+    }
+    ch.end = pos;
+    return code;
+}
+
+__device__ void frame_join(const IngestArgs& a);
+
+// One block per piece: its first plausible packet start, 16 KiB a round, then the walk (one
+// thread). Then the last block joins the walks.
 __global__ void __launch_bounds__(ING_SCAN_THREADS) k_frame_scan(const IngestArgs a) {
     __shared__ long long found;
     const int64_t b = blockIdx.x;
-    const int64_t c0 = b * ING_CHUNK, c1 = c0 + ING_CHUNK < a.n_bytes ? c0 + ING_CHUNK : a.n_bytes;
+    const int64_t c0 = b * a.chunk_bytes, c1 = c0 + a.chunk_bytes < a.n_bytes ? c0 + a.chunk_bytes : a.n_bytes;
     if (threadIdx.x == 0) found = b == 0 ? 0 : LLONG_MAX;
     __syncthreads();
-    if (b > 0) {
-        for (int64_t r0 = c0; r0 < c1; r0 += 16 * ING_SCAN_THREADS) {
-            const int64_t pos = r0 + 16 * int64_t(threadIdx.x);
-            if (pos < c1 && plausible_start(a.stream, pos, a.n_bytes, a.arr)) atomicMin(&found, (long long)pos);
-            __syncthreads();
-            if (found != LLONG_MAX) break;
+    for (int64_t r0 = c0; b > 0 && r0 < c1; r0 += 16 * ING_SCAN_THREADS * ING_SCAN_UNROLL) {
+        uint4 h[ING_SCAN_UNROLL];
+#pragma unroll
+        for (int k = 0; k < ING_SCAN_UNROLL; ++k) {
+            const int64_t pos = r0 + 16 * (ING_SCAN_THREADS * k + int64_t(threadIdx.x));
+            h[k] = pos < c1 && a.n_bytes - pos >= 48 ? __ldg(reinterpret_cast<const uint4*>(a.stream + pos))
+                                                     : make_uint4(0u, 0u, 0u, 0u);
         }
+#pragma unroll
+        for (int k = 0; k < ING_SCAN_UNROLL; ++k) {
+            const int64_t pos = r0 + 16 * (ING_SCAN_THREADS * k + int64_t(threadIdx.x));
+            if (header_like(h[k]) && plausible_start(a.stream, pos, a.n_bytes, a.arr)) atomicMin(&found, (long long)pos);
+        }
+        __syncthreads();
+        if (found != LLONG_MAX) break;
     }
-    if (threadIdx.x != 0) return;
-    IngChunk ch = {};
-    ch.err = 0;
-    ch.err_pos = -1;
-    if (found == LLONG_MAX) {
-        ch.first = -1;
-        ch.end = -1;
+    if (threadIdx.x == 0) {
+        IngChunk ch = {};
+        ch.first = ch.end = ch.last = -1;
+        if (found != LLONG_MAX) {
+            ch.first = found;
+            ch.err = walk_piece(a, b, ch);
+        }
         a.chunks[b] = ch;
-        return;
     }
-    ch.first = found;
-    int64_t pos = found;
-    int count = 0;
-    while (pos < c1) {
-        PktFields f;
-        const int code = pkt_check(a.stream, pos, a.n_bytes, a.arr, f);
-        if (code != RTA_STREAM_OK) {
-            ch.err = code;
-            ch.err_pos = pos;
-            break;
-        }
-        ++count;
-        pos += f.length;
-    }
-    ch.count = count;
-    ch.end = pos;
-    a.chunks[b] = ch;
+    if (last_block(&a.hdr->scan_done)) frame_join(a);
 }
 
 // Joins the walks (one block). The walks are on the true chain up to the first
 // piece whose first packet is not where the previous walk ended; from there one
 // thread walks on and rewrites the pieces' starts and counts, stopping at the
 // first framing/header/camera fault. Then an exclusive scan of the counts.
-__global__ void __launch_bounds__(1024) k_frame_join(const IngestArgs a) {
+__device__ void frame_join(const IngestArgs& a) {
     __shared__ long long first_bad;
+    __shared__ int cnt_s[ING_JOIN_SMEM];
     const int64_t nc = a.n_chunks;
     if (threadIdx.x == 0) first_bad = LLONG_MAX;
     __syncthreads();
+#pragma unroll 4
     for (int64_t b = threadIdx.x; b < nc; b += blockDim.x) {
         const IngChunk& ch = a.chunks[b];
+        if (b < ING_JOIN_SMEM) cnt_s[b] = ch.count;
         bool bad = ch.first < 0 || ch.err != 0;
         if (b > 0) bad = bad || ch.first != a.chunks[b - 1].end;
         if (bad) atomicMin(&first_bad, (long long)b);
@@ -156,6 +212,7 @@ __global__ void __launch_bounds__(1024) k_frame_join(const IngestArgs a) {
     __syncthreads();
     if (threadIdx.x == 0) {
         int64_t fb = first_bad;
+        a.hdr->first_bad_pk = LLONG_MAX;
         a.hdr->walk_err = 0;
         a.hdr->walk_err_pos = -1;
         if (fb != LLONG_MAX) {
@@ -163,92 +220,90 @@ __global__ void __launch_bounds__(1024) k_frame_join(const IngestArgs a) {
             int64_t pos = fb == 0 ? 0 : a.chunks[fb - 1].end;
             for (int64_t b = fb; b < nc; ++b) {
                 IngChunk ch = {};
-                const int64_t c1 = (b + 1) * ING_CHUNK < a.n_bytes ? (b + 1) * ING_CHUNK : a.n_bytes;
                 ch.first = pos;
-                int count = 0;
-                while (pos < c1) {
-                    PktFields f;
-                    const int code = pkt_check(a.stream, pos, a.n_bytes, a.arr, f);
-                    if (code != RTA_STREAM_OK) {
-                        a.hdr->walk_err = code;
-                        a.hdr->walk_err_pos = pos;
-                        break;
-                    }
-                    ++count;
-                    pos += f.length;
-                }
-                ch.count = count;
-                ch.end = pos;
+                const int code = walk_piece(a, b, ch);
                 a.chunks[b] = ch;
-                if (a.hdr->walk_err) {
-                    for (int64_t r = b + 1; r < nc; ++r) a.chunks[r].count = 0;
+                if (b < ING_JOIN_SMEM) cnt_s[b] = ch.count;
+                pos = ch.end;
+                if (code != RTA_STREAM_OK) {
+                    a.hdr->walk_err = code;
+                    a.hdr->walk_err_pos = pos;
+                    for (int64_t r = b + 1; r < nc; ++r) {
+                        a.chunks[r].count = 0;
+                        if (r < ING_JOIN_SMEM) cnt_s[r] = 0;
+                    }
                     break;
                 }
             }
         }
     }
     __syncthreads();
-    // exclusive scan of the pieces' packet counts, 1024 pieces at a time
+    // exclusive scan of the pieces' packet counts, a run of pieces per thread
     __shared__ long long wsum[32];
-    __shared__ long long carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t t0 = 0; t0 < nc; t0 += blockDim.x) {
-        const int64_t b = t0 + threadIdx.x;
-        const long long v = b < nc ? a.chunks[b].count : 0;
-        long long incl = v;
-        for (int d = 1; d < 32; d <<= 1) {
-            const long long u = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += u;
-        }
-        if (lane == 31) wsum[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            long long w = lane < int(blockDim.x >> 5) ? wsum[lane] : 0;
-            for (int d = 1; d < 32; d <<= 1) {
-                const long long u = __shfl_up_sync(0xffffffffu, w, d);
-                if (lane >= d) w += u;
-            }
-            wsum[lane] = w;              // inclusive over warps
-        }
-        __syncthreads();
-        const long long before = carry + (warp > 0 ? wsum[warp - 1] : 0) + incl - v;
-        if (b < nc) a.chunks[b].base = before;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = before + v;
-        __syncthreads();
+    const int64_t per = (nc + blockDim.x - 1) / blockDim.x, p0 = min((long long)nc, (long long)(per * threadIdx.x)),
+                  p1 = min((long long)nc, (long long)(p0 + per));
+    long long mine = 0;
+    auto count_of = [&](int64_t b) { return b < ING_JOIN_SMEM ? cnt_s[b] : a.chunks[b].count; };
+    for (int64_t b = p0; b < p1; ++b) mine += count_of(b);
+    long long incl = mine;
+    for (int d = 1; d < 32; d <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += u;
     }
-    if (threadIdx.x == 0) a.hdr->n_pk = carry;
-}
-
-// One block per piece: the packets' offsets (the first seg_cap + 1 of them).
-__global__ void __launch_bounds__(32) k_frame_list(const IngestArgs a) {
-    if (threadIdx.x != 0) return;
-    const IngChunk ch = a.chunks[blockIdx.x];
-    int64_t pos = ch.first;
-    for (int j = 0; j < ch.count; ++j) {
-        const int64_t k = ch.base + j;
-        if (k > a.seg_cap) break;
-        a.pk_off[k] = pos;
-        PktFields f;
-        pkt_check(a.stream, pos, a.n_bytes, a.arr, f);
-        pos += f.length;
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    long long base = incl - mine, total = 0;
+    for (int w = 0; w < int(blockDim.x >> 5); ++w) {
+        if (w < warp) base += wsum[w];
+        total += wsum[w];
     }
+    for (int64_t b = p0; b < p1; ++b) {
+        a.chunks[b].base = base;
+        base += count_of(b);
+    }
+    if (threadIdx.x == 0) a.hdr->n_pk = total;
 }
 
 // ---------------------------------------------------------------- per-packet checks
-// Segment order, and the scan values: image start (high word), event start (low).
-__global__ void __launch_bounds__(256) k_pkt_check(const IngestArgs a) {
+// One block per piece: its packets' offsets (the first seg_cap + 1 packets of the stream), from
+// the positions its walk kept and, past those, by walking on; then segment order, and the scan
+// values: image start (high word), event start (low).
+__global__ void __launch_bounds__(64) k_pkt_check(const IngestArgs a) {
+    const int64_t b = blockIdx.x;
+    const IngChunk ch = a.chunks[b];
     const int64_t n = a.hdr->n_pk < a.seg_cap + 1 ? a.hdr->n_pk : a.seg_cap + 1;
-    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
+    const int count = int(max(0ll, min((long long)ch.count, (long long)n - ch.base)));
+    if (count == 0) return;
+    const int kept = min(count, ING_SLOTS);
+    for (int j = threadIdx.x; j < kept; j += blockDim.x) a.pk_off[ch.base + j] = a.chunk_pos[b * ING_SLOTS + j];
+    if (threadIdx.x == 0 && kept < count) {
+        PktFields f;
+        int64_t pos = a.chunk_pos[b * ING_SLOTS + kept - 1];
+        for (int j = kept; j < count; ++j) {
+            pkt_check(a.stream, pos, a.n_bytes, a.arr, f);
+            pos += f.length;
+            a.pk_off[ch.base + j] = pos;
+        }
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < count; j += blockDim.x) {
+        const int64_t k = ch.base + j;
         PktFields f;
         pkt_check(a.stream, a.pk_off[k], a.n_bytes, a.arr, f);     // passed in the walk
         int err = 0;
         bool new_event = f.first == 0;
         if (k > 0) {
+            int64_t before;                      // the packet before this one, maybe an earlier piece's last
+            if (j > 0) {
+                before = a.pk_off[k - 1];
+            } else {
+                int64_t e = b - 1;
+                while (a.chunks[e].count == 0) --e;
+                before = a.chunks[e].last;
+            }
             PktFields g;
-            pkt_check(a.stream, a.pk_off[k - 1], a.n_bytes, a.arr, g);
+            pkt_check(a.stream, before, a.n_bytes, a.arr, g);
             if (g.first + g.n < g.P) {
                 if (f.apid != g.apid || f.event != g.event || f.first != g.first + g.n) err = RTA_STREAM_SEGMENT;
             } else if (f.first != 0) {
@@ -403,8 +458,10 @@ __global__ void __launch_bounds__(CRC_THREADS, 3) k_pkt_crc(const IngestArgs a) 
 
 // ---------------------------------------------------------------- scan of the packets' start flags
 // Inclusive scan of 64-bit values (image starts in the high word, event starts
-// in the low word) in blocks of 1024, then the blocks' offsets.
-__global__ void __launch_bounds__(1024) k_pkt_scan_local(const IngestArgs a) {
+// in the low word) in blocks of 1024; the last block forms the blocks' offsets.
+__device__ void scan_blocks(const IngestArgs& a, int64_t n_blk);
+
+__global__ void __launch_bounds__(1024) k_pkt_scan(const IngestArgs a) {
     __shared__ unsigned long long wsum[32];
     const int64_t n = a.hdr->n_pk < a.seg_cap + 1 ? a.hdr->n_pk : a.seg_cap + 1;
     const int64_t k = int64_t(blockIdx.x) * 1024 + threadIdx.x;
@@ -429,9 +486,10 @@ __global__ void __launch_bounds__(1024) k_pkt_scan_local(const IngestArgs a) {
     incl += warp > 0 ? wsum[warp - 1] : 0ull;
     if (k < n) a.pk_scan[k] = incl;
     if (threadIdx.x == 1023) a.blk_sum[blockIdx.x] = incl;
+    if (last_block(&a.hdr->sum_done)) scan_blocks(a, gridDim.x);
 }
 
-__global__ void __launch_bounds__(1024) k_pkt_scan_blocks(const IngestArgs a, int64_t n_blk) {
+__device__ void scan_blocks(const IngestArgs& a, int64_t n_blk) {
     // one block: exclusive offsets of the blocks, 1024 at a time
     __shared__ unsigned long long wsum[32];
     __shared__ unsigned long long carry;
@@ -465,23 +523,28 @@ __global__ void __launch_bounds__(1024) k_pkt_scan_blocks(const IngestArgs a, in
     }
 }
 
-// Adds the block offsets; then capacities, and the earliest faulty packet.
+__device__ void ingest_verdict(const IngestArgs& a);
+
+// Adds the block offsets; then the CRC, capacities, and the earliest faulty packet. The last
+// block gives the verdict.
 __global__ void __launch_bounds__(1024) k_pkt_final(const IngestArgs a) {
     const int64_t n = a.hdr->n_pk < a.seg_cap + 1 ? a.hdr->n_pk : a.seg_cap + 1;
     const int64_t k = int64_t(blockIdx.x) * 1024 + threadIdx.x;
-    if (k >= n) return;
-    const unsigned long long incl = a.pk_scan[k] + a.blk_sum[blockIdx.x];
-    a.pk_scan[k] = incl;
-    const int64_t img = int64_t(incl >> 32) - 1, evt = int64_t(incl & 0xFFFFFFFFull) - 1;
-    int err = a.pk_err[k];
-    if (!err && a.pk_crc[k] != 0u) err = RTA_STREAM_CRC;
-    if (!err && (k >= a.seg_cap || img >= a.img_cap || evt >= a.evt_cap)) err = RTA_STREAM_CAPACITY;
-    a.pk_err[k] = err;
-    if (err) atomicMin(reinterpret_cast<unsigned long long*>(&a.hdr->first_bad_pk), (unsigned long long)k);
+    if (k < n) {
+        const unsigned long long incl = a.pk_scan[k] + a.blk_sum[blockIdx.x];
+        a.pk_scan[k] = incl;
+        const int64_t img = int64_t(incl >> 32) - 1, evt = int64_t(incl & 0xFFFFFFFFull) - 1;
+        int err = a.pk_err[k];
+        if (!err && a.pk_crc[k] != 0u) err = RTA_STREAM_CRC;
+        if (!err && (k >= a.seg_cap || img >= a.img_cap || evt >= a.evt_cap)) err = RTA_STREAM_CAPACITY;
+        a.pk_err[k] = err;
+        if (err) atomicMin(reinterpret_cast<unsigned long long*>(&a.hdr->first_bad_pk), (unsigned long long)k);
+    }
+    if (last_block(&a.hdr->final_done) && threadIdx.x == 0) ingest_verdict(a);
 }
 
 // The verdict (one thread): the earliest faulty packet, else the walk's fault.
-__global__ void k_ingest_verdict(const IngestArgs a) {
+__device__ void ingest_verdict(const IngestArgs& a) {
     IngHdr& h = *a.hdr;
     const int64_t n = h.n_pk < a.seg_cap + 1 ? h.n_pk : a.seg_cap + 1;
     int64_t* c = a.counts;
@@ -586,7 +649,15 @@ cudaError_t launch_stream_meta(const ChainArgs& a, StreamImg* out, int64_t max_i
     return cudaGetLastError();
 }
 
-int64_t ingest_chunks(int64_t n_bytes) { return (n_bytes + ING_CHUNK - 1) / ING_CHUNK; }
+// A piece's walk is serial (about 0.7 us a packet), so short streams are cut into smaller pieces;
+// but every piece reads half a packet on average to find its first one, and all blocks should be
+// resident at once (eight an SM), so pieces grow with the stream, to at most 1 MiB (16 packets of
+// 64 KiB at least).
+int64_t ingest_chunk_bytes(int64_t n_bytes, int n_sm) {
+    int64_t c = int64_t(128) << 10;
+    while (c < (int64_t(1) << 20) && c * n_sm * 8 < n_bytes) c <<= 1;
+    return c;
+}
 
 cudaError_t launch_ingest(const IngestArgs& a, int verify_crc, int n_sm, cudaStream_t s) {
     const int64_t nc = a.n_chunks;
@@ -594,21 +665,16 @@ cudaError_t launch_ingest(const IngestArgs& a, int verify_crc, int n_sm, cudaStr
     const int64_t n_blk = (max_pk + 1023) / 1024;
     cudaError_t e;
     if ((e = cudaMemsetAsync(a.hdr, 0, sizeof(IngHdr), s)) != cudaSuccess) return e;
-    k_ingest_init<<<1, 1, 0, s>>>(a);
     k_frame_scan<<<unsigned(nc), ING_SCAN_THREADS, 0, s>>>(a);
-    k_frame_join<<<1, 1024, 0, s>>>(a);
-    k_frame_list<<<unsigned(nc), 32, 0, s>>>(a);
-    const int g = int(std::min<int64_t>((max_pk + 255) / 256, int64_t(n_sm) * 8));
-    k_pkt_check<<<g, 256, 0, s>>>(a);
+    k_pkt_check<<<unsigned(nc), 64, 0, s>>>(a);
     if (verify_crc) {
         // three CTAs an SM; warps take units as they finish others
         const int64_t wpb = CRC_THREADS / 32;
         k_pkt_crc<<<int(std::min<int64_t>((max_pk * CRC_UNITS + wpb - 1) / wpb, int64_t(n_sm) * 3)), CRC_THREADS, 0, s>>>(a);
     }
-    k_pkt_scan_local<<<unsigned(n_blk), 1024, 0, s>>>(a);
-    k_pkt_scan_blocks<<<1, 1024, 0, s>>>(a, n_blk);
+    k_pkt_scan<<<unsigned(n_blk), 1024, 0, s>>>(a);
     k_pkt_final<<<unsigned(n_blk), 1024, 0, s>>>(a);
-    k_ingest_verdict<<<1, 1, 0, s>>>(a);
+    const int g = int(std::min<int64_t>((max_pk + 255) / 256, int64_t(n_sm) * 8));
     k_pkt_emit<<<g, 256, 0, s>>>(a);
     return cudaGetLastError();
 }

@@ -1279,7 +1279,7 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
         CUDA_TRY(cudaMemsetAsync(d_evt_off, 0, sizeof(int32_t), s));
         return RTA_OK;
     }
-    const int64_t nc = rta::ingest_chunks(n_bytes);
+    const int64_t cb = rta::ingest_chunk_bytes(n_bytes, c->n_sm), nc = (n_bytes + cb - 1) / cb;
     const int64_t max_pk = seg_cap + 1;
     const int64_t n_blk = (max_pk + 1023) / 1024;
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
@@ -1289,7 +1289,8 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
     const size_t b_err = up(sizeof(int) * size_t(max_pk));
     const size_t b_scan = up(sizeof(unsigned long long) * size_t(max_pk));
     const size_t b_blk = up(sizeof(unsigned long long) * size_t(n_blk));
-    const size_t need = b_chunks + b_hdr + b_off + 3 * b_err + b_scan + b_blk;
+    const size_t b_pos = up(sizeof(long long) * rta::ING_SLOTS * size_t(nc));
+    const size_t need = b_chunks + b_hdr + b_off + 3 * b_err + b_scan + b_blk + b_pos;
     if (need > c->ingest_bytes) {
         CUDA_TRY(cudaStreamSynchronize(s));
         cudaFree(c->d_ingest);
@@ -1304,6 +1305,7 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
     a.stream = d_stream;
     a.n_bytes = n_bytes;
     a.n_chunks = nc;
+    a.chunk_bytes = cb;
     a.chunks = reinterpret_cast<rta::IngChunk*>(w);
     a.hdr = reinterpret_cast<rta::IngHdr*>(w + b_chunks);
     a.pk_off = reinterpret_cast<int64_t*>(w + b_chunks + b_hdr);
@@ -1312,6 +1314,7 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
     a.pk_crc = reinterpret_cast<unsigned int*>(w + b_chunks + b_hdr + b_off + 2 * b_err);
     a.pk_scan = reinterpret_cast<unsigned long long*>(w + b_chunks + b_hdr + b_off + 3 * b_err);
     a.blk_sum = reinterpret_cast<unsigned long long*>(w + b_chunks + b_hdr + b_off + 3 * b_err + b_scan);
+    a.chunk_pos = reinterpret_cast<long long*>(w + b_chunks + b_hdr + b_off + 3 * b_err + b_scan + b_blk);
     a.seg = d_seg;
     a.seg_cap = seg_cap;
     a.img_seg = d_img_seg;

@@ -152,11 +152,12 @@ cudaError_t launch_transient(const TransientArgs& t, cudaStream_t s);
 cudaError_t launch_skymap_sum(const unsigned int* slabs, unsigned long long use, unsigned int* out, cudaStream_t s);
 cudaError_t launch_stereo_to_events(const rta_stereo_t* st, int64_t n_evt, rta_event_t* ev, cudaStream_t s);
 // DL0 byte-stream ingest (k_ingest.cu).
-struct IngChunk {            // one 1 MiB piece of the stream
+constexpr int ING_SLOTS = 32;   // packet positions a piece keeps from its walk
+struct IngChunk {            // one piece of the stream
     long long first;         // its first packet (-1: none found)
+    long long last;          // its last packet
     long long end;           // where its walk stopped (>= the piece's end, or a fault)
     long long base;          // packets in the pieces before it
-    long long err_pos;
     int count;               // packets that start in it
     int err;
 };
@@ -165,6 +166,7 @@ struct IngHdr {
     long long first_bad_pk;  // earliest packet with a fault
     long long walk_err_pos;
     unsigned long long crc_ticket;   // next unit of the CRC check
+    unsigned int scan_done, sum_done, final_done;   // blocks that have finished a kernel (its last one goes on alone)
     int walk_err;
     int error;
 };
@@ -172,8 +174,9 @@ struct IngestArgs {
     DevArray arr;
     const uint8_t* stream;
     int64_t n_bytes;
-    int64_t n_chunks;
+    int64_t n_chunks, chunk_bytes;
     IngChunk* chunks;
+    long long* chunk_pos;        // ING_SLOTS per piece
     IngHdr* hdr;
     int64_t* pk_off;             // seg_cap + 1
     int* pk_err;
@@ -193,7 +196,7 @@ struct IngestArgs {
     int64_t* counts;
     unsigned int* status;
 };
-int64_t ingest_chunks(int64_t n_bytes);
+int64_t ingest_chunk_bytes(int64_t n_bytes, int n_sm);
 cudaError_t launch_ingest(const IngestArgs& a, int verify_crc, int n_sm, cudaStream_t s);
 
 // Lookup-table reconstruction and its training sums (k_lut.cu).
