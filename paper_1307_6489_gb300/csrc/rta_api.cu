@@ -341,10 +341,7 @@ int run_stereo(rta_ctx* c, const rta_hillas_t* d_h, const int32_t* d_img_tel, in
     a.n_evt_dev = d_n_evt;
     a.out = d_out;
     a.status = c->d_status;
-    const int epb = rta::stereo_events_per_block();
-    int64_t g = (n_evt + epb - 1) / epb;
-    g = std::min<int64_t>(g, int64_t(c->n_sm) * 16);
-    CUDA_TRY(rta::launch_stereo(a, int(std::max<int64_t>(g, 1)), s));
+    CUDA_TRY(rta::launch_stereo(a, c->n_sm, s));
     return RTA_OK;
 }
 

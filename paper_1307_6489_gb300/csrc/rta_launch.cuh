@@ -94,6 +94,7 @@ struct StereoArgs {
     unsigned int* status;
     int settled;               // event offsets and counts were written before the kernel this one follows
                                // on the stream started: they are read before the dependency wait
+    int per_cta;               // events a CTA takes per round (set by the launcher)
 };
 
 int chain_variant_warps(int v);
@@ -119,11 +120,10 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
 cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                         bool occ_only, int* occ);
 int chain_variant_min_blocks(int v);
-int stereo_events_per_block();
 cudaError_t launch_image_chain(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_clean(const CleanArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_hillas(const HillasArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_stereo(const StereoArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_stereo(StereoArgs a, int n_sm, cudaStream_t s);
 cudaError_t launch_wait_selftest(unsigned int* status, uint64_t timeout_ns, unsigned long long* waited_ns,
                                  cudaStream_t s);
 // stores a message for rta_last_error() on the calling thread

@@ -287,6 +287,41 @@ def test_stereo_degenerate_events(arr):
     assert g["flags"][0] == rta.RTA_SF_INVALID and g["flags"][1] == rta.RTA_SF_INVALID
 
 
+@pytest.mark.parametrize("n_evt", [1, 2, 9, 457, 913, 15000])
+def test_stereo_rows_do_not_depend_on_the_events_around(arr, n_evt):
+    """One event to more than a wave of CTAs with several events each, of 0, 1, 2, 8, 9, 24, 25 and
+    64 images (the edges of what lanes, warps and CTAs take) in turn: every row equals, bit for
+    bit, the row of the same event reconstructed alone; then with two malformed events."""
+    wl, ctx = arr
+    ref = oracle.reconstruct(wl)
+    rows32 = hillas_rows_as_f32(ref["hillas"])
+    sizes = np.array([8, 0, 24, 1, 64, 9, 2, 25], np.int64)
+    h = torch.from_numpy(np.tile(rows32, (8, 1)).reshape(-1)).cuda()
+    tel = torch.from_numpy(np.tile(wl.img_tel, 8)).cuda()
+    alone = []
+    for k, m in enumerate(sizes):                    # images k .. k + m
+        out = torch.zeros(8, dtype=torch.float32, device="cuda")
+        ctx.stereo(h[16 * k:], torch.tensor([0, int(m)], dtype=torch.int32, device="cuda"), tel[k:], out)
+        alone.append(out.cpu().numpy().view(np.uint32))
+    kind = np.arange(n_evt) % 8
+    src = torch.from_numpy(np.concatenate([np.arange(k, k + sizes[k]) for k in kind]).astype(np.int64)).cuda()
+    off = np.concatenate([[0], np.cumsum(sizes[kind])]).astype(np.int32)
+    hh, tt = h.view(-1, 16)[src].reshape(-1), tel[src]
+    out = torch.zeros(n_evt * 8, dtype=torch.float32, device="cuda")
+    ctx.stereo(hh, torch.from_numpy(off).cuda(), tt, out)
+    assert ctx.check() == 0
+    got = out.cpu().numpy().view(np.uint32).reshape(-1, 8)
+    np.testing.assert_array_equal(got, np.array(alone)[kind])
+    if n_evt > 2:
+        off[1] = len(src) + 1                        # events 0 and 1 leave the range
+        ctx.stereo(hh, torch.from_numpy(off).cuda(), tt, out)
+        with pytest.raises(rta.RtaError):
+            ctx.check()
+        bad = out.cpu().numpy().view(np.uint32).reshape(-1, 8)
+        assert bad[0, 5] == rta.RTA_SF_INVALID and bad[1, 5] == rta.RTA_SF_INVALID
+        np.testing.assert_array_equal(bad[2:], got[2:])
+
+
 def test_full_size_bundle_every_event():
     """The benchmark's workload (10,000 events, 46,292 images, ~5 GB) in the
     benchmark's launch configuration, against the oracle on every image and event:
