@@ -15,9 +15,10 @@
 //
 // FP64 runs at 2 lanes per clock per SM on this part, so a warp-wide FP64
 // instruction holds its sub-partition's pipe for a long time whatever the
-// number of active lanes. The group's events are therefore dealt round-robin
-// to the four warps (slot k -> warp k % 4, lane k / 4): the per-event sums and
-// divisions of one group run on all four sub-partitions at once.
+// number of active lanes. Four neighbouring threads therefore take one event,
+// a sum and a quotient each: an image costs a warp one addition for eight
+// events instead of four for the events of a thread each (10,000 events
+// LUT_A us; 18.6 with a thread per event).
 //
 // k_lut_train: one thread per training event, FP64 atomic sums per cell.
 // k_lut_finalize, k_lut_prepare: one thread per cell.
@@ -29,9 +30,9 @@ namespace rta {
 
 namespace {
 
-constexpr int LUT_THREADS = 128;
-constexpr int LUT_WARPS = LUT_THREADS / 32;
-constexpr int LUT_MAX_EPB = 128;    // events per group at most (one thread each)
+constexpr int LUT_THREADS = 512;
+constexpr int LUT_MAX_EPB = 128;    // events per group at most (four threads each)
+static_assert(LUT_THREADS == 4 * LUT_MAX_EPB, "four threads an event");
 constexpr int LUT_PIECE = 1024;     // per-image terms staged per pass
 
 // The lookup form of one cell (RTA_LUT_LOOKUP_BYTES = 64 bytes).
@@ -51,8 +52,9 @@ struct LutSmem {
     long long pre[LUT_MAX_EPB + 1];    // flat offset of each slot's first image in the group
     int first[LUT_MAX_EPB];            // its first image index
     float2 core[LUT_MAX_EPB];
-    double tw[LUT_PIECE], tl[LUT_PIECE], tn[LUT_PIECE], td[LUT_PIECE];
-    int tu[LUT_PIECE];                 // 1: the image is used
+    int state[LUT_MAX_EPB];            // 0 fold, 1 malformed, 2 no core, 3 no event
+    double term[4][LUT_PIECE];         // scaled width, scaled length, w_e, w_e mean_e
+    unsigned char tu[LUT_PIECE];       // 1: the image is used
 };
 
 // i with e[i] <= v < e[i + 1], -1 outside [e[0], e[n]) or for NaN. For sorted
@@ -107,7 +109,7 @@ __device__ __forceinline__ int64_t cell_index(const LutArgs& a, int cam, int iu,
 // issues each stage's loads for all of them before using any, so the chain
 // image row -> telescope -> cell costs three memory latencies per batch
 // instead of three per image.
-constexpr int LUT_ILP = 4;
+constexpr int LUT_ILP = 2;
 
 __device__ __forceinline__ void stage_terms(const LutArgs& a, LutSmem& sm, int epb, long long p0, long long p1) {
     for (long long base = p0 + threadIdx.x; base < p1; base += LUT_THREADS * LUT_ILP) {
@@ -191,10 +193,10 @@ __device__ __forceinline__ void stage_terms(const LutArgs& a, LutSmem& sm, int e
             // f0 = (1/sigma_w, 1/sigma_l), f1 = (w_e, w_e mean_e), f2 = (mean_w, mean_l), f3 = used
             const bool used = f3[u] != 0;
             const int k = int(base + u * LUT_THREADS - p0);
-            sm.tw[k] = used ? __dmul_rn(__dsub_rn(double(wid[u]), f2[u].x), f0[u].x) : 0.0;
-            sm.tl[k] = used ? __dmul_rn(__dsub_rn(double(h0[u].w), f2[u].y), f0[u].y) : 0.0;
-            sm.tn[k] = f1[u].y;
-            sm.td[k] = f1[u].x;
+            sm.term[0][k] = used ? __dmul_rn(__dsub_rn(double(wid[u]), f2[u].x), f0[u].x) : 0.0;
+            sm.term[1][k] = used ? __dmul_rn(__dsub_rn(double(h0[u].w), f2[u].y), f0[u].y) : 0.0;
+            sm.term[2][k] = f1[u].x;
+            sm.term[3][k] = f1[u].y;
             sm.tu[k] = used;
         }
     }
@@ -202,20 +204,19 @@ __device__ __forceinline__ void stage_terms(const LutArgs& a, LutSmem& sm, int e
 
 __global__ void __launch_bounds__(LUT_THREADS) k_lut_events(const LutArgs a) {
     __shared__ LutSmem sm;
+    grid_dependency_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int slot = lane * LUT_WARPS + warp;          // this thread's event in the group
+    const int slot = tid >> 2, part = tid & 3;         // this thread's event in the group and its sum
     for (int k = tid; k <= a.n_size; k += LUT_THREADS) sm.se[k] = a.size_edges[k];
     for (int k = tid; k <= a.n_dist; k += LUT_THREADS) sm.de[k] = a.dist_edges[k];
     const int epb = a.events_per_block;
     const double cw_lo = a.cut[0], cw_hi = a.cut[1], cl_lo = a.cut[2], cl_hi = a.cut[3];
     for (int64_t e0 = int64_t(blockIdx.x) * epb; e0 < a.n_evt; e0 += int64_t(gridDim.x) * epb) {
-        const int64_t e = e0 + slot;
-        const bool mine = slot < epb && e < a.n_evt;
-        int state = 3;                       // 0 fold, 1 malformed, 2 no core, 3 no event
-        if (slot < epb) {
+        if (tid < epb) {
+            const int64_t e = e0 + tid;
+            int state = 3, i0 = 0;
             long long cnt = 0;
-            int i0 = 0;
-            if (mine) {
+            if (e < a.n_evt) {
                 i0 = a.evt_off[e];
                 const int i1 = a.evt_off[e + 1];
                 if (i0 < 0 || i1 < i0 || i1 > a.n_img) {
@@ -229,12 +230,13 @@ __global__ void __launch_bounds__(LUT_THREADS) k_lut_events(const LutArgs a) {
                     } else {
                         state = 0;
                         cnt = i1 - i0;
-                        sm.core[slot] = make_float2(s0.z, s0.w);
+                        sm.core[tid] = make_float2(s0.z, s0.w);
                     }
                 }
             }
-            sm.cnt[slot] = cnt;
-            sm.first[slot] = i0;
+            sm.state[tid] = state;
+            sm.cnt[tid] = cnt;
+            sm.first[tid] = i0;
         }
         __syncthreads();
         // exclusive scan of the slots' image counts: warp 0, four slots a lane
@@ -261,51 +263,46 @@ __global__ void __launch_bounds__(LUT_THREADS) k_lut_events(const LutArgs a) {
         __syncthreads();
         const long long total = sm.pre[epb];
         const long long my0 = slot < epb ? sm.pre[slot] : 0, my1 = slot < epb ? sm.pre[slot + 1] : 0;
-        double sw = 0.0, sl = 0.0, sn = 0.0, sd = 0.0;
+        double sum = 0.0;                    // of the scaled widths, scaled lengths, w_e or w_e mean_e
         int n = 0;
         for (long long p0 = 0; p0 < total; p0 += LUT_PIECE) {
             const long long p1 = min(total, p0 + LUT_PIECE);
             stage_terms(a, sm, epb, p0, p1);
             __syncthreads();
             const long long j0 = max(my0, p0), j1 = min(my1, p1);
+            const double* term = sm.term[part];
             for (long long j = j0; j < j1; ++j) {
                 const int k = int(j - p0);
                 if (sm.tu[k]) {
                     ++n;
-                    sw = __dadd_rn(sw, sm.tw[k]);
-                    sl = __dadd_rn(sl, sm.tl[k]);
-                    sn = __dadd_rn(sn, sm.tn[k]);
-                    sd = __dadd_rn(sd, sm.td[k]);
+                    sum = __dadd_rn(sum, term[k]);
                 }
             }
             __syncthreads();
         }
-        if (mine) {
-            float4 o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
+        // mscw, mscl = sums / n; log E = sum(w_e mean_e) / sum(w_e); sigma = sqrt(1 / sum(w_e)): one
+        // quotient per thread (thread 2 forms sigma, thread 3 log E)
+        const double sd = __shfl_sync(0xffffffffu, sum, (lane & ~3) + 2);
+        const int state = slot < epb ? sm.state[slot] : 3;
+        const bool fold = state == 0 && n > 0;
+        const double top = part == 2 ? 1.0 : sum, under = part < 2 ? double(n) : sd;
+        double v = 0.0;
+        if (fold) v = __ddiv_rn(top, under);
+        if (fold && part == 2) v = __dsqrt_rn(v);
+        const bool in = fold && part < 2 && (part == 0 ? cw_lo <= v && v <= cw_hi : cl_lo <= v && v <= cl_hi);
+        const unsigned inside = __ballot_sync(0xffffffffu, in);
+        if (state != 3) {
+            // the row: log E, sigma, mscw, mscl, n_used, flags, two reserved
+            float* row = reinterpret_cast<float*>(a.out + e0 + slot);
+            row[part == 0 ? 2 : part == 1 ? 3 : part == 2 ? 1 : 0] = __double2float_rn(v);
             uint32_t flags = 0;
-            int n_used = 0;
-            if (state == 1) {
-                flags = RTA_LF_MALFORMED;
-                n_used = -1;
-            } else if (state == 2) {
-                flags = RTA_LF_NO_CORE;
-            } else if (n == 0) {
-                flags = RTA_LF_NO_IMAGE;
-            } else {
-                const double dn = double(n);
-                const double mscw = __ddiv_rn(sw, dn), mscl = __ddiv_rn(sl, dn);
-                const double le = __ddiv_rn(sn, sd);
-                const double sg = __dsqrt_rn(__ddiv_rn(1.0, sd));
-                if (cw_lo <= mscw && mscw <= cw_hi && cl_lo <= mscl && mscl <= cl_hi) flags = RTA_LF_GAMMA;
-                n_used = n;
-                o0 = make_float4(__double2float_rn(le), __double2float_rn(sg), __double2float_rn(mscw),
-                                 __double2float_rn(mscl));
-            }
-            o1.x = __int_as_float(n_used);
-            o1.y = __uint_as_float(flags);
-            float4* op = reinterpret_cast<float4*>(a.out + e);
-            op[0] = o0;
-            op[1] = o1;
+            if (state == 1) flags = RTA_LF_MALFORMED;
+            else if (state == 2) flags = RTA_LF_NO_CORE;
+            else if (n == 0) flags = RTA_LF_NO_IMAGE;
+            else if (((inside >> (lane & ~3)) & 3u) == 3u) flags = RTA_LF_GAMMA;
+            row[4 + part] = part == 0   ? __int_as_float(state == 1 ? -1 : state == 0 ? n : 0)
+                            : part == 1 ? __uint_as_float(flags)
+                                        : 0.f;
         }
         __syncthreads();   // the next group reuses the shared arrays
     }
@@ -392,8 +389,18 @@ int lut_events_per_block(int64_t n_evt, int n_sm) {
 }
 
 cudaError_t launch_lut_reconstruct(const LutArgs& a, int grid, cudaStream_t s) {
-    k_lut_events<<<grid, LUT_THREADS, 0, s>>>(a);
-    return cudaGetLastError();
+    // a programmatic dependent: its blocks start while the kernel before (the stereo kernel, as a
+    // rule) ends, and wait for it before they read anything
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(LUT_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_lut_events, a);
 }
 
 cudaError_t launch_lut_accumulate(const LutArgs& a, int grid, cudaStream_t s) {

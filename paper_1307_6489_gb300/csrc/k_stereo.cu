@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(ST_NT, ST_CTAS) k_stereo(const StereoArgs a) {
     // event offsets and counts settled (written before the image kernel started), they are
     // read before the dependency wait: the counts and the first round's offsets.
     if (!a.settled) grid_dependency_wait();
+    grid_dependents_launch();
     // a graph captured at capacity reads the bundle's counts at run time
     const int64_t n_evt = a.n_evt_dev ? min(*a.n_evt_dev, a.n_evt) : a.n_evt;
     const int64_t n_img = a.n_img_dev ? min(*a.n_img_dev, a.n_img) : a.n_img;
