@@ -123,10 +123,10 @@ int chain_chunk_pixels(int v, int stage_wave_bytes, int S) {
     return chunk_pixels(kVariants[v].iw * 32 * kVariants[v].ppt, stage_wave_bytes, S);
 }
 
-template <int IW, int PPT, int MB, bool ANY>
+template <int IW, int PPT, int MB, int OUT, bool ANY>
 static cudaError_t launch_t(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                             int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, false, false, false, false, ANY>;
+    auto kern = k_image_chain<IW, PPT, MB, false, false, 2, OUT, ANY>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;
@@ -144,30 +144,32 @@ static cudaError_t launch_t(const ChainArgs& a, int grid, size_t smem, cudaStrea
     return cudaGetLastError();
 }
 
-template <bool ANY>
+template <int OUT, bool ANY>
 static cudaError_t dispatch(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
                             int* occ) {
     switch (v) {
-    case 0: return launch_t<8, 1, 2, ANY>(a, grid, smem, s, occ_only, occ);
-    case 1: return launch_t<4, 2, 2, ANY>(a, grid, smem, s, occ_only, occ);
-    case 2: return launch_t<8, 2, 2, ANY>(a, grid, smem, s, occ_only, occ);
-    case 3: return launch_t<4, 1, 2, ANY>(a, grid, smem, s, occ_only, occ);
-    case 4: return launch_t<8, 1, 3, ANY>(a, grid, smem, s, occ_only, occ);   // registers for three CTAs per SM
+    case 0: return launch_t<8, 1, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
+    case 1: return launch_t<4, 2, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
+    case 2: return launch_t<8, 2, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
+    case 3: return launch_t<4, 1, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
+    case 4: return launch_t<8, 1, 3, OUT, ANY>(a, grid, smem, s, occ_only, occ);   // registers for three CTAs per SM
     default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_image_chain(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
-    // the image chain on a contiguous bundle (flat window, neighbour-peak window or
-    // digital filter) runs a lean instantiation; the per-pixel outputs (integrate-only
-    // charges and times, cleaning masks) are compiled into the general ones only
+    // the image chain's rows on a contiguous bundle; then byte streams, and the per-pixel outputs
+    // (integrate-only charges and times, cleaning masks)
     if (!a.smeta && !a.integrate_only && !a.mask_out)
         return a.any_window ? dispatch_image_chain_any(v, a, grid, smem, s, false, nullptr)
                             : dispatch_image_chain_lean(v, a, grid, smem, s, false, nullptr);
     if (a.pp.nbpeak) return dispatch_image_chain_nb(v, a, grid, smem, s, false, nullptr);
     if (a.smeta) return dispatch_image_chain_stream(v, a, grid, smem, s, false, nullptr);
-    return a.any_window ? dispatch<true>(v, a, grid, smem, s, false, nullptr)
-                        : dispatch<false>(v, a, grid, smem, s, false, nullptr);
+    if (a.integrate_only)
+        return a.any_window ? dispatch<OUT_CHARGES, true>(v, a, grid, smem, s, false, nullptr)
+                            : dispatch<OUT_CHARGES, false>(v, a, grid, smem, s, false, nullptr);
+    return a.any_window ? dispatch<OUT_MASKS, true>(v, a, grid, smem, s, false, nullptr)
+                        : dispatch<OUT_MASKS, false>(v, a, grid, smem, s, false, nullptr);
 }
 
 int chain_occupancy(int v, size_t smem, int kind) {
@@ -175,7 +177,7 @@ int chain_occupancy(int v, size_t smem, int kind) {
     ChainArgs dummy = {};
     const cudaError_t e = kind == CHAIN_NB       ? dispatch_image_chain_nb(v, dummy, 0, smem, nullptr, true, &n)
                           : kind == CHAIN_STREAM ? dispatch_image_chain_stream(v, dummy, 0, smem, nullptr, true, &n)
-                                                 : dispatch<false>(v, dummy, 0, smem, nullptr, true, &n);
+                                                 : dispatch<OUT_MASKS, false>(v, dummy, 0, smem, nullptr, true, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;

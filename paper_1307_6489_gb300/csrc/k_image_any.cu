@@ -10,7 +10,7 @@ constexpr size_t SMEM_PER_SM = size_t(227) * 1024;
 template <int IW, int PPT, int MB, bool NB, bool FILT = false>
 static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, NB, false, !FILT, FILT, true>;
+    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILT ? 1 : 0, OUT_ROWS, true>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;

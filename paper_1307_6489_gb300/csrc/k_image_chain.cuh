@@ -196,14 +196,20 @@ __device__ __forceinline__ void best_key_pair(const uint16_t* row0, int one, int
     key1 = best_key_x<S, W>(x, one, k128);
 }
 
-// Bits 0..15 of v spread to the even bit positions.
-__device__ __forceinline__ uint32_t spread_even(uint32_t v) {
-    v &= 0xFFFFu;
-    v = (v | (v << 8)) & 0x00FF00FFu;
-    v = (v | (v << 4)) & 0x0F0F0F0Fu;
-    v = (v | (v << 2)) & 0x33333333u;
-    v = (v | (v << 1)) & 0x55555555u;
-    return v;
+// First start of a window whose sum is `sum`, the largest of the row's (found by the packed
+// search): a rolled loop, taken by the few pixels that reach t_lo. Every camera shares its few
+// instructions: an unrolled search per sample count (300 instructions each) pushed the hot loop
+// out of the instruction caches.
+__device__ __forceinline__ int first_start(const uint16_t* row, int S, int W, int sum) {
+    int s = 0;
+    for (int k = 0; k < W; ++k) s += row[k];
+    int st = 0;
+#pragma unroll 1
+    while (s != sum && st < S - W) {
+        s += int(row[st + W]) - int(row[st]);
+        ++st;
+    }
+    return st;
 }
 
 __device__ __forceinline__ int best_key_serial(const uint16_t* row, int S, int W) {
@@ -215,6 +221,16 @@ __device__ __forceinline__ int best_key_serial(const uint16_t* row, int S, int W
         key = max(key, s * 128 + (127 - k));
     }
     return key;
+}
+
+// Bits 0..15 of v spread to the even bit positions.
+__device__ __forceinline__ uint32_t spread_even(uint32_t v) {
+    v &= 0xFFFFu;
+    v = (v | (v << 8)) & 0x00FF00FFu;
+    v = (v | (v << 4)) & 0x0F0F0F0Fu;
+    v = (v | (v << 2)) & 0x33333333u;
+    v = (v | (v << 1)) & 0x55555555u;
+    return v;
 }
 
 // Eight words at v into u[at..at + 7]; wide: v is 16-byte aligned.
@@ -706,13 +722,13 @@ struct NbShared {
     int* n_cand;          // candidates so far in this image
 };
 
-template <int S, int W, int IT, int PPT, bool NO_INTEG>
+template <int S, int W, int IT, int PPT, bool INTEG>
 __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
                                               const unsigned char* buf, const int32_t* cp16, const float* cscale,
                                               const NbShared& nb, const SlotView& v, int ct, int lane) {
     const int Sr = S ? S : h.S;
     const int Wr = W ? W : pp.W;
-    const bool integ = !NO_INTEG && a.integrate_only;
+    constexpr bool integ = INTEG;
 #pragma unroll
     for (int k = 0; k < PPT; ++k) {
         const int c = ct + k * IT;
@@ -727,12 +743,14 @@ __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcPara
                 int m = 0;
                 if (!integ && max_window6_packed<S>(row, m)) {
                     q0 = charge(m, Wr, cp16[c], cscale[c], num);
-                    exact = q0 >= pp.t_lo;
+                    exact = false;
+                    if (q0 >= pp.t_lo) st = first_start(row, S, W, m);
                 }
             }
             if (exact) {
                 int key;
-                if constexpr (S != 0) key = best_key_T<S, W>(row, pp.one, pp.k128);
+                if constexpr (S != 0 && !INTEG && W == 6) key = best_key_serial(row, S, W);
+                else if constexpr (S != 0) key = best_key_T<S, W>(row, pp.one, pp.k128);
                 else key = best_key_generic(row, Sr, Wr);
                 q0 = charge(key >> 7, Wr, cp16[c], cscale[c], num);
                 st = 127 - (key & 127);
@@ -761,7 +779,7 @@ __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcPara
 // among itself and its registered neighbours, then its own flat sum there, the
 // calibration multiply and the peak time; in the image chain q, t and the
 // bitmap bits go to the slot.
-template <bool NO_INTEG>
+template <bool INTEG>
 __device__ __forceinline__ void nb_pixel(const ChainArgs& a, const ProcParams& pp, const StageHdr& h, const DevCam& C,
                                          const uint64_t* key, int p, const SlotView& v) {
     uint64_t best = key[p];
@@ -790,7 +808,7 @@ __device__ __forceinline__ void nb_pixel(const ChainArgs& a, const ProcParams& p
     const int p16 = __ldg(a.arr.p16 + h.row + p);
     int num;
     const float q = charge(sum, Wr, p16, __ldg(a.arr.scale + h.row + p), num);
-    if (!NO_INTEG && a.integrate_only) {
+    if (INTEG) {
         a.q_out[h.pix_off + p] = q;
         if (a.t_out) a.t_out[h.pix_off + p] = peak_time(row, wst, Wr, p16, num);
     } else {
@@ -813,16 +831,16 @@ __device__ __forceinline__ void nb_pixel(const ChainArgs& a, const ProcParams& p
 // ANY: the generic path (S == 0) searches sliding windows; without it only the fixed window is
 // left there. SKEW: chunks of skewed_rows cameras are laid out in SKEW_BLOCKS runs, and
 // split_rows cameras take two threads a pixel.
-template <int S, int W, int IT, int PPT, bool NO_INTEG, bool NO_FILTER, bool ANY = false, bool SKEW = false>
+template <int S, int W, int IT, int PPT, bool INTEG, int FILTER, bool ANY = false, bool SKEW = false>
 __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
                                                 const unsigned char* buf, const int32_t* cp16, const float* cscale,
                                                 const SlotView& v, int ct, int lane, const int* wts) {
     const int Sr = S ? S : h.S;
     const int Wr = W ? W : pp.W;
-    // NO_INTEG / NO_FILTER: instantiations that never see the integrate-only call
-    // or the digital filter leave those branches out of their code
-    const bool integ = !NO_INTEG && a.integrate_only;
-    const bool filt = !NO_FILTER && pp.filter;
+    // INTEG: the integrate-only call; FILTER: the digital filter never (0), always (1) or as the call
+    // says (2). An instantiation carries only the code of the calls it serves.
+    constexpr bool integ = INTEG;
+    const bool filt = FILTER == 1 || (FILTER == 2 && pp.filter);
     // charge, outputs and thresholds of chunk pixel c with window sum `sum` starting at `wst`
     auto emit = [&](int c, int sum, int wst, const uint16_t* row, bool& hi, bool& lo) {
         const int p16 = cp16[c];
@@ -903,9 +921,15 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                         }
                     }
                     if (!done) {
-                        const int key = best_key_T<S, W>(row, pp.one, pp.k128);
-                        sum = key >> 7;
-                        wst = 127 - (key & 127);
+                        if (!integ && !filt && m > 0) {
+                            sum = m;
+                            wst = first_start(row, S, W, m);
+                        } else {
+                            const int key = !INTEG && FILTER == 0 ? best_key_serial(row, S, W)
+                                                                  : best_key_T<S, W>(row, pp.one, pp.k128);
+                            sum = key >> 7;
+                            wst = 127 - (key & 127);
+                        }
                     }
                 } else if constexpr (S != 0) {
                     const int key = best_key_T<S, W>(row, pp.one, pp.k128);
@@ -1008,21 +1032,21 @@ static __device__ __forceinline__ int stream_chunk_copy(const ChainArgs& a, cons
 
 // NB: the neighbour-peak window (keys and candidates in shared memory, a
 // candidate pass after each image). STREAM: a byte-stream bundle (per-image
-// records from k_stream_meta, chunks copied from the stream's segments). LEAN:
-// the image chain only, without the integrate-only outputs and the digital
-// filter; FILT: the image chain with the digital filter, without the
-// integrate-only outputs. Each combination is a separate instantiation, so that
-// every kernel carries only the code of the calls it serves (branches left in,
-// even untaken, cost the hot loop instruction-cache misses and scheduling).
+// records from k_stream_meta, chunks copied from the stream's segments).
+// FILTER: the digital filter never (0), always (1) or as the call says (2). Each
+// combination is a separate instantiation, so that every kernel carries only the
+// code of the calls it serves (branches left in, even untaken, cost the hot loop
+// instruction-cache misses and scheduling).
 // ANY: the sliding search that takes any sample count and window width; without it the kernel
 // has only the specialised ones (and the fixed window), for launches all of whose cameras have one (its code and
 // registers, left in, cost those launches 11 % on the 10,000-event bundle, 926 against 834 us).
-template <int IW, int PPT, int MB, bool NB, bool STREAM = false, bool LEAN = false, bool FILT = false,
-          bool ANY = true>
+// OUT: what a launch writes -- Hillas rows, charges and times only (the integrate-only call), or
+// rows and cleaning masks.
+enum { OUT_ROWS = 0, OUT_CHARGES = 1, OUT_MASKS = 2 };
+template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, bool ANY>
 __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArgs a) {
-    static_assert(!(LEAN && FILT) && !(NB && FILT), "the filter form is of the flat-window chain");
-    constexpr bool NO_INTEG = LEAN || STREAM || FILT;     // STREAM: never integrate-only
-    const bool integ = !NO_INTEG && a.integrate_only;
+    static_assert(!(NB && FILTER) && !(STREAM && OUT != OUT_ROWS), "the calls there are");
+    constexpr bool integ = OUT == OUT_CHARGES;
     constexpr bool SKEW = ANY && !NB && !STREAM;
     constexpr int IT = IW * 32;          // integrator threads
     constexpr int CHUNK = IT * PPT;      // largest chunk in pixels
@@ -1269,9 +1293,7 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
             const DevCam C = a.arr.cams[sh.cam];
             const ImgBits ib = {v.hi, v.lo, core, maskb};
             clean_bits<!NB>(C, pp, ib, lane, 32, WarpBar());
-            if constexpr (!NO_INTEG) {
-                if (a.mask_out) write_mask(a, C, maskb, sh.img, lane);
-            }
+            if constexpr (OUT == OUT_MASKS) write_mask(a, C, maskb, sh.img, lane);
             hillas_bits(v.q, v.t, C, maskb, sm.red, lane, 32, WarpBar(), a.out + sh.img);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.slot_free[slot]);
@@ -1326,13 +1348,13 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
             // during this image's candidate pass, after every warp has passed nb_free
             const NbShared nb = {nbk, nbc, &sm.nb_cnt[nb_img & 1]};
             if (pp.W == 6 && h.S == 40)
-                nb_keys_chunk<40, 6, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
+                nb_keys_chunk<40, 6, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             else if (pp.W == 6 && h.S == 30)
-                nb_keys_chunk<30, 6, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
+                nb_keys_chunk<30, 6, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             else if (pp.W == 6 && h.S == 25)
-                nb_keys_chunk<25, 6, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
+                nb_keys_chunk<25, 6, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             else if constexpr (ANY)
-                nb_keys_chunk<0, 0, IT, PPT, NO_INTEG>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
+                nb_keys_chunk<0, 0, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
             if (++stage == NST) { stage = 0; phase ^= 1u; }
@@ -1344,10 +1366,10 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
                 // ...so the candidate pass can look at any pixel's neighbours
                 const DevCam C = a.arr.cams[h.cam];
                 if (integ) {
-                    for (int p = ct; p < h.P; p += IT) nb_pixel<NO_INTEG>(a, pp, h, C, nbk, p, v);
+                    for (int p = ct; p < h.P; p += IT) nb_pixel<integ>(a, pp, h, C, nbk, p, v);
                 } else {
                     const int n = *nb.n_cand;
-                    for (int j = ct; j < n; j += IT) nb_pixel<NO_INTEG>(a, pp, h, C, nbk, nbc[j], v);
+                    for (int j = ct; j < n; j += IT) nb_pixel<integ>(a, pp, h, C, nbk, nbc[j], v);
                 }
                 if (ct == 0) sm.nb_cnt[(nb_img + 1) & 1] = 0;
                 ++nb_img;
@@ -1356,15 +1378,15 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
             }
         } else {
             if (pp.sliding && pp.W == 6 && h.S == 40)
-                integrate_chunk<40, 6, IT, PPT, NO_INTEG, LEAN>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<40, 6, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else if (pp.sliding && pp.W == 6 && h.S == 30)
-                integrate_chunk<30, 6, IT, PPT, NO_INTEG, LEAN>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<30, 6, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else if (pp.sliding && pp.W == 6 && h.S == 25)
-                integrate_chunk<25, 6, IT, PPT, NO_INTEG, LEAN>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<25, 6, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else if (pp.sliding && pp.W == 5 && h.S == 16)
-                integrate_chunk<16, 5, IT, PPT, NO_INTEG, LEAN>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<16, 5, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else
-                integrate_chunk<0, 0, IT, PPT, NO_INTEG, LEAN, ANY, SKEW>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<0, 0, IT, PPT, integ, FILTER, ANY, SKEW>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
             if (++stage == NST) { stage = 0; phase ^= 1u; }

@@ -1,10 +1,7 @@
-// The lean instantiations of the fused image kernel (k_image_chain.cuh): the
-// image chain on contiguous bundles without the integrate-only outputs -- the
-// flat window and the neighbour-peak window (LEAN = true, also without the
-// digital filter) and the digital filter (FILT = true) -- so that those
-// branches are not compiled into the kernels the reconstruction runs, for
-// launches whose cameras all have a specialised window search (ANY = false).
-// Compiled apart from the other instantiations so that the builds run in parallel.
+// The instantiations of the fused image kernel (k_image_chain.cuh) that run the image chain on
+// contiguous bundles whose cameras all have a specialised window search (ANY = false): flat
+// window, neighbour-peak window and digital filter, rows only. Compiled apart from the others so
+// that the builds run in parallel.
 #include "k_image_chain.cuh"
 
 namespace rta {
@@ -13,7 +10,7 @@ namespace rta {
 template <int IW, int PPT, int MB, bool NB, bool FILT = false>
 static cudaError_t launch_lean(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, NB, false, !FILT, FILT, false>;
+    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILT ? 1 : 0, OUT_ROWS, false>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;

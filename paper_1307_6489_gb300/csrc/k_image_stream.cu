@@ -1,8 +1,7 @@
 // The byte-stream instantiations of the fused image kernel (k_image_chain with
 // STREAM = true, k_image_chain.cuh): the producer copies each chunk from the
-// segments of an ingested stream. The stream path never runs integrate-only; a
-// lean form (LEAN = true) also leaves out the digital filter and serves every
-// other window mode. Compiled apart so the builds run in parallel.
+// segments of an ingested stream; with the digital filter and without it (LEAN).
+// Compiled apart so the builds run in parallel.
 #include "k_image_chain.cuh"
 
 namespace rta {
@@ -10,7 +9,7 @@ namespace rta {
 template <int IW, int PPT, int MB, bool LEAN, bool ANY>
 static cudaError_t launch_stream(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                  int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, false, true, LEAN, false, ANY>;
+    auto kern = k_image_chain<IW, PPT, MB, false, true, LEAN ? 0 : 1, OUT_ROWS, ANY>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;

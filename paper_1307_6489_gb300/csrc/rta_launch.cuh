@@ -19,7 +19,7 @@ struct ChainArgs {
     float* q_out;            // integrate-only mode
     float* t_out;
     rta_hillas_t* out;       // full mode
-    uint8_t* mask_out;       // full mode, optional: cleaning masks (general instantiations only)
+    uint8_t* mask_out;       // full mode, optional: cleaning masks
     unsigned int* counter;   // zeroed before the launch
     unsigned int* status;
     int stage_wave_bytes;    // multiple of 128
