@@ -100,7 +100,6 @@ static const ChainVariant kVariants[RTA_CHAIN_VARIANTS] = {{8, 1, 2}, {4, 2, 2},
 int chain_variant_warps(int v) { return kVariants[v].iw; }
 int chain_variant_ppt(int v) { return kVariants[v].ppt; }
 int chain_variant_min_blocks(int v) { return kVariants[v].min_blocks; }
-int chain_threads(int v) { return kVariants[v].iw * 32 + 64; }
 
 int chain_stage_wave_bytes(int v, int max_S) {
     const int chunk = kVariants[v].iw * 32 * kVariants[v].ppt;
@@ -109,13 +108,14 @@ int chain_stage_wave_bytes(int v, int max_S) {
     return swb < cap ? swb : cap;
 }
 
-size_t chain_smem_bytes(int v, int nstage, int stage_wave_bytes, int max_P, int nb_keys, int stream_recs) {
-    const size_t head = (sizeof(ChainSmem) + 127) & ~size_t(127);
+size_t chain_smem_bytes(int v, int nstage, int stage_wave_bytes, int max_P, int nb_keys, int stream_recs, int tails) {
+    const size_t head = ((tails > 1 ? sizeof(ChainSmem<SMALL_TAILS>) : sizeof(ChainSmem<2>)) + 127) & ~size_t(127);
     const size_t words = (max_P + 31) / 32;
     const size_t chunk = size_t(kVariants[v].iw) * 32 * kVariants[v].ppt;
     const size_t keys = nb_keys ? 10 * size_t(max_P) + 16 : 0;   // 64-bit keys, 16-bit candidate ids
     const size_t recs = stream_recs ? 2 * sizeof(StreamImg) + 16 : 0;   // the producer's two stream records
-    return head + size_t(nstage) * (stage_wave_bytes + 2 * chunk * 4) + NSLOT * slot_bytes(max_P) + 8 * words + 16 +
+    return head + size_t(nstage) * (stage_wave_bytes + 2 * chunk * 4) + chain_slots(tails) * slot_bytes(max_P) +
+           8 * tails * words + 16 +
            keys + recs;
 }
 
@@ -138,9 +138,9 @@ static cudaError_t launch_t(const ChainArgs& a, int grid, size_t smem, cudaStrea
     }
     if (occupancy_only) {
         *occ = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, IW * 32 + 64, smem);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, chain_block(IW, 1), smem);
     }
-    kern<<<grid, IW * 32 + 64, smem, s>>>(a);
+    kern<<<grid, chain_block(IW, 1), smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -1,5 +1,7 @@
 // The image chain on contiguous bundles (as k_image_lean.cu) for launches with a
 // camera whose sample count or window has no specialised search (ANY = true).
+#include <algorithm>
+
 #include "k_image_chain.cuh"
 
 namespace rta {
@@ -7,10 +9,10 @@ namespace rta {
 constexpr size_t SMEM_PER_SM = size_t(227) * 1024;
 
 // FILT: the form with the digital filter (LEAN = false, FILT = true).
-template <int IW, int PPT, int MB, bool NB, bool FILT = false>
+template <int IW, int PPT, int MB, bool NB, bool FILT = false, int TAILS = 1>
 static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILT ? 1 : 0, OUT_ROWS, true>;
+    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILT ? 1 : 0, OUT_ROWS, true, TAILS>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;
@@ -22,9 +24,9 @@ static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStr
     }
     if (occupancy_only) {
         *occ = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, IW * 32 + 64, smem);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, chain_block(IW, TAILS), smem);
     }
-    kern<<<grid, IW * 32 + 64, smem, s>>>(a);
+    kern<<<grid, chain_block(IW, TAILS), smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -34,7 +36,7 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
     // variant 4 is variant 0's tile in the 64 registers that let three CTAs share an SM; where
     // shared memory holds fewer, its spills buy nothing (4096 pixels x 128 samples: 516 us, and
     // 478 with variant 0's 88 registers)
-    if (v == 4 && 3 * smem > SMEM_PER_SM) v = 0;
+    if (v == 4 && 3 * smem > SMEM_PER_SM && a.arr.max_P > SMALL_PIX) v = 0;
     if (a.pp.nbpeak) {
         switch (v) {
         case 0: return launch_any<8, 1, 2, true>(a, grid, smem, s, occ_only, occ);
@@ -54,6 +56,14 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
         case 4: return launch_any<8, 1, 3, false, true>(a, grid, smem, s, occ_only, occ);
         default: return cudaErrorInvalidValue;
         }
+    }
+    // small cameras: variant 4's tile with a tail warp for each of eight slots, two CTAs an SM (an
+    // image of 256 pixels is integrated in a fraction of the time its cleaning and moments take:
+    // 2,000 of them 21.4 us, 35.5 with one tail warp for two slots)
+    if (v == 4 && a.arr.max_P <= SMALL_PIX && !occ_only) {
+        const size_t sm8 = chain_smem_bytes(4, a.nstage, a.stage_wave_bytes, a.arr.max_P, 0, 0, SMALL_TAILS);
+        const int g8 = int(std::min<int64_t>(a.n_img, 2 * int64_t(a.n_sm)));
+        if (sm8 <= size_t(227) * 1024) return launch_any<8, 1, 2, false, false, SMALL_TAILS>(a, g8, sm8, s, false, nullptr);
     }
     switch (v) {
     case 0: return launch_any<8, 1, 2, false>(a, grid, smem, s, occ_only, occ);

@@ -638,13 +638,20 @@ __device__ __forceinline__ void write_bad_row(rta_hillas_t* out) {
 // searches in flight. Integrated images go through two shared-memory slots (q, t
 // and the hi/lo bitmaps of one image each): the integrators fill one slot while
 // the tail warp cleans and parameterises the other.
-constexpr int NSLOT = 2;      // (the kernel's opening writes both by name)
+//
+// TAILS tail warps: one for both slots, or (small cameras, whose images take longer to clean and
+// parameterise than to integrate) as many as there are slots, one each.
+__host__ __device__ constexpr int chain_slots(int tails) { return tails > 2 ? tails : 2; }
+__host__ __device__ constexpr int chain_block(int iw, int tails) { return iw * 32 + 32 + 32 * tails; }
+constexpr int SMALL_TAILS = 8;
+constexpr int SMALL_PIX = 512;      // pixels of the largest camera that counts as small
 enum { SLOT_END = 1 };
 
 struct SlotHdr {
     int img, cam, flags, pad;
 };
 
+template <int NSLOT>
 struct ChainSmem {
     uint64_t full[MAX_STAGES];
     uint64_t empty[MAX_STAGES];
@@ -1043,16 +1050,18 @@ static __device__ __forceinline__ int stream_chunk_copy(const ChainArgs& a, cons
 // OUT: what a launch writes -- Hillas rows, charges and times only (the integrate-only call), or
 // rows and cleaning masks.
 enum { OUT_ROWS = 0, OUT_CHARGES = 1, OUT_MASKS = 2 };
-template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, bool ANY>
-__global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArgs a) {
+template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, bool ANY, int TAILS = 1>
+__global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(const ChainArgs a) {
     static_assert(!(NB && FILTER) && !(STREAM && OUT != OUT_ROWS), "the calls there are");
     constexpr bool integ = OUT == OUT_CHARGES;
     constexpr bool SKEW = ANY && !NB && !STREAM;
     constexpr int IT = IW * 32;          // integrator threads
     constexpr int CHUNK = IT * PPT;      // largest chunk in pixels
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    ChainSmem& sm = *reinterpret_cast<ChainSmem*>(smem_raw);
-    const size_t head = (sizeof(ChainSmem) + 127) & ~size_t(127);
+    constexpr int NSLOT = chain_slots(TAILS);
+    static_assert(TAILS == 1 || TAILS == NSLOT, "a tail warp for all slots or for one");
+    ChainSmem<NSLOT>& sm = *reinterpret_cast<ChainSmem<NSLOT>*>(smem_raw);
+    const size_t head = (sizeof(ChainSmem<NSLOT>) + 127) & ~size_t(127);
     const int NST = a.nstage;
     const int calib_bytes = CHUNK * 4;
     const int stage_bytes = a.stage_wave_bytes + 2 * calib_bytes;
@@ -1069,10 +1078,10 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
         v.lo = v.hi + maxw;
         return v;
     };
-    uint32_t* core = reinterpret_cast<uint32_t*>(slots + NSLOT * slot_bytes(maxP));
-    uint32_t* maskb = core + maxw;
+    uint32_t* core = reinterpret_cast<uint32_t*>(slots + NSLOT * slot_bytes(maxP));   // core and mask of each tail warp
+    uint32_t* tail_end = core + 2 * TAILS * maxw;
     // neighbour-peak keys and candidates of the image being integrated
-    uint64_t* nbk = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(maskb + maxw) + 15) & ~uintptr_t(15));
+    uint64_t* nbk = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(tail_end) + 15) & ~uintptr_t(15));
     int16_t* nbc = reinterpret_cast<int16_t*>(nbk + maxP);
     // byte stream: the records of the image whose chunks the producer issues and of
     // the next one, copied in by cp.async one image ahead (after the keys, if any)
@@ -1100,7 +1109,9 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
         fence_mbar_init();
     }
     if (!NB && !integ)
-        for (int w = tid; w < 2 * maxw; w += IT + 64) slot_view(0).hi[w] = slot_view(1).hi[w] = 0u;   // hi and lo
+        for (int w = tid; w < 2 * maxw; w += chain_block(IW, TAILS))
+#pragma unroll
+            for (int k = 0; k < NSLOT; ++k) slot_view(k).hi[w] = 0u;      // hi and lo
     if (tid == 0) {
 #pragma unroll
         for (int k = 0; k < RTA_MAX_W; ++k) sm.wts[k] = a.pp.wts[k];   // constant indices: no copy of the parameters
@@ -1282,8 +1293,11 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
     };
 
     if (tid >= 32 + IT) {
-        // ---------------- tail warp: cleaning + Hillas of integrated images
-        int slot = 0;
+        // ---------------- tail warps: cleaning + Hillas of integrated images
+        const int tw = TAILS > 1 ? (tid - 32 - IT) >> 5 : 0;
+        uint32_t* const my_core = core + 2 * tw * maxw;
+        uint32_t* const maskb = my_core + maxw;
+        int slot = tw;
         uint32_t ph = 0;
         for (;;) {
             if (!mbar_wait(&sm.slot_full[slot], ph, abort_flag)) { give_up(); break; }
@@ -1291,13 +1305,14 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
             if (sh.flags & SLOT_END) break;
             const SlotView v = slot_view(slot);
             const DevCam C = a.arr.cams[sh.cam];
-            const ImgBits ib = {v.hi, v.lo, core, maskb};
+            const ImgBits ib = {v.hi, v.lo, my_core, maskb};
             clean_bits<!NB>(C, pp, ib, lane, 32, WarpBar());
             if constexpr (OUT == OUT_MASKS) write_mask(a, C, maskb, sh.img, lane);
             hillas_bits(v.q, v.t, C, maskb, sm.red, lane, 32, WarpBar(), a.out + sh.img);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.slot_free[slot]);
-            if (++slot == NSLOT) { slot = 0; ph ^= 1u; }
+            if (TAILS > 1) ph ^= 1u;                   // always its own slot
+            else if (++slot == NSLOT) { slot = 0; ph ^= 1u; }
         }
         return;
     }
@@ -1313,11 +1328,14 @@ __global__ void __launch_bounds__(IW * 32 + 64, MB) k_image_chain(const ChainArg
         if (!mbar_wait(&sm.full[stage], phase, abort_flag)) { give_up(); break; }
         const StageHdr h = sm.hdr[stage];
         if (h.flags & HDR_END) {
-            // tell the tail warp there is nothing more
-            if (!mbar_wait(&sm.slot_free[slot], sphase ^ 1u, abort_flag)) { give_up(); break; }
-            if (ct == 0) sm.shdr[slot].flags = SLOT_END;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.slot_full[slot]);
+            // tell the tail warps there is nothing more
+            for (int k = 0; k < TAILS; ++k) {
+                if (!mbar_wait(&sm.slot_free[slot], sphase ^ 1u, abort_flag)) { give_up(); break; }
+                if (ct == 0) sm.shdr[slot].flags = SLOT_END;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.slot_full[slot]);
+                if (++slot == NSLOT) { slot = 0; sphase ^= 1u; }
+            }
             break;
         }
         if (h.flags & HDR_BAD) {

@@ -21,9 +21,9 @@ static cudaError_t launch_nb(const ChainArgs& a, int grid, size_t smem, cudaStre
     }
     if (occupancy_only) {
         *occ = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, IW * 32 + 64, smem);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, chain_block(IW, 1), smem);
     }
-    kern<<<grid, IW * 32 + 64, smem, s>>>(a);
+    kern<<<grid, chain_block(IW, 1), smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -313,6 +313,7 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
     a.nstage = std::max(2, std::min(cfg.nstage, 8));
     a.integrate_only = integrate_only;
     a.any_window = needs_any_window(c, pp);
+    a.n_sm = c->n_sm;
     a.n_img_dev = d_n_img;
     a.seg = d_seg;
     a.img_seg = d_img_seg;

@@ -25,6 +25,7 @@ struct ChainArgs {
     int stage_wave_bytes;    // multiple of 128
     int nstage;
     int integrate_only;
+    int n_sm;                // of the device
     int any_window;          // some camera has no specialised window search (window_specialised)
     // a byte-stream bundle (rta_ingest's directory): wave is the stream, wave_off unused;
     // smeta: one prepared record per image (k_stream_meta)
@@ -99,9 +100,9 @@ struct StereoArgs {
 
 int chain_variant_warps(int v);
 int chain_variant_ppt(int v);
-int chain_threads(int v);
 int chain_stage_wave_bytes(int v, int max_S);
-size_t chain_smem_bytes(int v, int nstage, int stage_wave_bytes, int max_P, int nb_keys = 0, int stream_recs = 0);
+size_t chain_smem_bytes(int v, int nstage, int stage_wave_bytes, int max_P, int nb_keys = 0, int stream_recs = 0,
+                        int tails = 1);
 int chain_chunk_pixels(int v, int stage_wave_bytes, int S);
 // which instantiation family of the fused kernel a launch uses (the occupancy of
 // a family's general instantiation stands for its lean ones: same launch bounds,
