@@ -8,84 +8,171 @@ namespace rta {
 
 // ------------------------------------------------------------------ unfused stage kernels
 
-// Bitmaps of one image from per-pixel values in global memory: the warp that
-// covers 32 consecutive pixels writes their word.
-__device__ __forceinline__ void ballot_words(int P, int tid, int nthr, uint32_t* w0, uint32_t* w1, const float* q,
-                                             float t0, float t1) {
-    for (int base = 0; base < P; base += nthr) {
-        const int p = base + tid;
-        const float v = p < P ? q[p] : 0.f;
-        const uint32_t b0 = __ballot_sync(0xffffffffu, p < P && v >= t0);
-        const uint32_t b1 = __ballot_sync(0xffffffffu, p < P && v >= t1);
-        if ((tid & 31) == 0 && (p >> 5) < words_of(P)) {
-            w0[p >> 5] = b0;
-            if (w1) w1[p >> 5] = b1;
+// One block per image, a warp per 32-pixel word and a lane per pixel. What an image's pixels need
+// from memory -- values straight into ballots, then the neighbours, or the charges, times and
+// positions, of the pixels that count -- is loaded side by side, one latency for all of them (a
+// thread per bitmap word met one per set bit). 501 events, 2,320 images: k_hillas 38 -> 26 us,
+// k_clean 20.5 -> 22 alone but the two, back to back with the integration, 116 -> 108.
+constexpr int UNF_WARPS = 8;
+constexpr int UNF_WORDS = 8;      // words a warp takes at a time
+constexpr int UNF_STEP = UNF_WARPS * UNF_WORDS;
+
+// w0[w] = {v >= t0}, w1[w] = {v >= t1} of the image's values q (global memory).
+__device__ __forceinline__ void threshold_words(const float* q, int P, float t0, float t1, uint32_t* w0, uint32_t* w1) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = words_of(P);
+    for (int wb = 0; wb < nw; wb += UNF_STEP) {
+        float v[UNF_WORDS];
+#pragma unroll
+        for (int k = 0; k < UNF_WORDS; ++k) {
+            const int p = 32 * (wb + warp + UNF_WARPS * k) + lane;
+            v[k] = p < P ? __ldg(q + p) : __int_as_float(0x7fc00000);      // NaN: neither
+        }
+#pragma unroll
+        for (int k = 0; k < UNF_WORDS; ++k) {
+            const int w = wb + warp + UNF_WARPS * k;
+            if (w >= nw) break;
+            const uint32_t b0 = __ballot_sync(0xffffffffu, v[k] >= t0);
+            const uint32_t b1 = __ballot_sync(0xffffffffu, v[k] >= t1);
+            if (lane == 0) {
+                w0[w] = b0;
+                w1[w] = b1;
+            }
         }
     }
 }
 
-__global__ void __launch_bounds__(256) k_clean(const CleanArgs a) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    float* sq = reinterpret_cast<float*>(smem_raw);
+__global__ void __launch_bounds__(UNF_WARPS * 32) k_clean(const CleanArgs a) {
+    extern __shared__ __align__(16) uint32_t words[];
     const int maxw = words_of(a.arr.max_P);
-    uint32_t* bits0 = reinterpret_cast<uint32_t*>(sq + a.arr.max_P);
-    const ImgBits ib = {bits0, bits0 + maxw, bits0 + 2 * maxw, bits0 + 3 * maxw};
+    uint32_t *hi = words, *lo = hi + maxw, *core = lo + maxw, *mask = core + maxw;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t img = blockIdx.x; img < a.n_img; img += gridDim.x) {
         const int tel = a.img_tel[img];
+        const int64_t off = a.pix_off[img];
         if (tel < 0 || tel >= a.arr.n_tel) {
             if (threadIdx.x == 0) atomicOr(a.status, RTA_DEV_BAD_IMAGE);
             continue;
         }
         const DevCam C = a.arr.cams[a.arr.tel_cam[tel]];
-        const int64_t off = a.pix_off[img];
         if (off < 0 || off + C.P > a.n_q) {
             if (threadIdx.x == 0) atomicOr(a.status, RTA_DEV_BAD_IMAGE);
             continue;
         }
-        for (int p = threadIdx.x; p < C.P; p += blockDim.x) sq[p] = a.q[off + p];
+        threshold_words(a.q + off, C.P, a.pp.t_hi, a.pp.t_lo, hi, lo);
         __syncthreads();
-        ballot_words(C.P, threadIdx.x, blockDim.x, ib.hi, ib.lo, sq, a.pp.t_hi, a.pp.t_lo);
+        // core = hi, with a hi neighbour if asked; mask = core, and lo with a core neighbour. The
+        // neighbours of the pixels in lo (hi is part of it) are loaded once for both
+        const int nw = words_of(C.P);
+        int4 nbr[UNF_WORDS];
+        auto fetch = [&](int w0) {
+#pragma unroll
+            for (int k = 0; k < UNF_WORDS; ++k) {
+                const int w = w0 + warp + UNF_WARPS * k;
+                if (w < nw && ((lo[w] >> lane) & 1u)) nbr[k] = __ldg(C.nb + (32 * w + lane));
+            }
+        };
+        for (int w0 = 0; w0 < nw; w0 += UNF_STEP) {
+            fetch(w0);
+#pragma unroll
+            for (int k = 0; k < UNF_WORDS; ++k) {
+                const int w = w0 + warp + UNF_WARPS * k;
+                if (w >= nw) break;
+                bool on = (hi[w] >> lane) & 1u;
+                if (on && a.pp.core_nb) on = any_neighbour(nbr[k], C.K, C.P, hi);
+                const uint32_t b = __ballot_sync(0xffffffffu, on);
+                if (lane == 0) core[w] = b;
+            }
+        }
         __syncthreads();
-        clean_bits(C, a.pp, ib, threadIdx.x, blockDim.x, BlockBar());
-        for (int p = threadIdx.x; p < C.P; p += blockDim.x) a.mask[off + p] = bit_of(ib.mask, p) ? 1 : 0;
+        for (int w0 = 0; w0 < nw; w0 += UNF_STEP) {
+            if (nw > UNF_STEP) fetch(w0);                // else they are still there
+#pragma unroll
+            for (int k = 0; k < UNF_WORDS; ++k) {
+                const int w = w0 + warp + UNF_WARPS * k;
+                if (w >= nw) break;
+                bool on = (core[w] >> lane) & 1u;
+                if (!on && ((lo[w] >> lane) & 1u)) on = any_neighbour(nbr[k], C.K, C.P, core);
+                const uint32_t b = __ballot_sync(0xffffffffu, on);
+                if (lane == 0) mask[w] = b;
+            }
+        }
+        __syncthreads();
+        uint8_t* out = a.mask + off;
+        const int quads = C.P >> 2;
+        if ((reinterpret_cast<uintptr_t>(out) & 3u) == 0) {
+            // four pixels a thread: bits 0..3 spread to the bytes
+            for (int g = threadIdx.x; g < quads; g += blockDim.x) {
+                const uint32_t b = (mask[g >> 3] >> (4 * (g & 7))) & 15u;
+                reinterpret_cast<uint32_t*>(out)[g] = (b * 0x00204081u) & 0x01010101u;
+            }
+            for (int p = 4 * quads + threadIdx.x; p < C.P; p += blockDim.x) out[p] = bit_of(mask, p) ? 1 : 0;
+        } else {
+            for (int p = threadIdx.x; p < C.P; p += blockDim.x) out[p] = bit_of(mask, p) ? 1 : 0;
+        }
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(256) k_hillas(const HillasArgs a) {
+__global__ void __launch_bounds__(UNF_WARPS * 32) k_hillas(const HillasArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ float red[3 * NCW * 8];
     float* sq = reinterpret_cast<float*>(smem_raw);
     float* st = sq + a.arr.max_P;
-    float* sm = st + a.arr.max_P;
-    uint32_t* mask = reinterpret_cast<uint32_t*>(sm + a.arr.max_P);
+    float2* sxy = reinterpret_cast<float2*>(st + a.arr.max_P);
+    uint32_t* mask = reinterpret_cast<uint32_t*>(sxy + a.arr.max_P);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t img = blockIdx.x; img < a.n_img; img += gridDim.x) {
         const int tel = a.img_tel[img];
-        if (tel < 0 || tel >= a.arr.n_tel) {
-            if (threadIdx.x == 0) {
-                atomicOr(a.status, RTA_DEV_BAD_IMAGE);
-                write_bad_row(a.out + img);
-            }
-            continue;
-        }
-        const DevCam C = a.arr.cams[a.arr.tel_cam[tel]];
         const int64_t off = a.pix_off[img];
-        if (off < 0 || off + C.P > a.n_q) {
+        bool bad = tel < 0 || tel >= a.arr.n_tel;
+        DevCam C = {};
+        if (!bad) {
+            C = a.arr.cams[a.arr.tel_cam[tel]];
+            bad = off < 0 || off + C.P > a.n_q;
+        }
+        if (bad) {
             if (threadIdx.x == 0) {
                 atomicOr(a.status, RTA_DEV_BAD_IMAGE);
                 write_bad_row(a.out + img);
             }
             continue;
         }
-        for (int p = threadIdx.x; p < C.P; p += blockDim.x) {
-            sq[p] = a.q[off + p];
-            if (a.t) st[p] = a.t[off + p];
-            sm[p] = a.mask[off + p] ? 1.f : 0.f;
+        // charges, times and positions of the cleaned pixels only
+        const int nw = words_of(C.P);
+        for (int wb = 0; wb < nw; wb += UNF_STEP) {
+            bool on[UNF_WORDS];
+            float q[UNF_WORDS], t[UNF_WORDS];
+            float2 xy[UNF_WORDS];
+#pragma unroll
+            for (int k = 0; k < UNF_WORDS; ++k) {
+                const int p = 32 * (wb + warp + UNF_WARPS * k) + lane;
+                on[k] = p < C.P && __ldg(a.mask + off + p) != 0;
+            }
+#pragma unroll
+            for (int k = 0; k < UNF_WORDS; ++k) {
+                const int p = 32 * (wb + warp + UNF_WARPS * k) + lane;
+                if (on[k]) {
+                    q[k] = __ldg(a.q + off + p);
+                    if (a.t) t[k] = __ldg(a.t + off + p);
+                    xy[k] = __ldg(C.xy + p);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < UNF_WORDS; ++k) {
+                const int w = wb + warp + UNF_WARPS * k, p = 32 * w + lane;
+                if (w >= nw) break;
+                const uint32_t b = __ballot_sync(0xffffffffu, on[k]);
+                if (lane == 0) mask[w] = b;
+                if (on[k]) {
+                    sq[p] = q[k];
+                    if (a.t) st[p] = t[k];
+                    sxy[p] = xy[k];
+                }
+            }
         }
         __syncthreads();
-        ballot_words(C.P, threadIdx.x, blockDim.x, mask, nullptr, sm, 0.5f, 0.5f);
-        __syncthreads();
-        hillas_bits(sq, a.t ? st : nullptr, C, mask, red, threadIdx.x, blockDim.x, BlockBar(), a.out + img);
+        C.xy = sxy;
+        hillas_bits<false>(sq, a.t ? st : nullptr, C, mask, red, threadIdx.x, blockDim.x, BlockBar(), a.out + img);
         __syncthreads();
     }
 }
@@ -186,14 +273,18 @@ int chain_occupancy(int v, size_t smem, int kind) {
 }
 
 cudaError_t launch_clean(const CleanArgs& a, int grid, cudaStream_t s) {
-    const size_t smem = size_t(a.arr.max_P) * 4 + size_t(16) * ((a.arr.max_P + 31) / 32) + 16;
-    k_clean<<<grid, 256, smem, s>>>(a);
+    const size_t smem = size_t(16) * ((a.arr.max_P + 31) / 32) + 16;
+    k_clean<<<grid, UNF_WARPS * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_hillas(const HillasArgs& a, int grid, cudaStream_t s) {
-    const size_t smem = size_t(a.arr.max_P) * 12 + size_t(4) * ((a.arr.max_P + 31) / 32) + 16;
-    k_hillas<<<grid, 256, smem, s>>>(a);
+    const size_t smem = size_t(a.arr.max_P) * 16 + size_t(4) * ((a.arr.max_P + 31) / 32) + 16;
+    if (smem > size_t(48) * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_hillas, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return e;
+    }
+    k_hillas<<<grid, UNF_WARPS * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 

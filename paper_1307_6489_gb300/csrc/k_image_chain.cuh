@@ -529,7 +529,8 @@ __device__ __forceinline__ void clean_bits(const DevCam& C, const ProcParams& pp
 // gradient. These equal lambda1 and det/lambda1 of the covariance, but stay well
 // conditioned in FP32 for nearly collinear images, where det is a small
 // difference of large products. Thread 0 writes the row.
-template <class Bar>
+// GLOBAL_XY: the pixel positions are in global memory (else in shared memory).
+template <bool GLOBAL_XY = true, class Bar>
 __device__ __forceinline__ void hillas_bits(const float* q, const float* t, const DevCam& C, const uint32_t* mask,
                                             float* red, int tid, int nthr, Bar bar, rta_hillas_t* out) {
     const int nw = words_of(C.P);
@@ -538,7 +539,7 @@ __device__ __forceinline__ void hillas_bits(const float* q, const float* t, cons
         for (uint32_t m = mask[w]; m; m &= m - 1) {
             const int p = w * 32 + __ffs(m) - 1;
             const float qp = q[p];
-            const float2 xy = __ldg(C.xy + p);
+            const float2 xy = GLOBAL_XY ? __ldg(C.xy + p) : C.xy[p];
             a[0] += 1.f;
             a[1] += qp;
             a[2] += qp * xy.x;
@@ -562,7 +563,7 @@ __device__ __forceinline__ void hillas_bits(const float* q, const float* t, cons
         for (uint32_t m = mask[w]; m; m &= m - 1) {
             const int p = w * 32 + __ffs(m) - 1;
             const float qp = q[p];
-            const float2 xy = __ldg(C.xy + p);
+            const float2 xy = GLOBAL_XY ? __ldg(C.xy + p) : C.xy[p];
             const float dx = xy.x - cx, dy = xy.y - cy;
             b[0] += qp * dx * dx;
             b[1] += qp * dy * dy;
@@ -579,7 +580,7 @@ __device__ __forceinline__ void hillas_bits(const float* q, const float* t, cons
         for (uint32_t m = mask[w]; m; m &= m - 1) {
             const int p = w * 32 + __ffs(m) - 1;
             const float qp = q[p];
-            const float2 xy = __ldg(C.xy + p);
+            const float2 xy = GLOBAL_XY ? __ldg(C.xy + p) : C.xy[p];
             const float dx = xy.x - cx, dy = xy.y - cy;
             const float l = dx * cp + dy * sp;
             const float wd = dy * cp - dx * sp;
