@@ -196,7 +196,9 @@ int rta_set_chain_config(rta_ctx* ctx, int variant, int n_stages, int ctas_per_s
 /* The configuration a launch outside the neighbour-peak mode would use now (the
  * byte-stream path too, unless rta_autotune_stream has tuned its own):
  * variant, stages, CTAs per SM, grid size and dynamic shared memory per CTA in
- * bytes (NULL outputs are skipped). */
+ * bytes (NULL outputs are skipped). Launches of at most one image per SM use more
+ * stages than the default configuration's two, and small cameras (at most 512
+ * pixels) more image slots; results do not depend on it. */
 int rta_get_chain_config(rta_ctx* ctx, int* variant, int* n_stages, int* ctas_per_sm, int* grid,
                          size_t* smem_bytes);
 

@@ -3,7 +3,8 @@
 // Sec. 5).
 //
 // k_image_chain is the hot path. It is a persistent, warp-specialised kernel:
-//   warp 0      producer: takes the next image from a global work counter and
+//   warp 0      producer: takes its first image by its block index and the next ones from a
+//               global work counter, and
 //               streams it, chunk by chunk, into a ring of shared-memory stages
 //               with bulk copies on the TMA engine (cp.async.bulk, one mbarrier
 //               per stage, transaction-count completion); the calibration rows
@@ -1140,7 +1141,7 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
         // image's chunks are issued: neither the work counter's atomic nor those
         // loads wait at an image boundary
         constexpr bool stream_mode = STREAM;
-        int64_t next = atomicAdd(a.counter, 1u);
+        int64_t next = blockIdx.x;     // then from the counter, which counts from the grid's size
         int next_tel = -1;
         int64_t next_woff = 0;
         int rec_next = 0;              // byte stream: the record buffer the next image's record goes to
@@ -1169,7 +1170,7 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
                 rec_next ^= 1;
             }
             if (img < n_img) {
-                next = atomicAdd(a.counter, 1u);
+                next = int64_t(gridDim.x) + atomicAdd(a.counter, 1u);
                 fetch_next();
             }
             if (img >= n_img) {

@@ -20,7 +20,8 @@ struct ChainArgs {
     float* t_out;
     rta_hillas_t* out;       // full mode
     uint8_t* mask_out;       // full mode, optional: cleaning masks
-    unsigned int* counter;   // zeroed before the launch
+    unsigned int* counter;   // images taken beyond the first of every block; zeroed before the launch when
+                             // there are more images than blocks
     unsigned int* status;
     int stage_wave_bytes;    // multiple of 128
     int nstage;
