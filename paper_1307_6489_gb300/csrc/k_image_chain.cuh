@@ -116,7 +116,7 @@ __device__ __forceinline__ int best_key_T(const uint16_t* row, int one, int k128
     return best_key_x<S, W>(x, one, k128);
 }
 
-// Maximum W = 6 window sum of one pixel when every loaded 16-bit sample is below
+// Maximum window sum of one pixel, W of 4 to 8 samples, when every loaded 16-bit sample is below
 // 4096 (true for 12-bit digitisers; checked here): two samples per 32-bit word,
 // pair sums and window sums formed two lanes at a time with plain 32-bit adds
 // (each lane stays below 2^15, so no carry crosses a lane), then the maximum
@@ -125,11 +125,12 @@ __device__ __forceinline__ int best_key_T(const uint16_t* row, int one, int k128
 // k + 1, and the windows that would reach outside the row are masked. Returns
 // false (nothing computed) when a sample is 4096 or more; the window start is
 // not computed here.
-template <int S>
-__device__ __forceinline__ bool max_window6_packed(const uint16_t* row, int& M) {
-    constexpr int NK = S - 6 + 1;                 // window starts 0 .. NK - 1
+template <int S, int W>
+__device__ __forceinline__ bool max_window_packed(const uint16_t* row, int& M) {
+    static_assert(W >= 4 && W <= 8, "window sums of two to four pairs, and a sample for odd widths");
+    constexpr int NK = S - W + 1;                 // window starts 0 .. NK - 1
     constexpr int JQ = NK / 2 + 1;                // packed window words
-    constexpr int NW = JQ + 3;                    // loaded words
+    constexpr int NW = JQ + W / 2;                // loaded words
     const uintptr_t a = reinterpret_cast<uintptr_t>(row);
     const bool odd = (S % 2 == 1) && (a & 2u);
     const uint32_t* v = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
@@ -160,7 +161,10 @@ __device__ __forceinline__ bool max_window6_packed(const uint16_t* row, int& M) 
     uint32_t m[JQ];
 #pragma unroll
     for (int j = 0; j < JQ; ++j) {
-        uint32_t q = P[j] + P[j + 1] + P[j + 2];  // lanes: windows (2j + 1 : 2j), or (2j : 2j - 1) for odd rows
+        uint32_t q = P[j] + P[j + 1];             // lanes: windows (2j + 1 : 2j), or (2j : 2j - 1) for odd rows
+#pragma unroll
+        for (int i = 2; i < W / 2; ++i) q += P[j + i];
+        if (W % 2) q += u[j + W / 2];
         const bool lo_ok = odd ? (j >= 1 && 2 * j <= NK) : (2 * j <= NK - 1);
         const bool hi_ok = odd ? (2 * j <= NK - 1) : (2 * j + 1 <= NK - 1);
         q &= (hi_ok ? 0xFFFF0000u : 0u) | (lo_ok ? 0xFFFFu : 0u);
@@ -289,7 +293,7 @@ __device__ __forceinline__ void window_words(const uint32_t (&u)[16], int W, uin
 }
 
 // The search for any sample count and any window of up to 16 samples (the cameras and windows
-// without a specialised one), eight words of window starts at a time. As in max_window6_packed,
+// without a specialised one), eight words of window starts at a time. As in max_window_packed,
 // samples must be below 4096 (checked), and rows that start on an odd 16-bit position are read
 // from the word below. Words read past the row's end stay inside the stage (its calibration
 // rows follow) and their windows are dropped.
@@ -750,7 +754,7 @@ __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcPara
             bool exact = true;
             if constexpr (S != 0 && W == 6) {
                 int m = 0;
-                if (!integ && max_window6_packed<S>(row, m)) {
+                if (!integ && max_window_packed<S, W>(row, m)) {
                     q0 = charge(m, Wr, cp16[c], cscale[c], num);
                     exact = false;
                     if (q0 >= pp.t_lo) st = first_start(row, S, W, m);
@@ -868,7 +872,7 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
             if (lo) v.t[p] = peak_time(row, wst, Wr, p16, num);
         }
     };
-    if constexpr (S != 0 && S % 2 == 1 && PPT == 2) {
+    if constexpr (S != 0 && S % 2 == 1 && PPT == 2 && (W == 5 || W == 6)) {
         // adjacent pixel pairs 2ct, 2ct + 1 (P is a multiple of 8 for odd S, so
         // chunks hold whole pairs); the warp covers 64 consecutive pixels
         const int c0 = 2 * ct;
@@ -914,7 +918,7 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                 const uint16_t* row = reinterpret_cast<const uint16_t*>(at) + size_t(c) * Sr;
                 int sum = 0, wst = 0;
                 bool done = false;
-                if constexpr (S != 0 && W == 6) {
+                if constexpr (S > 16 && W >= 4) {
                     // The charge needs only the maximum; the window start (first
                     // maximum) only for pixels whose peak time is needed. The packed
                     // maximum decides: below t_lo its charge is the pixel's whole
@@ -922,7 +926,7 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                     // runs for the pixels that reach t_lo or whose samples are out of
                     // its range.
                     int m = 0;
-                    if (!integ && !filt && max_window6_packed<S>(row, m)) {
+                    if (!integ && !filt && max_window_packed<S, W>(row, m)) {
                         const float q0 = __fmul_rn(__int2float_rn(16 * m - W * cp16[c]), cscale[c]);
                         if (q0 < pp.t_lo) {
                             v.q[h.base + c] = q0;
@@ -934,8 +938,9 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                             sum = m;
                             wst = first_start(row, S, W, m);
                         } else {
-                            const int key = !INTEG && FILTER == 0 ? best_key_serial(row, S, W)
-                                                                  : best_key_T<S, W>(row, pp.one, pp.k128);
+                            int key;
+                            if constexpr (!INTEG && FILTER == 0) key = best_key_serial(row, S, W);
+                            else key = best_key_T<S, W>(row, pp.one, pp.k128);
                             sum = key >> 7;
                             wst = 127 - (key & 127);
                         }
@@ -1052,8 +1057,12 @@ static __device__ __forceinline__ int stream_chunk_copy(const ChainArgs& a, cons
 // OUT: what a launch writes -- Hillas rows, charges and times only (the integrate-only call), or
 // rows and cleaning masks.
 enum { OUT_ROWS = 0, OUT_CHARGES = 1, OUT_MASKS = 2 };
-template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, bool ANY, int TAILS = 1>
+// WIN: the width of the sliding window that has specialised searches for 40, 30 and 25 samples (a
+// launch has one width; the kernels of 4, 5, 7 and 8 samples serve flat windows, rows only).
+template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, bool ANY, int TAILS = 1, int WIN = 6>
 __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(const ChainArgs a) {
+    // flat windows of 6 for the rows alone: the 16-sample camera's window of 5 is the WIN = 5 kernel's
+    constexpr bool ROWS6 = WIN == 6 && OUT == OUT_ROWS && FILTER == 0 && !STREAM && !ANY;
     static_assert(!(NB && FILTER) && !(STREAM && OUT != OUT_ROWS), "the calls there are");
     constexpr bool integ = OUT == OUT_CHARGES;
     constexpr bool SKEW = ANY && !NB && !STREAM;
@@ -1397,13 +1406,13 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
                 if (lane == 0) mbar_arrive(&sm.nb_free);
             }
         } else {
-            if (pp.sliding && pp.W == 6 && h.S == 40)
-                integrate_chunk<40, 6, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
-            else if (pp.sliding && pp.W == 6 && h.S == 30)
-                integrate_chunk<30, 6, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
-            else if (pp.sliding && pp.W == 6 && h.S == 25)
-                integrate_chunk<25, 6, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
-            else if (pp.sliding && pp.W == 5 && h.S == 16)
+            if (pp.sliding && pp.W == WIN && h.S == 40)
+                integrate_chunk<40, WIN, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+            else if (pp.sliding && pp.W == WIN && h.S == 30)
+                integrate_chunk<30, WIN, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+            else if (pp.sliding && pp.W == WIN && h.S == 25)
+                integrate_chunk<25, WIN, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+            else if ((WIN == 5 || !ROWS6) && pp.sliding && pp.W == 5 && h.S == 16)
                 integrate_chunk<16, 5, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else
                 integrate_chunk<0, 0, IT, PPT, integ, FILTER, ANY, SKEW>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);

@@ -2,73 +2,35 @@
 // contiguous bundles whose cameras all have a specialised window search (ANY = false): flat
 // window, neighbour-peak window and digital filter, rows only. Compiled apart from the others so
 // that the builds run in parallel.
-#include <algorithm>
-
-#include "k_image_chain.cuh"
+#include "k_image_rows.cuh"
 
 namespace rta {
-
-// FILT: the form with the digital filter (LEAN = false, FILT = true).
-template <int IW, int PPT, int MB, bool NB, bool FILT = false, int TAILS = 1>
-static cudaError_t launch_lean(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
-                               int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILT ? 1 : 0, OUT_ROWS, false, TAILS>;
-    // the dynamic shared-memory opt-in is per device; remember the largest size set
-    static size_t attr_bytes[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || attr_bytes[dev] < smem) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_bytes[dev] = smem;
-    }
-    if (occupancy_only) {
-        *occ = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, chain_block(IW, TAILS), smem);
-    }
-    kern<<<grid, chain_block(IW, TAILS), smem, s>>>(a);
-    return cudaGetLastError();
-}
 
 // The same tile variants as the other window modes (kVariants in k_image.cu).
 cudaError_t dispatch_image_chain_lean(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                       bool occ_only, int* occ) {
     if (a.pp.nbpeak) {
         switch (v) {
-        case 0: return launch_lean<8, 1, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_lean<4, 2, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_lean<8, 2, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_lean<4, 1, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_lean<8, 1, 3, true>(a, grid, smem, s, occ_only, occ);
+        case 0: return launch_rows<8, 1, 2, 6, true>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_rows<4, 2, 2, 6, true>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_rows<8, 2, 2, 6, true>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_rows<4, 1, 2, 6, true>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_rows<8, 1, 3, 6, true>(a, grid, smem, s, occ_only, occ);
         default: return cudaErrorInvalidValue;
         }
     }
     if (a.pp.filter) {
         switch (v) {
-        case 0: return launch_lean<8, 1, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_lean<4, 2, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_lean<8, 2, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_lean<4, 1, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_lean<8, 1, 3, false, true>(a, grid, smem, s, occ_only, occ);
+        case 0: return launch_rows<8, 1, 2, 6, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_rows<4, 2, 2, 6, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_rows<8, 2, 2, 6, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_rows<4, 1, 2, 6, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_rows<8, 1, 3, 6, false, 1>(a, grid, smem, s, occ_only, occ);
         default: return cudaErrorInvalidValue;
         }
     }
-    // small cameras: variant 4's tile with a tail warp for each of eight slots, two CTAs an SM (an
-    // image of 256 pixels is integrated in a fraction of the time its cleaning and moments take:
-    // 2,000 of them 21.4 us, 35.5 with one tail warp for two slots)
-    if (v == 4 && a.arr.max_P <= SMALL_PIX && !occ_only) {
-        const size_t sm8 = chain_smem_bytes(4, a.nstage, a.stage_wave_bytes, a.arr.max_P, 0, 0, SMALL_TAILS);
-        const int g8 = int(std::min<int64_t>(a.n_img, 2 * int64_t(a.n_sm)));
-        if (sm8 <= size_t(227) * 1024) return launch_lean<8, 1, 2, false, false, SMALL_TAILS>(a, g8, sm8, s, false, nullptr);
-    }
-    switch (v) {
-    case 0: return launch_lean<8, 1, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 1: return launch_lean<4, 2, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 2: return launch_lean<8, 2, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 3: return launch_lean<4, 1, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 4: return launch_lean<8, 1, 3, false>(a, grid, smem, s, occ_only, occ);   // registers for three CTAs per SM
-    default: return cudaErrorInvalidValue;
-    }
+    if (a.pp.sliding && a.pp.W != 6 && !occ_only) return dispatch_image_chain_win(v, a, grid, smem, s);
+    return dispatch_rows<6>(v, a, grid, smem, s, occ_only, occ);
 }
 
 }  // namespace rta

@@ -274,9 +274,9 @@ int chain_launch_config(rta_ctx* c, int64_t n_img, int* grid, size_t* smem, int*
     return config_launch(c, cfg_of(c, kind), n_img, grid, smem, swb, kind);
 }
 
-int needs_any_window(const rta_ctx* c, const rta::ProcParams& pp) {
+int needs_any_window(const rta_ctx* c, const rta::ProcParams& pp, bool rows) {
     for (int t = 0; t < c->n_tel; ++t)
-        if (!rta::window_specialised(pp, c->cams[c->tel_cam[t]].S)) return 1;
+        if (!rta::window_specialised(pp, c->cams[c->tel_cam[t]].S, rows)) return 1;
     return 0;
 }
 
@@ -326,7 +326,7 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
     a.stage_wave_bytes = swb;
     a.nstage = std::max(2, std::min(cfg.nstage, 8));
     a.integrate_only = integrate_only;
-    a.any_window = needs_any_window(c, pp);
+    a.any_window = needs_any_window(c, pp, !integrate_only && !d_mask && !d_smeta);
     a.n_sm = c->n_sm;
     a.n_img_dev = d_n_img;
     a.seg = d_seg;
@@ -1126,7 +1126,7 @@ int rta_graph_create(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const i
     g->pp = make_pp(c, window_mode, start, W, core_needs_neighbour, t_hi, t_lo);
     g->d_hillas = d_hillas;
     g->d_stereo = d_stereo;
-    if ((rc = graph_capture(g, needs_any_window(c, g->pp)))) {
+    if ((rc = graph_capture(g, needs_any_window(c, g->pp, true)))) {
         delete g;
         return rc;
     }
@@ -1138,7 +1138,7 @@ int rta_graph_launch(rta_graph* g, void* stream) {
     if (!g) return fail(RTA_E_INVALID, "graph is NULL");
     int rc = check_ctx(g->ctx);
     if (rc) return rc;
-    const int k = needs_any_window(g->ctx, g->pp);
+    const int k = needs_any_window(g->ctx, g->pp, true);
     if (!g->exec[k] && (rc = graph_capture(g, k))) return rc;
     CUDA_TRY(cudaGraphLaunch(g->exec[k], (cudaStream_t)stream));
     return RTA_OK;

@@ -38,9 +38,11 @@ struct ChainArgs {
 
 // Whether the fused kernel has a search compiled for S samples and windows of W (the fixed
 // window needs none): launches all of whose cameras have one run the instantiations that carry
-// no other.
-inline bool window_specialised(const ProcParams& pp, int S) {
-    return !pp.sliding || ((pp.W == 6 && (S == 40 || S == 30 || S == 25)) || (pp.W == 5 && S == 16 && !pp.nbpeak));
+// no other. rows: flat windows of a contiguous bundle, rows only.
+inline bool window_specialised(const ProcParams& pp, int S, bool rows) {
+    if (!pp.sliding) return true;
+    const bool width = pp.W == 6 || (rows && !pp.nbpeak && !pp.filter && pp.W >= 4 && pp.W <= 8);
+    return (width && (S == 40 || S == 30 || S == 25)) || (pp.W == 5 && S == 16 && !pp.nbpeak);
 }
 
 // One image of a byte stream as the image kernel's producer needs it: checked
@@ -117,6 +119,7 @@ cudaError_t dispatch_image_chain_nb(int v, const ChainArgs& a, int grid, size_t 
                                     int* occ);
 cudaError_t dispatch_image_chain_lean(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                       bool occ_only, int* occ);
+cudaError_t dispatch_image_chain_win(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                      bool occ_only, int* occ);
 cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,

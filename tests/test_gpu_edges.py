@@ -161,7 +161,10 @@ def test_generic_paths_and_largest_camera(kind, P, S, W, sliding):
     ("hex", 72, 1, 1), ("hex", 72, 2, 2), ("hex", 40, 16, 16), ("hex", 40, 17, 16), ("grid", 64, 31, 3),
     ("hex", 331, 32, 8), ("square", 1030, 48, 5), ("hex", 152, 63, 9), ("square", 257, 64, 16), ("hex", 1855, 40, 7),
     ("hex", 1000, 65, 2), ("square", 516, 96, 15), ("hex", 130, 100, 12), ("square", 1030, 112, 6),
-    ("hex", 264, 127, 16), ("square", 2049, 128, 4)])
+    ("hex", 264, 127, 16), ("square", 2049, 128, 4),
+    # widths other than 6 of the 40-, 30- and 25-sample cameras: small and large, odd rows
+    ("hex", 1855, 40, 8), ("hex", 1855, 40, 4), ("hex", 331, 40, 5), ("square", 1028, 30, 7), ("hex", 264, 30, 8),
+    ("hex", 132, 30, 4), ("hex", 1000, 25, 8), ("square", 2048, 25, 7), ("hex", 264, 25, 5), ("hex", 520, 25, 4)])
 def test_any_camera_and_window(kind, P, S, W):
     """The sliding search for cameras and windows without a specialised one: sample counts around
     a word, a block of starts and the split of long rows, odd rows, rows that share banks, pixel
