@@ -8,7 +8,7 @@ namespace rta {
 
 constexpr size_t SMEM_PER_SM = size_t(227) * 1024;
 
-// FILT: the form with the digital filter (LEAN = false, FILT = true).
+// FILT: the form with the digital filter.
 template <int IW, int PPT, int MB, bool NB, bool FILT = false, int TAILS = 1>
 static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                int* occ) {
@@ -34,8 +34,8 @@ static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStr
 cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                       bool occ_only, int* occ) {
     // variant 4 is variant 0's tile in the 64 registers that let three CTAs share an SM; where
-    // shared memory holds fewer, its spills buy nothing (4096 pixels x 128 samples: 516 us, and
-    // 478 with variant 0's 88 registers)
+    // shared memory holds fewer, variant 0's registers (90) are there to be used: 1,000 images of
+    // 4096 pixels x 128 samples, W = 16, 360 us and 370 in 64; 3,000 of 1600 x 100, W = 6, 267 and 276
     if (v == 4 && 3 * smem > SMEM_PER_SM && a.arr.max_P > SMALL_PIX) v = 0;
     if (a.pp.nbpeak) {
         switch (v) {

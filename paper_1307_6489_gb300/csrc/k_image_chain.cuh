@@ -201,14 +201,13 @@ __device__ __forceinline__ void best_key_pair(const uint16_t* row0, int one, int
     key1 = best_key_x<S, W>(x, one, k128);
 }
 
-// First start of a window whose sum is `sum`, the largest of the row's (found by the packed
-// search): a rolled loop, taken by the few pixels that reach t_lo. Every camera shares its few
+// First start, at `st` or after it, of a window whose sum is `sum`, the largest of the row's (found
+// by the packed search): a rolled loop, taken by the few pixels that reach t_lo. Every camera shares its few
 // instructions: an unrolled search per sample count (300 instructions each) pushed the hot loop
 // out of the instruction caches.
-__device__ __forceinline__ int first_start(const uint16_t* row, int S, int W, int sum) {
+__device__ __forceinline__ int first_start(const uint16_t* row, int S, int W, int sum, int st = 0) {
     int s = 0;
-    for (int k = 0; k < W; ++k) s += row[k];
-    int st = 0;
+    for (int k = 0; k < W; ++k) s += row[st + k];
 #pragma unroll 1
     while (s != sum && st < S - W) {
         s += int(row[st + W]) - int(row[st]);
@@ -238,145 +237,128 @@ __device__ __forceinline__ uint32_t spread_even(uint32_t v) {
     return v;
 }
 
-// Eight words at v into u[at..at + 7]; wide: v is 16-byte aligned.
-template <int AT>
-__device__ __forceinline__ void load_words8(const uint32_t* v, bool wide, uint32_t (&u)[16]) {
-    if (wide) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const uint4 q = reinterpret_cast<const uint4*>(v)[k];
-            u[AT + 4 * k] = q.x; u[AT + 4 * k + 1] = q.y; u[AT + 4 * k + 2] = q.z; u[AT + 4 * k + 3] = q.w;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) u[AT + k] = v[k];
-    }
-}
-
-// The W-sample sums of the sixteen windows that start in the words u[0..7], two per word
-// (low half: the window of the word's low sample). Sums of 2, 4, 8 and 16 samples are built by
-// doubling and the bits of W pick the ones a window is made of, longest last: every shift is
-// then a whole number of words known at compile time although W is not. Halves stay below
-// 16 * 4096 = 2^16, so plain 32-bit adds carry nothing from one half into the other.
-__device__ __forceinline__ void window_words(const uint32_t (&u)[16], int W, uint32_t (&r)[8]) {
-    uint32_t p[15], t[15];
-#pragma unroll
-    for (int j = 0; j < 15; ++j) {
-        p[j] = u[j] + __byte_perm(u[j], u[j + 1], 0x5432);      // 2 samples
-        t[j] = (W & 1) ? u[j] : 0u;
-    }
-    if (W & 2) {
-#pragma unroll
-        for (int j = 0; j < 14; ++j) t[j] = p[j] + t[j + 1];
-    }
-    if (W > 3) {
-#pragma unroll
-        for (int j = 0; j < 14; ++j) p[j] += p[j + 1];          // 4 samples
-        if (W & 4) {
-#pragma unroll
-            for (int j = 0; j < 12; ++j) t[j] = p[j] + t[j + 2];
-        }
-        if (W > 7) {
-#pragma unroll
-            for (int j = 0; j < 12; ++j) p[j] += p[j + 2];      // 8 samples
-            if (W == 16) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) t[j] = p[j] + p[j + 4];
-            } else {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) t[j] = p[j] + t[j + 4];
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) r[j] = t[j];
-}
-
 // The search for any sample count and any window of up to 16 samples (the cameras and windows
-// without a specialised one), eight words of window starts at a time. As in max_window_packed,
-// samples must be below 4096 (checked), and rows that start on an odd 16-bit position are read
-// from the word below. Words read past the row's end stay inside the stage (its calibration
-// rows follow) and their windows are dropped.
-// Bound: issue slots. The serial search it replaces (two 16-bit shared loads per window start,
-// all lanes of a 256-byte row stride in one bank) took 3,583 us for 1,000 images of 4096 pixels
-// x 128 samples, W = 16; this one 478 us, of which the HBM read is 155.
+// without a specialised one), eight words of a row at a time. As in max_window_packed, samples
+// must be below 4096 (checked: sums of 16 stay below 2^16, so plain 32-bit adds carry nothing
+// from one half of a word into the other), and rows that start on an odd 16-bit position are
+// read from the word below.
+// A block forms, in the order of its words, the sums of 2, 4 and 8 samples that END in them, and
+// a window is the one to four of these (and of single samples) that its width is made of: each
+// sum is formed once, and a block keeps the last few for the next. Nothing masks the windows
+// that reach out of the row: samples are not negative and what lies outside counts as 0, so such
+// a window's sum is at most the first or the last whole window's; where it is equal, the first
+// start is still the whole window's.
+// Bound: issue slots, most of them of the half-rate integer pipe. The serial search (two 16-bit
+// shared loads per window start) took 3,583 us for 1,000 images of 4096 pixels x 128 samples,
+// W = 16; blocks of window starts with the width known at run time only 473; this one 360 us,
+// of which the HBM read is 155.
 struct PackedRow {
+    const uint16_t* row;
     const uint32_t* v;
-    int W, odd, n_pos, n_row;    // n_pos: half-word positions of window starts; n_row: words of the row
+    int S, W, odd;
     bool wide;
 
-    __device__ __forceinline__ PackedRow(const uint16_t* row, int S, int W_) : W(W_) {
+    __device__ __forceinline__ PackedRow(const uint16_t* row_, int S_, int W_) : row(row_), S(S_), W(W_) {
         const uintptr_t a = reinterpret_cast<uintptr_t>(row);
         v = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
         odd = (a & 2u) ? 1 : 0;
         wide = (S & 7) == 0;     // rows of whole 16-byte pieces
-        n_pos = S - W + 1 + odd;
-        n_row = (S + odd + 1) >> 1;
     }
-    __device__ __forceinline__ int blocks() const { return (n_pos + 15) >> 4; }
+    __device__ __forceinline__ int blocks() const { return (S + odd + 15) >> 4; }
 
-    // window sums of block j0 / 8 from its words u, invalid windows as 0
-    __device__ __forceinline__ void sums(int j0, const uint32_t (&u)[16], uint32_t (&r)[8]) const {
-        window_words(u, W, r);
-        if (odd && j0 == 0) r[0] &= 0xFFFF0000u;     // the half-word before the row
-        if (2 * (j0 + 8) > n_pos) {
+    // the words of block b into u[8..15], those outside the row as 0
+    __device__ __forceinline__ void load_block(int b, uint32_t (&u)[16]) const {
+        const int left = S + odd - 16 * b;       // half-words of the row from here on
+        if (wide) {
+            const uint4* q = reinterpret_cast<const uint4*>(v + 8 * b);
+            const uint4 lo = q[0], hi = left >= 16 ? q[1] : make_uint4(0u, 0u, 0u, 0u);
+            u[8] = lo.x; u[9] = lo.y; u[10] = lo.z; u[11] = lo.w;
+            u[12] = hi.x; u[13] = hi.y; u[14] = hi.z; u[15] = hi.w;
+        } else {
+            if (left >= 16) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int left = n_pos - 2 * (j0 + k);
-                r[k] = left >= 2 ? r[k] : left == 1 ? r[k] & 0xFFFFu : 0u;
+                for (int k = 0; k < 8; ++k) u[8 + k] = v[8 * b + k];
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    u[8 + k] = 2 * k < left ? v[8 * b + k] : 0u;
+                    if (2 * k + 1 == left) u[8 + k] &= 0xFFFFu;
+                }
             }
+            if (odd && b == 0) u[8] &= 0xFFFF0000u;
         }
     }
 
-    // Largest sum of the blocks [b0, b1) and the first of them that holds it; any: the OR of
-    // their words (all blocks' together cover the row: a window is at most 16 samples).
+    // Largest sum of the windows that end in the blocks [b0, b1) and the first block that holds
+    // it; any: the OR of their words. Windows that begin before block b0 count only what lies in it.
+    template <int WW>
     __device__ __forceinline__ void best_of(int b0, int b1, int& best, int& best_b, uint32_t& any) const {
+        uint32_t u[16], p2[16], p4[16], p8[16];      // by word; 8..15: this block's
         best = 0;
         best_b = b0;
         any = 0;
-        if (b0 >= b1) return;
-        uint32_t u[16];
-        load_words8<0>(v + 8 * b0, wide, u);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) u[k] = p2[k] = p4[k] = p8[k] = 0u;
 #pragma unroll 1
-        for (int b = b0;;) {
-            const int j0 = 8 * b;
-            load_words8<8>(v + j0 + 8, wide, u);
-            if (j0 + 16 <= n_row) {
+        for (int b = b0; b < b1; ++b) {
+            load_block(b, u);
+            uint32_t r[16];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) any |= u[k];
-            } else {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) any |= j0 + k < n_row ? u[k] : 0u;
+            for (int k = 8; k < 16; ++k) {
+                any |= u[k];
+                p2[k] = u[k] + __byte_perm(u[k - 1], u[k], 0x5432);
+                p4[k] = p2[k] + p2[k - 1];
+                p8[k] = p4[k] + p4[k - 2];
+                uint32_t q = 0;
+                int o = k;
+                if (WW & 16) q = p8[o] + p8[o - 4];
+                if (WW & 8) { q += p8[o]; o -= 4; }
+                if (WW & 4) { q += p4[o]; o -= 2; }
+                if (WW & 2) { q += p2[o]; o -= 1; }
+                if (WW & 1) q += u[o];
+                r[k] = q;
             }
-            uint32_t r[8];
-            sums(j0, u, r);
-            const uint32_t m = __vimax3_u16x2(__vimax3_u16x2(r[0], r[1], r[2]), __vimax3_u16x2(r[3], r[4], r[5]),
-                                              __vmaxu2(r[6], r[7]));
+            const uint32_t m = __vimax3_u16x2(__vimax3_u16x2(r[8], r[9], r[10]), __vimax3_u16x2(r[11], r[12], r[13]),
+                                              __vmaxu2(r[14], r[15]));
             const int mb = int(max(m >> 16, m & 0xFFFFu));
             if (mb > best) {
                 best = mb;
                 best_b = b;
             }
-            if (++b == b1) break;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) u[k] = u[k + 8];
+            for (int k = 0; k < 8; ++k) {
+                u[k] = u[k + 8];
+                p2[k] = p2[k + 8];
+                p4[k] = p4[k + 8];
+                p8[k] = p8[k + 8];
+            }
         }
     }
 
-    // first window start of block b whose sum is `best`
-    __device__ __forceinline__ int start_in(int b, int best) const {
-        uint32_t u[16], r[8];
-        load_words8<0>(v + 8 * b, wide, u);
-        load_words8<8>(v + 8 * b + 8, wide, u);
-        sums(8 * b, u, r);
-        int pos = 0;
-#pragma unroll
-        for (int k = 7; k >= 0; --k) {
-            const int p = 2 * (8 * b + k);
-            if (int(r[k] >> 16) == best && p + 1 < n_pos) pos = p + 1;
-            if (int(r[k] & 0xFFFFu) == best && p < n_pos && p >= odd) pos = p;
+    __device__ __forceinline__ void best_of(int b0, int b1, int& best, int& best_b, uint32_t& any) const {
+        switch (W) {
+        case 1: return best_of<1>(b0, b1, best, best_b, any);
+        case 2: return best_of<2>(b0, b1, best, best_b, any);
+        case 3: return best_of<3>(b0, b1, best, best_b, any);
+        case 4: return best_of<4>(b0, b1, best, best_b, any);
+        case 5: return best_of<5>(b0, b1, best, best_b, any);
+        case 6: return best_of<6>(b0, b1, best, best_b, any);
+        case 7: return best_of<7>(b0, b1, best, best_b, any);
+        case 8: return best_of<8>(b0, b1, best, best_b, any);
+        case 9: return best_of<9>(b0, b1, best, best_b, any);
+        case 10: return best_of<10>(b0, b1, best, best_b, any);
+        case 11: return best_of<11>(b0, b1, best, best_b, any);
+        case 12: return best_of<12>(b0, b1, best, best_b, any);
+        case 13: return best_of<13>(b0, b1, best, best_b, any);
+        case 14: return best_of<14>(b0, b1, best, best_b, any);
+        case 15: return best_of<15>(b0, b1, best, best_b, any);
+        default: return best_of<16>(b0, b1, best, best_b, any);
         }
-        return pos - odd;
+    }
+
+    // first window start whose sum is `best`, block b the first in which a window of it ends
+    __device__ __forceinline__ int start_in(int b, int best) const {
+        return first_start(row, S, W, best, max(0, 16 * b - odd - W + 1));
     }
 };
 
@@ -956,8 +938,9 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                         const PackedRow pr(row, h.S, Wr);
                         int b0 = 0, b1 = pr.blocks(), blk;
                         if (split) {
-                            const int mid = (b1 + 1) >> 1;
-                            if (half) b0 = mid;
+                            // the upper half begins a block early: the sums that its first windows need
+                            const int mid = b1 / 2 + 1;
+                            if (half) b0 = mid - 1;
                             else b1 = mid;
                         }
                         uint32_t any;
