@@ -234,6 +234,84 @@ def test_any_camera_and_window(kind, P, S, W):
     ctx.close()
 
 
+@pytest.mark.parametrize("kind,P,S,start,W", [
+    ("hex", 331, 32, 20, 12), ("square", 1030, 32, 0, 1), ("hex", 1000, 64, 17, 16), ("square", 257, 96, 95, 1),
+    ("square", 2049, 128, 112, 16), ("hex", 130, 128, 0, 7), ("square", 1600, 100, 9, 6), ("hex", 1000, 48, 40, 8)])
+def test_fixed_window_of_long_rows(kind, P, S, start, W):
+    """The fixed window on rows of a multiple of 32 samples (chunks in padded runs, from 64 samples
+    two threads a row) and on their neighbours: decisions exact, rows within the usual rules, the
+    same through every tile shape and with one CTA an SM, samples up to full scale."""
+    rng = np.random.default_rng(100 * S + start)
+    xy, nb = synth.lattice(kind, P, 0.1)
+    n_img = 7
+    wave = rng.integers(380, 421, (n_img, P, S)).astype(np.uint16)
+    for i in range(n_img):
+        d = ((xy - xy[rng.integers(P)]) ** 2).sum(1)
+        amp = (np.array([60, 900, 3500, 60000, 200, 0, 1500])[i] * np.exp(-d / 0.02)).astype(np.int64)
+        wave[i, :, start + W // 2] = np.minimum(wave[i, :, start + W // 2] + amp, 65535)
+    p16 = np.full(P, 16 * 400, np.int32)
+    scale = (1 / (16 * 8.0 * rng.uniform(0.9, 1.1, P))).astype(np.float32)
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), p16, scale)
+    d_wave = torch.from_numpy(wave.reshape(-1).view(np.int16)).cuda()
+    off = torch.arange(n_img, dtype=torch.int64, device="cuda") * (P * S)
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    hi, lo = 10.0, 5.0
+    rows = []
+    for i in range(n_img):
+        qr, tr, _, _ = oracle.integrate(wave[i], p16, scale, False, start, W)
+        rows.append(oracle.hillas(xy, qr, tr, oracle.clean(qr, nb, hi, lo, 1)))
+    first = None
+    for config in (None, (4, 2, 1), (0, 3, 1), (1, 2, 0), (3, 4, 1)):
+        try:
+            if config:
+                ctx.set_chain_config(*config)
+        except rta.RtaError:
+            continue                                 # no room for this camera
+        out = torch.zeros(n_img * 16, dtype=torch.float32, device="cuda")
+        ctx.image_chain(d_wave, off, tel, rta.RTA_WINDOW_FIXED, start, W, hi, lo, 1, out)
+        assert ctx.check() == 0
+        raw = out.cpu().numpy().view(np.uint32)
+        if first is None:
+            first = raw
+            compare_hillas(hillas_rows(out, n_img), np.array(rows), f"{kind}{P}x{S} fixed {start}+{W}")
+        np.testing.assert_array_equal(raw, first)
+    ctx.close()
+
+
+@pytest.mark.parametrize("P,S,W", [(256, 16, 5), (331, 40, 6), (1855, 40, 6), (1600, 100, 6)])
+def test_rows_do_not_depend_on_the_launch_size(P, S, W):
+    """Launches of up to an image per SM (a deeper pipeline), up to the resident CTAs (no counter
+    reset) and beyond: each image's row is the one it has alone, call after call."""
+    rng = np.random.default_rng(P)
+    kind = "square" if P == 256 else "hex"
+    xy, nb = synth.lattice(kind, P, 0.1)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    kinds = 5                                        # distinct images, repeated
+    wave = rng.integers(380, 421, (kinds, P, S)).astype(np.uint16)
+    for i in range(kinds):
+        d = ((xy - xy[rng.integers(P)]) ** 2).sum(1)
+        wave[i, :, S // 2] += (300 * (i + 1) * np.exp(-d / 0.03)).astype(np.uint16)
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                       np.full(P, 1 / 128, np.float32))
+    d_wave = torch.from_numpy(wave.reshape(-1).view(np.int16)).cuda()
+    single = None
+    for n_img in (kinds, n_sm - 1, n_sm, n_sm + 1, 2 * n_sm, 2 * n_sm + 1, 3 * n_sm, 3 * n_sm + 1, 5 * n_sm, 3, n_sm):
+        off = (torch.arange(n_img, dtype=torch.int64, device="cuda") % kinds) * (P * S)
+        tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+        out = torch.full((n_img * 16,), -1.0, dtype=torch.float32, device="cuda")
+        ctx.image_chain(d_wave, off, tel, rta.RTA_WINDOW_SLIDING, 0, W, 10.0, 5.0, 1, out)
+        assert ctx.check() == 0
+        raw = out.cpu().numpy().view(np.uint32).reshape(n_img, 16)
+        if single is None:
+            single = raw
+        np.testing.assert_array_equal(raw, single[np.arange(n_img) % kinds])
+    ctx.close()
+
+
 def test_argument_checks(arr):
     wl, ctx = arr
     dev = Dev(wl)
