@@ -8,11 +8,11 @@ namespace rta {
 
 constexpr size_t SMEM_PER_SM = size_t(227) * 1024;
 
-// FILT: the form with the digital filter.
-template <int IW, int PPT, int MB, bool NB, bool FILT = false, int TAILS = 1>
+// FILTER 1: the form with the digital filter.
+template <int IW, int PPT, int MB, bool NB, int FILTER = 0, int TAILS = 1>
 static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILT ? 1 : 0, OUT_ROWS, true, TAILS>;
+    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILTER, OUT_ROWS, true, TAILS>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;
@@ -49,11 +49,11 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
     }
     if (a.pp.filter) {
         switch (v) {
-        case 0: return launch_any<8, 1, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_any<4, 2, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_any<8, 2, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_any<4, 1, 2, false, true>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_any<8, 1, 3, false, true>(a, grid, smem, s, occ_only, occ);
+        case 0: return launch_any<8, 1, 2, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_any<4, 2, 2, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_any<8, 2, 2, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_any<4, 1, 2, false, 1>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_any<8, 1, 3, false, 1>(a, grid, smem, s, occ_only, occ);
         default: return cudaErrorInvalidValue;
         }
     }
@@ -63,7 +63,7 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
     if (v == 4 && a.arr.max_P <= SMALL_PIX && !occ_only) {
         const size_t sm8 = chain_smem_bytes(4, a.nstage, a.stage_wave_bytes, a.arr.max_P, 0, 0, SMALL_TAILS);
         const int g8 = int(std::min<int64_t>(a.n_img, 2 * int64_t(a.n_sm)));
-        if (sm8 <= size_t(227) * 1024) return launch_any<8, 1, 2, false, false, SMALL_TAILS>(a, g8, sm8, s, false, nullptr);
+        if (sm8 <= size_t(227) * 1024) return launch_any<8, 1, 2, false, 0, SMALL_TAILS>(a, g8, sm8, s, false, nullptr);
     }
     switch (v) {
     case 0: return launch_any<8, 1, 2, false>(a, grid, smem, s, occ_only, occ);

@@ -4,16 +4,15 @@
 //
 // k_image_chain is the hot path. It is a persistent, warp-specialised kernel:
 //   warp 0      producer: takes its first image by its block index and the next ones from a
-//               global work counter, and
-//               streams it, chunk by chunk, into a ring of shared-memory stages
+//               global work counter, and streams them, chunk by chunk, into a ring of shared-memory stages
 //               with bulk copies on the TMA engine (cp.async.bulk, one mbarrier
 //               per stage, transaction-count completion); the calibration rows
 //               of the chunk's pixels travel with it;
-//   warps 1..8  consumers: one thread per pixel of the chunk computes the
+//   warps 1..IW integrators: one thread per pixel of the chunk computes the
 //               integer window sum, the single FP32 calibration multiply and the
-//               peak time, keeping q and t in shared memory; after the image's
-//               last chunk they clean it and reduce the Hillas moments with warp
-//               shuffles, while the producer already streams the next image.
+//               peak time, keeping q and t in an image slot in shared memory;
+//   the last TAILS warps clean the finished images and reduce their Hillas moments,
+//               while the integrators fill the other slots.
 // Waveform bytes are read from HBM exactly once; per-pixel values never leave
 // the SM. Every mbarrier wait is bounded by the global timer; a wait that runs
 // out sets RTA_DEV_TIMEOUT, raises a CTA-wide abort flag and the CTA drains its

@@ -1,15 +1,15 @@
 // The byte-stream instantiations of the fused image kernel (k_image_chain with
 // STREAM = true, k_image_chain.cuh): the producer copies each chunk from the
-// segments of an ingested stream; with the digital filter and without it (LEAN).
+// segments of an ingested stream; with the digital filter (FILTER 1) and without it.
 // Compiled apart so the builds run in parallel.
 #include "k_image_chain.cuh"
 
 namespace rta {
 
-template <int IW, int PPT, int MB, bool LEAN, bool ANY>
+template <int IW, int PPT, int MB, int FILTER, bool ANY>
 static cudaError_t launch_stream(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
                                  int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, false, true, LEAN ? 0 : 1, OUT_ROWS, ANY>;
+    auto kern = k_image_chain<IW, PPT, MB, false, true, FILTER, OUT_ROWS, ANY>;
     // the dynamic shared-memory opt-in is per device; remember the largest size set
     static size_t attr_bytes[64] = {};
     int dev = 0;
@@ -33,20 +33,20 @@ static cudaError_t dispatch_stream(int v, const ChainArgs& a, int grid, size_t s
                                    int* occ) {
     if (!a.pp.filter && !occ_only) {
         switch (v) {
-        case 0: return launch_stream<8, 1, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_stream<4, 2, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_stream<8, 2, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_stream<4, 1, 2, true, ANY>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_stream<8, 1, 3, true, ANY>(a, grid, smem, s, occ_only, occ);
+        case 0: return launch_stream<8, 1, 2, 0, ANY>(a, grid, smem, s, occ_only, occ);
+        case 1: return launch_stream<4, 2, 2, 0, ANY>(a, grid, smem, s, occ_only, occ);
+        case 2: return launch_stream<8, 2, 2, 0, ANY>(a, grid, smem, s, occ_only, occ);
+        case 3: return launch_stream<4, 1, 2, 0, ANY>(a, grid, smem, s, occ_only, occ);
+        case 4: return launch_stream<8, 1, 3, 0, ANY>(a, grid, smem, s, occ_only, occ);
         default: return cudaErrorInvalidValue;
         }
     }
     switch (v) {
-    case 0: return launch_stream<8, 1, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
-    case 1: return launch_stream<4, 2, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
-    case 2: return launch_stream<8, 2, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
-    case 3: return launch_stream<4, 1, 2, false, ANY>(a, grid, smem, s, occ_only, occ);
-    case 4: return launch_stream<8, 1, 3, false, ANY>(a, grid, smem, s, occ_only, occ);
+    case 0: return launch_stream<8, 1, 2, 1, ANY>(a, grid, smem, s, occ_only, occ);
+    case 1: return launch_stream<4, 2, 2, 1, ANY>(a, grid, smem, s, occ_only, occ);
+    case 2: return launch_stream<8, 2, 2, 1, ANY>(a, grid, smem, s, occ_only, occ);
+    case 3: return launch_stream<4, 1, 2, 1, ANY>(a, grid, smem, s, occ_only, occ);
+    case 4: return launch_stream<8, 1, 3, 1, ANY>(a, grid, smem, s, occ_only, occ);
     default: return cudaErrorInvalidValue;
     }
 }

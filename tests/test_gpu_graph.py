@@ -45,3 +45,44 @@ def test_graph_at_capacity_matches_direct_launches_for_any_count():
     finally:
         rta.rta_graph_destroy(g)
     ctx.close()
+
+
+@pytest.mark.parametrize("S0,S1", [(40, 48), (48, 40), (31, 30)])
+def test_graph_follows_a_camera_registered_again(S0, S1):
+    """A graph captured with a camera of S0 samples launches after the camera was registered again
+    with S1, which needs the image kernel for any window where S0 does not (or the reverse): its
+    rows are the direct launch's, before and after."""
+    P, n_img, W = 264, 9, 6
+    rng = np.random.default_rng(S0)
+    xy, nb = synth.lattice("hex", P, 0.1)
+    n = n_img * P * max(S0, S1)
+    wave = torch.from_numpy(rng.integers(380, 480, n).astype(np.int16)).cuda()
+    off = torch.zeros(n_img, dtype=torch.int64, device="cuda")
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    evt = torch.arange(n_img + 1, dtype=torch.int32, device="cuda")
+    n_d = torch.tensor([n_img], dtype=torch.int64, device="cuda")
+    h, st = torch.zeros(n_img * 16, device="cuda"), torch.zeros(n_img * 8, device="cuda")
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S0)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                       np.full(P, 1 / 128, np.float32))
+    args = (rta.RTA_WINDOW_SLIDING, 0, W, 3.0, 1.5, 1)
+    g = rta.rta_graph_create(ctx.handle, wave.data_ptr(), n, off.data_ptr(), tel.data_ptr(), n_d.data_ptr(), n_img,
+                             evt.data_ptr(), n_d.data_ptr(), n_img, *args, h.data_ptr(), st.data_ptr())
+    stream = torch.cuda.current_stream().cuda_stream
+    try:
+        for S in (S0, S1, S0):
+            torch.cuda.synchronize()
+            ctx.register_camera(5, xy, nb, S)
+            off.copy_(torch.arange(n_img, device="cuda") * (P * S))
+            ref, ref_st = torch.zeros_like(h), torch.zeros_like(st)
+            ctx.reconstruct(wave, off, tel, evt, *args, ref, ref_st)
+            h.fill_(float("nan"))
+            rta.rta_graph_launch(g, stream)
+            ctx.check(stream)
+            assert torch.equal(h.view(torch.int32), ref.view(torch.int32))
+            assert torch.equal(st.view(torch.int32), ref_st.view(torch.int32))
+            assert int(h.view(torch.int32).view(n_img, 16)[:, 10].min()) > 0
+    finally:
+        rta.rta_graph_destroy(g)
+    ctx.close()

@@ -138,6 +138,37 @@ def test_short_packets_crc_like_the_oracle():
     ctx.close()
 
 
+@pytest.mark.parametrize("seg", [50, 51, 101, 102, 408, 409, 410, 818])
+def test_crc_around_the_block_and_share_sizes(seg):
+    """Packets of 48 + 80 seg bytes: a little under and over one and two 4096-byte blocks, under, at
+    and over the 32 KiB that a warp takes, and nearly the largest; the clean stream, and one bit
+    flipped at the first sample, on either side of each block and share boundary counted from the
+    packet's start and its end, in the padding and in the CRC field itself."""
+    wl = synth.make_workload(1, 3)
+    ctx = make_ctx(wl)
+    buf, plan = synth.encode_stream(wl, seg_pixels={1: seg})
+    off, size = plan["off"], plan["size"]
+    k = int(np.argmax(size[1:])) + 1
+    L = int(size[k])
+    assert L == 48 + 80 * seg
+    d = GpuDir(len(plan["img"]) + 5, wl.n_img + 3, wl.n_evt + 1)
+    db = dev_bytes(buf)
+    r = ingest.decode_stream(buf, wl.tel_cam, cams_of(wl), verify_crc=True)
+    assert r["error"] == 0
+    compare_dirs(d.ingest(ctx, db, len(buf), True), r)
+    edges = [e for step in (512, 4096, 32768) for e in (step, 2 * step, L - step, L - 2 * step, L // step * step)]
+    at = {32, L - 17, L - 16, L - 3, L - 2, L - 1} | {e + j for e in edges for j in (-16, -1, 0, 15) if 32 <= e + j < L}
+    for i, b in enumerate(sorted(at)):
+        pos = int(off[k]) + b
+        old = int(db[pos])
+        db[pos] = old ^ (1 << (i % 8))
+        g = d.ingest(ctx, db, len(buf), True)
+        assert (g["error"], g["error_offset"]) == (ingest.CRC, off[k]), (seg, b)
+        db[pos] = old
+    compare_dirs(d.ingest(ctx, db, len(buf), True), r)
+    ctx.close()
+
+
 def test_capacities_like_the_oracle(sset):
     wl, ctx = sset
     buf, plan = synth.encode_stream(wl)
