@@ -279,4 +279,21 @@ int serve_infer(rta_model* md, const rta_hillas_t* d_h, const int32_t* d_img_tel
 // telescope registered. RTA_OK or RTA_E_INVALID / RTA_E_ALIGN with the message set.
 int check_bundle_images(rta_ctx* c, const int64_t* h_wave_off, const int32_t* h_img_tel, int64_t n_img,
                         int64_t n_wave);
+// The kernels of a training step, and those of an ingest, are launched as programmatic dependents
+// of one another: each signals at once, and waits (grid_dependency_wait) before it reads anything.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 }  // namespace rta

@@ -148,23 +148,6 @@ struct UpdateArgs {
 };
 
 cudaError_t launch_features(const FeatArgs& a, int grid, cudaStream_t s);
-// A training step's kernels are launched as programmatic dependents of one another: each
-// signals at once, and waits (grid_dependency_wait) before it reads anything.
-template <class... P, class... A>
-cudaError_t launch_dependent(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, P(args)...);
-}
-
 // Tensor-core GEMM (tcgen05) of a forward layer: A K-major, B MN-major, one split.
 cudaError_t launch_gemm(const GemmArgs& g, int n_sm, cudaStream_t s);
 // Partial sums that `splits` K-ranges of a weight gradient come to (the reduction is cut into
