@@ -326,6 +326,7 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
     a.counter = counter ? counter : take_counter(c);
     a.status = c->d_status;
     a.stage_wave_bytes = swb;
+    a.max_S = c->max_S;
     a.nstage = std::max(2, std::min(cfg.nstage, 8));
     a.integrate_only = integrate_only;
     a.any_window = needs_any_window(c, pp, !integrate_only && !d_mask && !d_smeta);

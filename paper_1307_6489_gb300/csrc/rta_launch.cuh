@@ -25,6 +25,7 @@ struct ChainArgs {
     unsigned int* status;
     int stage_wave_bytes;    // multiple of 128
     int nstage;
+    int max_S;               // longest rows of the array's cameras
     int integrate_only;
     int n_sm;                // of the device
     int any_window;          // some camera has no specialised window search (window_specialised)

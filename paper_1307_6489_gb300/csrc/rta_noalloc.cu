@@ -187,6 +187,7 @@ extern "C" int rta_image_chain_noalloc(const rta_camera_desc_t* h_cams, int n_ca
     a.counter = scratch + kCounterWord;
     a.status = scratch + kStatusWord;
     a.stage_wave_bytes = swb;
+    a.max_S = max_S;
     a.nstage = nstage;
     a.integrate_only = 0;
     a.n_sm = n_sm;
