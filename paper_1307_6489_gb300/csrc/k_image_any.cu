@@ -35,8 +35,8 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
                                       bool occ_only, int* occ) {
     // variant 4 is variant 0's tile in the 64 registers that let three CTAs share an SM; where
     // shared memory holds fewer, variant 0's registers (90) are there to be used: 1,000 images of
-    // 4096 pixels x 128 samples, W = 16, 360 us and 370 in 64; 3,000 of 1600 x 100, W = 6, 267 and 276
-    if (v == 4 && 3 * smem > SMEM_PER_SM && (a.arr.max_P > SMALL_PIX || split_rows(a.max_S))) v = 0;
+    // 4096 pixels x 128 samples, W = 16, 360 us and 370 in 64; 3,000 of 1600 x 100, W = 6, 267 and 276 (rows split)
+    if (v == 4 && 3 * smem > SMEM_PER_SM && (a.arr.max_P > SMALL_PIX || a.max_S >= 64)) v = 0;
     if (a.pp.nbpeak) {
         switch (v) {
         case 0: return launch_any<8, 1, 2, true>(a, grid, smem, s, occ_only, occ);
@@ -60,8 +60,8 @@ cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t
     // small cameras: variant 4's tile with a tail warp for each of eight slots, two CTAs an SM (an
     // image of 256 pixels is integrated in a fraction of the time its cleaning and moments take:
     // 2,000 of them 21.4 us, 35.5 with one tail warp for two slots); with rows of 64 samples and more
-    // the search sets the pace again (3,571 of 280 x 100: 102 us so, 98 with three CTAs an SM)
-    if (v == 4 && a.arr.max_P <= SMALL_PIX && !split_rows(a.max_S) && !occ_only) {
+    // the search sets the pace again (303 of 208 x 100: 30.3 us so, 28.9 with three CTAs an SM)
+    if (v == 4 && a.arr.max_P <= SMALL_PIX && a.max_S < 64 && !occ_only) {
         const size_t sm8 = chain_smem_bytes(4, a.nstage, a.stage_wave_bytes, a.arr.max_P, 0, 0, SMALL_TAILS);
         const int g8 = int(std::min<int64_t>(a.n_img, 2 * int64_t(a.n_sm)));
         if (sm8 <= size_t(227) * 1024) return launch_any<8, 1, 2, false, 0, SMALL_TAILS>(a, g8, sm8, s, false, nullptr);

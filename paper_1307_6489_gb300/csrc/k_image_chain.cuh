@@ -678,9 +678,10 @@ __host__ __device__ __forceinline__ size_t slot_bytes(int max_P) {
 constexpr int SKEW_BLOCKS = 8, SKEW_PAD = 16;
 __host__ __device__ __forceinline__ bool skewed_rows(int S) { return S >= 32 && S % 16 == 0; }
 
-// Long rows are searched by two threads each, which keeps every integrator warp busy on the
-// smaller chunks that the same stages then hold.
-__host__ __device__ __forceinline__ bool split_rows(int S) { return S >= 64; }
+// Long rows in padded runs are searched by two threads each, which keeps every integrator warp busy
+// on the smaller chunks that the same stages then hold. (Other long rows are not: 3,000 images of
+// 1600 pixels x 100 samples, W = 6, 230 us, 267 split.)
+__host__ __device__ __forceinline__ bool split_rows(int S) { return S >= 64 && skewed_rows(S); }
 
 __host__ __device__ __forceinline__ int chunk_pixels(int chunk, int stage_wave_bytes, int S) {
     const int slack = skewed_rows(S) ? 16 + (SKEW_BLOCKS - 1) * SKEW_PAD : 16;

@@ -235,7 +235,7 @@ int config_launch(rta_ctx* c, const ChainCfg& k, int64_t n_img, int* grid, size_
     const int want = k.ctas_per_sm > 0 ? k.ctas_per_sm : rta::chain_variant_min_blocks(k.variant);
     // smaller stages (still at least 128 pixels of the longest camera per chunk) so that the
     // requested number of CTAs fits on an SM, or else as many as can (3,000 images of 1600 pixels
-    // x 100 samples: 267 us with two of three CTAs, 418 with the full stages' one)
+    // x 100 samples, then split: 267 us with two of three CTAs, 418 with the full stages' one)
     const bool fits = occ >= 1;
     for (int w = want; occ < w && (w == want || fits); --w) {
         for (int s2 = (*swb - 1024) & ~127; s2 >= 4096; s2 -= 1024) {
