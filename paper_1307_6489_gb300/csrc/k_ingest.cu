@@ -165,6 +165,7 @@ __global__ void __launch_bounds__(ING_SCAN_THREADS) k_frame_scan(const IngestArg
     if (threadIdx.x == 0) found = b == 0 ? 0 : LLONG_MAX;
     __syncthreads();
     for (int64_t r0 = c0; b > 0 && r0 < c1; r0 += 16 * ING_SCAN_THREADS * ING_SCAN_UNROLL) {
+        bool hit = false;
         uint4 h[ING_SCAN_UNROLL];
 #pragma unroll
         for (int k = 0; k < ING_SCAN_UNROLL; ++k) {
@@ -175,10 +176,14 @@ __global__ void __launch_bounds__(ING_SCAN_THREADS) k_frame_scan(const IngestArg
 #pragma unroll
         for (int k = 0; k < ING_SCAN_UNROLL; ++k) {
             const int64_t pos = r0 + 16 * (ING_SCAN_THREADS * k + int64_t(threadIdx.x));
-            if (header_like(h[k]) && plausible_start(a.stream, pos, a.n_bytes, a.arr)) atomicMin(&found, (long long)pos);
+            if (header_like(h[k]) && plausible_start(a.stream, pos, a.n_bytes, a.arr)) {
+                atomicMin(&found, (long long)pos);
+                hit = true;
+            }
         }
-        __syncthreads();
-        if (found != LLONG_MAX) break;
+        // the barrier decides for the whole block: a warp that read `found` itself could already
+        // see the next round's and leave alone
+        if (__syncthreads_or(hit)) break;
     }
     if (threadIdx.x == 0) {
         IngChunk ch = {};
