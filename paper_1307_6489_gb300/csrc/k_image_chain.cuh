@@ -226,6 +226,22 @@ __device__ __forceinline__ int best_key_serial(const uint16_t* row, int S, int W
     return key;
 }
 
+// The same where none of a launch's own cameras come: as little code as it goes. (In place of
+// best_key_serial, which the bright pixels of 4096 and more take, rolled loops cost the
+// 10,000-event bundle 7 %, 865 us.)
+__device__ __forceinline__ int best_key_rolled(const uint16_t* row, int S, int W) {
+    int s = 0;
+#pragma unroll 1
+    for (int k = 0; k < W; ++k) s += row[k];
+    int key = s * 128 + 127;
+#pragma unroll 1
+    for (int k = 1; k + W <= S; ++k) {
+        s += int(row[k + W - 1]) - int(row[k - 1]);
+        key = max(key, s * 128 + (127 - k));
+    }
+    return key;
+}
+
 // Bits 0..15 of v spread to the even bit positions.
 __device__ __forceinline__ uint32_t spread_even(uint32_t v) {
     v &= 0xFFFFu;
@@ -371,12 +387,14 @@ __device__ __forceinline__ int best_key_generic(const uint16_t* row, int S, int 
 }
 
 // Window start and integer sum of one pixel whose S samples start at `row`
-// (shared memory), for the cameras without a specialised search.
+// (shared memory), for the cameras without a specialised search. A search is part of every
+// kernel: a caller's own capture of a launch stays with the kernel it was captured with when
+// a camera is registered again with a sample count that has no compiled search there.
 template <bool ANY>
 __device__ __forceinline__ void window_sum(const uint16_t* row, int S, const ProcParams& pp, int& sum, int& st) {
     const int W = pp.W;
-    if (ANY && pp.sliding) {
-        const int key = best_key_serial(row, S, W);
+    if (pp.sliding) {
+        const int key = ANY ? best_key_serial(row, S, W) : best_key_rolled(row, S, W);
         sum = key >> 7;
         st = 127 - (key & 127);
     } else {
@@ -717,7 +735,8 @@ struct NbShared {
     int* n_cand;          // candidates so far in this image
 };
 
-template <int S, int W, int IT, int PPT, bool INTEG>
+// ANY: the generic path (S == 0) has the packed search for any window, else the rolled one.
+template <int S, int W, int IT, int PPT, bool INTEG, bool ANY = false>
 __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
                                               const unsigned char* buf, const int32_t* cp16, const float* cscale,
                                               const NbShared& nb, const SlotView& v, int ct, int lane) {
@@ -746,7 +765,8 @@ __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcPara
                 int key;
                 if constexpr (S != 0 && !INTEG && W == 6) key = best_key_serial(row, S, W);
                 else if constexpr (S != 0) key = best_key_T<S, W>(row, pp.one, pp.k128);
-                else key = best_key_generic(row, Sr, Wr);
+                else if constexpr (ANY) key = best_key_generic(row, Sr, Wr);
+                else key = best_key_rolled(row, Sr, Wr);
                 q0 = charge(key >> 7, Wr, cp16[c], cscale[c], num);
                 st = 127 - (key & 127);
             }
@@ -823,8 +843,8 @@ __device__ __forceinline__ void nb_pixel(const ChainArgs& a, const ProcParams& p
 // compile-time for the specialised sliding-window cameras (the camera is the
 // same for the whole chunk, so the dispatch happens once per chunk); S == 0 is
 // the generic path with run-time S and W.
-// ANY: the generic path (S == 0) searches sliding windows; without it only the fixed window is
-// left there. SKEW: chunks of skewed_rows cameras are laid out in SKEW_BLOCKS runs, and
+// ANY: the generic path (S == 0) has the packed search for any sliding window; without it the
+// fixed window and the rolled search. SKEW: chunks of skewed_rows cameras are laid out in SKEW_BLOCKS runs, and
 // split_rows cameras take two threads a pixel.
 template <int S, int W, int IT, int PPT, bool INTEG, int FILTER, bool ANY = false, bool SKEW = false>
 __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
@@ -1034,9 +1054,11 @@ static __device__ __forceinline__ int stream_chunk_copy(const ChainArgs& a, cons
 // combination is a separate instantiation, so that every kernel carries only the
 // code of the calls it serves (branches left in, even untaken, cost the hot loop
 // instruction-cache misses and scheduling).
-// ANY: the sliding search that takes any sample count and window width; without it the kernel
-// has only the specialised ones (and the fixed window), for launches all of whose cameras have one (its code and
-// registers, left in, cost those launches 11 % on the 10,000-event bundle, 926 against 834 us).
+// ANY: the packed search that takes any sample count and window width; without it the kernel has
+// the specialised ones and the fixed window, for launches all of whose cameras have one (its code and
+// registers, left in, cost those launches 11 % on the 10,000-event bundle, 926 against 834 us),
+// and a rolled serial search for a camera that gets another sample count after a capture (0.7 % of
+// 2,000 events with the neighbour-peak window, 1 % of 2,000 images of 256 pixels, else nothing).
 // OUT: what a launch writes -- Hillas rows, charges and times only (the integrate-only call), or
 // rows and cleaning masks.
 enum { OUT_ROWS = 0, OUT_CHARGES = 1, OUT_MASKS = 2 };
@@ -1365,8 +1387,8 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
                 nb_keys_chunk<30, 6, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             else if (pp.W == 6 && h.S == 25)
                 nb_keys_chunk<25, 6, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
-            else if constexpr (ANY)
-                nb_keys_chunk<0, 0, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
+            else
+                nb_keys_chunk<0, 0, IT, PPT, integ, ANY>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
             if (++stage == NST) { stage = 0; phase ^= 1u; }

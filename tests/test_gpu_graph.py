@@ -86,3 +86,52 @@ def test_graph_follows_a_camera_registered_again(S0, S1):
     finally:
         rta.rta_graph_destroy(g)
     ctx.close()
+
+
+@pytest.mark.parametrize("P", [264, 1000])
+@pytest.mark.parametrize("mode,W", [(rta.RTA_WINDOW_SLIDING, 6), (rta.RTA_WINDOW_SLIDING, 8),
+                                    (rta.RTA_WINDOW_NEIGHBOUR, 6), (rta.RTA_WINDOW_FILTER, 6)])
+def test_a_callers_capture_follows_a_camera_registered_again(mode, W, P):
+    """A capture of rta_reconstruct by the caller keeps the image kernel it was captured with, here the
+    one that has a compiled search for 40 samples alone. Its rows stay the direct call's when the
+    camera comes back with other sample counts (odd, below and above, one that the direct call
+    serves with padded runs)."""
+    n_img, S0 = 11, 40
+    rng = np.random.default_rng(P + W)
+    xy, nb = synth.lattice("hex", P, 0.1)
+    n = n_img * P * 48
+    wave = rng.integers(380, 480, n)
+    wave[::97] += 900                                # peaks here and there, and samples beyond 12 bits
+    wave[:: 50021] = 5000
+    wave = torch.from_numpy(wave.astype(np.int16)).cuda()
+    off = torch.arange(n_img, device="cuda") * (P * S0)
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    evt = torch.tensor([0, 4, 5, 5, n_img], dtype=torch.int32, device="cuda")
+    h, st = torch.zeros(n_img * 16, device="cuda"), torch.zeros(4 * 8, device="cuda")
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S0)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                       np.full(P, 1 / 128, np.float32))
+    if mode == rta.RTA_WINDOW_FILTER:
+        rta.rta_set_filter_weights(ctx.handle, [1, 4, 9, 8, 4, 2])
+    args = (mode, 0, W, 3.0, 1.5, 1)
+    ctx.reconstruct(wave, off, tel, evt, *args, h, st)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ctx.reconstruct(wave, off, tel, evt, *args, h, st)
+    for S in (S0, 31, 48, 24, S0):
+        torch.cuda.synchronize()
+        ctx.register_camera(5, xy, nb, S)
+        off.copy_(torch.arange(n_img, device="cuda") * (P * S))
+        ref, ref_st = torch.zeros_like(h), torch.zeros_like(st)
+        ctx.reconstruct(wave, off, tel, evt, *args, ref, ref_st)
+        h.fill_(float("nan"))
+        st.fill_(float("nan"))
+        g.replay()
+        torch.cuda.synchronize()
+        assert ctx.check() == 0
+        assert torch.equal(h.view(torch.int32), ref.view(torch.int32)), S
+        assert torch.equal(st.view(torch.int32), ref_st.view(torch.int32)), S
+        assert int(h.view(torch.int32).view(n_img, 16)[:, 10].min()) > 0
+    ctx.close()
