@@ -155,7 +155,13 @@ int rta_destroy(rta_ctx* ctx);
 /* Register camera type `cam` (0 <= cam < 16): n_pix pixels (1..4096), n_samples
  * samples per pixel (1..128, n_pix*n_samples a multiple of 8), pixel centres
  * h_pix_xy[2*p], h_pix_xy[2*p+1] in degrees, and neighbour lists
- * h_nb[p*K + j] (pixel ids, -1 padded, 1 <= K <= 8). Host arrays are copied. */
+ * h_nb[p*K + j] (pixel ids, -1 padded, 1 <= K <= 8). Host arrays are copied.
+ * A camera may be registered again while no call of the context is in flight.
+ * With more pixels than its telescopes have calibration rows for, its images are
+ * skipped (RTA_HF_BAD_INPUT, RTA_DEV_BAD_IMAGE) until rta_register_array. A
+ * caller's own CUDA graph of a call follows the camera, but was set up for the
+ * cameras of its capture: images with more pixels than the largest of those, rows
+ * too long for its buffers or shorter than the window are skipped in the same way. */
 int rta_register_camera(rta_ctx* ctx, int cam, int n_pix, int n_samples, const float* h_pix_xy,
                         const int16_t* h_nb, int K);
 
@@ -166,7 +172,8 @@ int rta_register_camera(rta_ctx* ctx, int cam, int n_pix, int n_samples, const f
  * h_scale[row] = 1 / (16 * gain * window containment) that converts the
  * 1/16-ADC window numerator into photoelectrons (finite and > 0, else
  * RTA_E_INVALID). Rows of telescope t start at sum of n_pix of telescopes < t.
- * Host arrays are copied. */
+ * Host arrays are copied. Replaces the array's device tables, which a caller's own
+ * CUDA graph of a call reads: capture it again. */
 int rta_register_array(rta_ctx* ctx, int n_tel, const int32_t* h_tel_cam, const float* h_tel_xy,
                        const int32_t* h_p16, const float* h_scale);
 
@@ -312,15 +319,18 @@ int rta_reconstruct(rta_ctx* ctx, const uint16_t* d_wave, int64_t n_wave, const 
                     int start, int W, float t_hi, float t_lo, int core_needs_neighbour, rta_hillas_t* d_hillas,
                     rta_stereo_t* d_stereo, void* stream);
 
-/* The pass of rta_reconstruct captured once into a CUDA graph (one memset and
- * two kernel launches) for repeated launches on fixed buffers. The graph is
+/* The pass of rta_reconstruct captured into a CUDA graph (two kernel launches,
+ * before them a memset unless the capacity is an image per block at most) for
+ * repeated launches on fixed buffers. The graph is
  * captured at capacity (max_img images, max_evt events); the actual counts are
  * read at run time from the device-resident int64 values *d_n_img (<= max_img)
  * and *d_n_evt (<= max_evt), so one graph serves bundles of any size up to its
  * capacity: write the counts (and the bundle) on the launch stream, then
  * rta_graph_launch. All buffers must stay valid for the graph's lifetime; the
- * launch configuration is the context's at capture time. Launches of one graph
- * must not overlap on the GPU (they share a work counter). */
+ * launch configuration is the context's at capture time. The first launch after
+ * a camera or an array was registered captures the pass again, and returns
+ * RTA_E_INVALID when the window no longer fits the array's cameras. Launches of
+ * one graph must not overlap on the GPU (they share a work counter). */
 typedef struct rta_graph rta_graph;
 int rta_graph_create(rta_ctx* ctx, const uint16_t* d_wave, int64_t n_wave, const int64_t* d_wave_off,
                      const int32_t* d_img_tel, const int64_t* d_n_img, int64_t max_img, const int32_t* d_evt_off,

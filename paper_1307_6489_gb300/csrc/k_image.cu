@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(UNF_WARPS * 32) k_clean(const CleanArgs a) {
             continue;
         }
         const DevCam C = a.arr.cams[a.arr.tel_cam[tel]];
-        if (off < 0 || off + C.P > a.n_q) {
+        if (off < 0 || off + C.P > a.n_q || C.P > a.arr.max_P) {      // max_P: a captured launch's shared memory
             if (threadIdx.x == 0) atomicOr(a.status, RTA_DEV_BAD_IMAGE);
             continue;
         }
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(UNF_WARPS * 32) k_hillas(const HillasArgs a) {
         DevCam C = {};
         if (!bad) {
             C = a.arr.cams[a.arr.tel_cam[tel]];
-            bad = off < 0 || off + C.P > a.n_q;
+            bad = off < 0 || off + C.P > a.n_q || C.P > a.arr.max_P;
         }
         if (bad) {
             if (threadIdx.x == 0) {

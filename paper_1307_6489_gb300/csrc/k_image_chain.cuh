@@ -684,9 +684,6 @@ __host__ __device__ __forceinline__ size_t slot_bytes(int max_P) {
     return size_t(max_P) * 8 + size_t(8) * ((max_P + 31) / 32);
 }
 
-// Pixels of camera S per stage: a multiple of 32 (chunks start on bitmap words)
-// that fits the stage's waveform area with 16 bytes of slack for the unaligned
-// row loads of odd sample counts.
 // Rows of 64, 96, 128 ... bytes put eight neighbouring rows on the same shared-memory banks
 // (two to eight of them; 128-bit loads are served eight lanes at a time). The kernel without a
 // specialised search stages such a chunk as SKEW_BLOCKS runs of consecutive pixels, SKEW_PAD
@@ -701,9 +698,15 @@ __host__ __device__ __forceinline__ bool skewed_rows(int S) { return S >= 32 && 
 // 1600 pixels x 100 samples, W = 6, 230 us, 267 split.)
 __host__ __device__ __forceinline__ bool split_rows(int S) { return S >= 64 && skewed_rows(S); }
 
+// Bytes of a stage beside its rows: the padding between runs, and 16 for the unaligned row loads of
+// odd sample counts.
+__host__ __device__ __forceinline__ int row_slack(int S) {
+    return skewed_rows(S) ? 16 + (SKEW_BLOCKS - 1) * SKEW_PAD : 16;
+}
+
+// Pixels of a camera of S samples per stage: a multiple of 32 (chunks start on bitmap words).
 __host__ __device__ __forceinline__ int chunk_pixels(int chunk, int stage_wave_bytes, int S) {
-    const int slack = skewed_rows(S) ? 16 + (SKEW_BLOCKS - 1) * SKEW_PAD : 16;
-    const int cp = ((stage_wave_bytes - slack) / (2 * S)) & ~31;
+    const int cp = ((stage_wave_bytes - row_slack(S)) / (2 * S)) & ~31;
     return cp < chunk ? cp : chunk;
 }
 
@@ -1139,6 +1142,7 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
         if (tid != 0) return;
         // a graph captured at capacity reads the bundle's image count at run time
         const int64_t n_img = a.n_img_dev ? min(*a.n_img_dev, a.n_img) : a.n_img;
+        const int min_S = (a.pp.sliding ? 0 : a.pp.start) + a.pp.W;
         const uint64_t pol_stream = l2_policy_evict_first();
         const uint64_t pol_keep = l2_policy_evict_last();
         int stage = 0;
@@ -1222,9 +1226,13 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
                     P = C.P;
                     S = C.S;
                     row = a.arr.tel_row[tel];
-                    bad = woff + int64_t(P) * S > a.n_wave;   // never read past the waveform buffer
+                    // never read past the waveform buffer or the telescope's calibration
+                    bad = woff + int64_t(P) * S > a.n_wave || row < 0;
                 }
             }
+            // A launch takes a camera when its shared memory holds the pixels, a stage 32 of the rows
+            // (chunk_pixels), a row the window: one registered again after a capture may not fit.
+            bad = bad || P > maxP || 64 * S + row_slack(S) > a.stage_wave_bytes || S < min_S;
             if (!bad && integ) {
                 poff = a.pix_off[img];
                 bad = poff < 0 || poff + P > a.n_q;            // never write past q / t
@@ -1371,7 +1379,7 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
             nb_fph ^= 1u;
         }
         if (h.base == 0 && !integ) {
-            // the slot must be free: the tail warp is done with the image two back
+            // the slot must be free: its tail warp is done with the image NSLOT back
             if (!mbar_wait(&sm.slot_free[slot], sphase ^ 1u, abort_flag)) { give_up(); break; }
         }
         const unsigned char* buf = stages + size_t(stage) * stage_bytes;

@@ -634,6 +634,7 @@ __global__ void __launch_bounds__(256) k_stream_meta(const ChainArgs a, StreamIm
             m.P = C.P;
             m.S = C.S;
             m.row = a.arr.tel_row[tel];
+            ok = m.row >= 0;
         }
         const int seg0 = a.img_seg[i], seg1 = a.img_seg[i + 1];
         ok = ok && seg0 >= 0 && seg1 > seg0 && seg1 <= a.n_seg;

@@ -86,6 +86,9 @@ struct rta_ctx {
     int32_t* d_tel_cam = nullptr;
     float2* d_tel_xy = nullptr;
     int64_t* d_tel_row = nullptr;
+    std::vector<int64_t> tel_row;
+    std::vector<int> tel_pix;     // pixels of the telescope's camera when the array was registered
+    unsigned registrations = 0;   // of cameras and arrays: what a captured launch was set up for
     int32_t* d_p16 = nullptr;
     float* d_scale = nullptr;
     unsigned int* d_status = nullptr;
@@ -158,6 +161,13 @@ int refresh_cams(rta_ctx* c) {
         dc[i].nb = h.d_nb;
     }
     CUDA_TRY(cudaMemcpy(c->d_cams, dc, sizeof dc, cudaMemcpyHostToDevice));
+    if (c->n_tel > 0) {
+        // a telescope whose camera has outgrown its calibration rows has none
+        std::vector<int64_t> row(c->tel_row);
+        for (int t = 0; t < c->n_tel; ++t)
+            if (c->cams[c->tel_cam[t]].P > c->tel_pix[t]) row[t] = -1;
+        CUDA_TRY(cudaMemcpy(c->d_tel_row, row.data(), sizeof(int64_t) * c->n_tel, cudaMemcpyHostToDevice));
+    }
     return RTA_OK;
 }
 
@@ -509,6 +519,7 @@ int rta_register_camera(rta_ctx* c, int cam, int n_pix, int n_samples, const flo
             if (v < -1 || v >= n_pix || v == p) return fail(RTA_E_INVALID, "neighbour %d of pixel %d is invalid", v, p);
             nb[size_t(p) * RTA_NB_PAD + j] = int16_t(v);
         }
+    ++c->registrations;
     HostCam& h = c->cams[cam];
     cudaFree(h.d_xy);
     cudaFree(h.d_nb);
@@ -541,12 +552,14 @@ int rta_register_array(rta_ctx* c, int n_tel, const int32_t* h_tel_cam, const fl
                 return fail(RTA_E_INVALID, "calibration scale %lld is not finite and positive", (long long)r);
     }
     std::vector<int64_t> row(n_tel);
+    std::vector<int> pix(n_tel);
     int64_t rows = 0, src_rows = 0;
     for (int t = 0; t < n_tel; ++t) {
         int cam = h_tel_cam[t];
         if (cam < 0 || cam >= RTA_MAX_CAMS || !c->cams[cam].valid)
             return fail(RTA_E_INVALID, "telescope %d uses unregistered camera %d", t, cam);
         row[t] = rows;
+        pix[t] = c->cams[cam].P;
         rows += (c->cams[cam].P + RTA_CALIB_ALIGN - 1) / RTA_CALIB_ALIGN * RTA_CALIB_ALIGN;
         src_rows += c->cams[cam].P;
     }
@@ -562,6 +575,7 @@ int rta_register_array(rta_ctx* c, int n_tel, const int32_t* h_tel_cam, const fl
         }
         s += P;
     }
+    ++c->registrations;
     cudaFree(c->d_tel_cam); cudaFree(c->d_tel_xy); cudaFree(c->d_tel_row); cudaFree(c->d_p16); cudaFree(c->d_scale);
     c->d_tel_cam = nullptr; c->d_tel_xy = nullptr; c->d_tel_row = nullptr; c->d_p16 = nullptr; c->d_scale = nullptr;
     c->n_tel = 0;
@@ -576,6 +590,8 @@ int rta_register_array(rta_ctx* c, int n_tel, const int32_t* h_tel_cam, const fl
     CUDA_TRY(cudaMemcpy(c->d_p16, p16.data(), sizeof(int32_t) * rows, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(c->d_scale, scale.data(), sizeof(float) * rows, cudaMemcpyHostToDevice));
     c->tel_cam.assign(h_tel_cam, h_tel_cam + n_tel);
+    c->tel_row = row;
+    c->tel_pix = pix;
     c->n_tel = n_tel;
     (void)src_rows;
     return RTA_OK;
@@ -1053,13 +1069,13 @@ int rta_selftest_wait_timeout(rta_ctx* c, int timeout_ms, uint64_t* waited_ns, v
     return RTA_OK;
 }
 
-// exec[k]: the pass captured with the image kernel that carries the search for any window
-// (k = 1) or only the specialised ones (k = 0). A camera registered after the capture may need
-// the other one, which is then captured at the launch.
+// The captured launches are set up for the registered cameras and hold the array's tables, so a
+// launch after another registration captures the pass again.
 struct rta_graph {
     rta_ctx* ctx = nullptr;
-    cudaGraph_t graph[2] = {};
-    cudaGraphExec_t exec[2] = {};
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    unsigned registrations = 0;      // the context's when it was captured
     unsigned int* counter = nullptr;
     const uint16_t* d_wave;
     int64_t n_wave;
@@ -1075,10 +1091,16 @@ struct rta_graph {
     rta_stereo_t* d_stereo;
 };
 
-static int graph_capture(rta_graph* g, int k) {
+static int graph_capture(rta_graph* g) {
+    const rta::ProcParams& pp = g->pp;
+    int rc = check_array(g->ctx);
+    if (rc || (rc = check_proc(g->ctx, pp.sliding ? RTA_WINDOW_SLIDING : RTA_WINDOW_FIXED, pp.start, pp.W, false, 0.f, 0.f)))
+        return rc;
+    const unsigned registrations = g->ctx->registrations;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
     cudaStream_t s = nullptr;
     if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return fail(RTA_E_CUDA, "stream creation failed");
-    int rc = RTA_OK;
     cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         rc = run_chain(g->ctx, g->d_wave, g->n_wave, g->d_wave_off, g->d_img_tel, nullptr, g->max_img, g->pp, nullptr,
@@ -1086,19 +1108,24 @@ static int graph_capture(rta_graph* g, int k) {
         if (!rc)
             rc = run_stereo(g->ctx, g->d_hillas, g->d_img_tel, g->max_img, g->d_evt_off, g->max_evt, g->d_stereo, s,
                             g->d_n_img, g->d_n_evt);
-        cudaError_t e2 = cudaStreamEndCapture(s, &g->graph[k]);
+        cudaError_t e2 = cudaStreamEndCapture(s, &graph);
         if (!rc && e2 != cudaSuccess) rc = fail(RTA_E_CUDA, "capture failed: %s", cudaGetErrorString(e2));
     } else {
         rc = fail(RTA_E_CUDA, "cudaStreamBeginCapture: %s", cudaGetErrorString(e));
     }
-    if (!rc && cudaGraphInstantiate(&g->exec[k], g->graph[k], 0) != cudaSuccess)
-        rc = fail(RTA_E_CUDA, "graph instantiation failed");
+    if (!rc && cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) rc = fail(RTA_E_CUDA, "graph instantiation failed");
     cudaStreamDestroy(s);
-    if (rc && g->graph[k]) {
-        cudaGraphDestroy(g->graph[k]);
-        g->graph[k] = nullptr;
+    if (rc) {
+        if (graph) cudaGraphDestroy(graph);
+        return rc;
     }
-    return rc;
+    // (the launches still in flight of an executable that is destroyed complete)
+    if (g->exec) cudaGraphExecDestroy(g->exec);
+    if (g->graph) cudaGraphDestroy(g->graph);
+    g->graph = graph;
+    g->exec = exec;
+    g->registrations = registrations;
+    return RTA_OK;
 }
 
 int rta_graph_create(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t* d_wave_off,
@@ -1129,7 +1156,7 @@ int rta_graph_create(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const i
     g->pp = make_pp(c, window_mode, start, W, core_needs_neighbour, t_hi, t_lo);
     g->d_hillas = d_hillas;
     g->d_stereo = d_stereo;
-    if ((rc = graph_capture(g, needs_any_window(c, g->pp, true)))) {
+    if ((rc = graph_capture(g))) {
         delete g;
         return rc;
     }
@@ -1141,19 +1168,16 @@ int rta_graph_launch(rta_graph* g, void* stream) {
     if (!g) return fail(RTA_E_INVALID, "graph is NULL");
     int rc = check_ctx(g->ctx);
     if (rc) return rc;
-    const int k = needs_any_window(g->ctx, g->pp, true);
-    if (!g->exec[k] && (rc = graph_capture(g, k))) return rc;
-    CUDA_TRY(cudaGraphLaunch(g->exec[k], (cudaStream_t)stream));
+    if (g->registrations != g->ctx->registrations && (rc = graph_capture(g))) return rc;
+    CUDA_TRY(cudaGraphLaunch(g->exec, (cudaStream_t)stream));
     return RTA_OK;
 }
 
 int rta_graph_destroy(rta_graph* g) {
     if (!g) return RTA_OK;
     cudaSetDevice(g->ctx->device);
-    for (int k = 0; k < 2; ++k) {
-        if (g->exec[k]) cudaGraphExecDestroy(g->exec[k]);
-        if (g->graph[k]) cudaGraphDestroy(g->graph[k]);
-    }
+    if (g->exec) cudaGraphExecDestroy(g->exec);
+    if (g->graph) cudaGraphDestroy(g->graph);
     delete g;
     return RTA_OK;
 }

@@ -30,7 +30,7 @@ struct DevArray {
     const DevCam* cams;      // RTA_MAX_CAMS entries in device memory
     const int32_t* tel_cam;  // n_tel
     const float2* tel_xy;    // n_tel (m)
-    const int64_t* tel_row;  // n_tel: first (8-aligned) calibration row
+    const int64_t* tel_row;  // n_tel: first (8-aligned) calibration row; -1: fewer rows than pixels
     const int32_t* p16;      // padded calibration table
     const float* scale;
     int n_tel;

@@ -135,3 +135,104 @@ def test_a_callers_capture_follows_a_camera_registered_again(mode, W, P):
         assert torch.equal(st.view(torch.int32), ref_st.view(torch.int32)), S
         assert int(h.view(torch.int32).view(n_img, 16)[:, 10].min()) > 0
     ctx.close()
+
+
+def camera_case(rng, n_img, P_max, S_max):
+    """Device buffers of n_img images of one telescope, for cameras up to P_max x S_max."""
+    n = n_img * P_max * S_max
+    wave = torch.from_numpy(rng.integers(380, 480, n).astype(np.int16)).cuda()
+    off = torch.zeros(n_img, dtype=torch.int64, device="cuda")
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    evt = torch.arange(n_img + 1, dtype=torch.int32, device="cuda")
+    return wave, off, tel, evt, torch.zeros(n_img * 16, device="cuda"), torch.zeros(n_img * 8, device="cuda")
+
+
+def register(ctx, P, S, array=True):
+    xy, nb = synth.lattice("hex", P, 0.1)
+    ctx.register_camera(5, xy, nb, S)
+    if array:
+        ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                           np.full(P, 1 / 128, np.float32))
+
+
+@pytest.mark.parametrize("mode", [rta.RTA_WINDOW_SLIDING, rta.RTA_WINDOW_NEIGHBOUR])
+def test_graph_follows_growing_cameras_and_arrays(mode):
+    """The graph's launches match the direct call's after the camera came back with more pixels and
+    longer rows (of the same kind of search and of the other), the array registered with it; a
+    window wider than the rows is refused, and the graph launches again after a longer camera."""
+    n_img, W = 9, 6
+    wave, off, tel, evt, h, st = camera_case(np.random.default_rng(3), n_img, 2048, 128)
+    ctx = rta.Context(0)
+    register(ctx, 264, 9)
+    n_d = torch.tensor([n_img], dtype=torch.int64, device="cuda")
+    args = (mode, 0, W, 3.0, 1.5, 1)
+    g = rta.rta_graph_create(ctx.handle, wave.data_ptr(), wave.numel(), off.data_ptr(), tel.data_ptr(), n_d.data_ptr(),
+                             n_img, evt.data_ptr(), n_d.data_ptr(), n_img, *args, h.data_ptr(), st.data_ptr())
+    stream = torch.cuda.current_stream().cuda_stream
+    try:
+        for P, S in [(264, 9), (264, 128), (2048, 31), (1000, 5), (1000, 40), (2048, 40), (264, 30), (520, 128)]:
+            torch.cuda.synchronize()
+            register(ctx, P, S)
+            off.copy_(torch.arange(n_img, device="cuda") * (P * S))
+            if S < W:
+                with pytest.raises(rta.RtaError) as e:
+                    rta.rta_graph_launch(g, stream)
+                assert e.value.code == rta.RTA_E_INVALID
+                continue
+            ref, ref_st = torch.zeros_like(h), torch.zeros_like(st)
+            ctx.reconstruct(wave, off, tel, evt, *args, ref, ref_st)
+            h.fill_(float("nan"))
+            rta.rta_graph_launch(g, stream)
+            assert ctx.check(stream) == 0
+            assert torch.equal(h.view(torch.int32), ref.view(torch.int32)), (P, S)
+            assert torch.equal(st.view(torch.int32), ref_st.view(torch.int32)), (P, S)
+            assert int(h.view(torch.int32).view(n_img, 16)[:, 10].min()) > 0
+    finally:
+        rta.rta_graph_destroy(g)
+    ctx.close()
+
+
+@pytest.mark.parametrize("mode,start,W", [(rta.RTA_WINDOW_SLIDING, 0, 6), (rta.RTA_WINDOW_FIXED, 20, 6),
+                                          (rta.RTA_WINDOW_NEIGHBOUR, 0, 6)])
+def test_a_capture_flags_images_that_it_was_not_set_up_for(mode, start, W):
+    """A caller's capture replayed after the camera came back larger than its shared memory, with rows
+    too long for its stages or too short for the window: every image is flagged and none read;
+    once the camera is the old one again the rows are too. More pixels than the telescope has
+    calibration rows for are flagged by direct calls as well."""
+    n_img = 9
+    wave, off, tel, evt, h, st = camera_case(np.random.default_rng(4), n_img, 520, 128)
+    ctx = rta.Context(0)
+    S0 = 30 if mode == rta.RTA_WINDOW_FIXED else 9
+    register(ctx, 264, S0)
+    off.copy_(torch.arange(n_img, device="cuda") * (264 * S0))
+    args = (mode, start, W, 3.0, 1.5, 1)
+    first, first_st = torch.zeros_like(h), torch.zeros_like(st)
+    ctx.reconstruct(wave, off, tel, evt, *args, first, first_st)
+    assert ctx.check() == 0
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ctx.reconstruct(wave, off, tel, evt, *args, h, st)
+
+    def flagged(call):
+        h.fill_(float("nan"))
+        call()
+        torch.cuda.synchronize()
+        with pytest.raises(rta.RtaError) as e:
+            ctx.check()
+        assert e.value.code == rta.RTA_E_DEVICE and e.value.bits == rta.RTA_DEV_BAD_IMAGE
+        rows = rta.hillas_to_numpy(h.cpu().numpy())
+        assert (rows["flags"] & rta.RTA_HF_BAD_INPUT).all() and (rows["n_pix"] == 0).all()
+
+    for P, S in [(520, S0), (264, 24 if mode == rta.RTA_WINDOW_FIXED else 5)] + ([(264, 128)] if S0 == 9 else []):
+        torch.cuda.synchronize()
+        register(ctx, P, S, array=False)
+        flagged(g.replay)
+        if P > 264:
+            flagged(lambda: ctx.reconstruct(wave, off, tel, evt, *args, h, st))
+    register(ctx, 264, S0, array=False)
+    g.replay()
+    torch.cuda.synchronize()
+    assert ctx.check() == 0
+    assert torch.equal(h.view(torch.int32), first.view(torch.int32))
+    assert torch.equal(st.view(torch.int32), first_st.view(torch.int32))
+    ctx.close()
