@@ -492,7 +492,8 @@ typedef struct rta_segment_t {
  * d_img_tel[i]) and events (d_evt_off: n_evt + 1 image offsets; event number
  * and event time in ns = seconds * 1e9 + floor(fine * 1e9 / 65536)). Nothing is
  * copied: rta_reconstruct_stream reads the samples where they are. Packets are
- * found in parallel: the stream is cut into 1 MiB pieces, each piece looks for
+ * found in parallel: the stream is cut into pieces of 128 KiB to 4 MiB, by its
+ * length and, above 1 MiB, by the packets that seg_cap expects; each looks for
  * its first valid packet (a header whose fixed fields hold and whose successor
  * also starts a valid header) and walks from there; the walks must join up.
  * verify_crc != 0 also checks every packet's CRC (reads every byte once).

@@ -4,10 +4,10 @@
 // the image kernel reads each chunk of pixels from the segment that holds it.
 //
 // Framing: packets follow one another and only a walk from byte 0 knows where
-// they start. The stream is cut into pieces (128 KiB to 1 MiB). Each piece looks
+// they start. The stream is cut into pieces (128 KiB to 4 MiB). Each piece looks
 // for its first valid packet (16-byte aligned positions, a header whose fields
 // hold and whose successor's header holds too; 1,024 positions per round) and walks
-// from there to the end of the piece, keeping the first 32 packets' positions.
+// from there to the end of the piece, keeping the first ING_SLOTS packets' positions.
 // The walks must join up: piece b's first packet
 // is where piece b-1's walk ended. Where they do not (a fault, or a payload that
 // happens to look like a header) a single thread walks on from the last joined
@@ -667,11 +667,15 @@ cudaError_t launch_stream_meta(const ChainArgs& a, StreamImg* out, int64_t max_i
 
 // A piece's walk is serial (about 0.7 us a packet), so short streams are cut into smaller pieces;
 // but every piece reads half a packet on average to find its first one, and all blocks should be
-// resident at once (eight an SM), so pieces grow with the stream, to at most 4 MiB (a 5.1 GB
-// stream without the CRC: 146 us, 187 in pieces of 1 MiB; of 8 MiB the same).
-int64_t ingest_chunk_bytes(int64_t n_bytes, int n_sm) {
+// resident at once (eight an SM), so pieces grow with the stream: to 1 MiB, and to 4 MiB as far as
+// the segment capacity promises at most twice as many packets in one as the piece keeps. 5.2 GB
+// without the CRC in pieces of 1 and of 4 MiB: 200 and 153 us with packets of 51 kB (81 a piece of
+// 4 MiB), 524 and 661 us with 12 kB, 2,016 and 2,988 us with 3 kB.
+int64_t ingest_chunk_bytes(int64_t n_bytes, int64_t seg_cap, int n_sm) {
     int64_t c = int64_t(128) << 10;
-    while (c < (int64_t(4) << 20) && c * n_sm * 8 < n_bytes) c <<= 1;
+    while (c * n_sm * 8 < n_bytes &&
+           (c < (int64_t(1) << 20) || (c < (int64_t(4) << 20) && 2 * c * seg_cap <= 2 * ING_SLOTS * n_bytes)))
+        c <<= 1;
     return c;
 }
 

@@ -1320,7 +1320,7 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
         CUDA_TRY(cudaMemsetAsync(d_evt_off, 0, sizeof(int32_t), s));
         return RTA_OK;
     }
-    const int64_t cb = rta::ingest_chunk_bytes(n_bytes, c->n_sm), nc = (n_bytes + cb - 1) / cb;
+    const int64_t cb = rta::ingest_chunk_bytes(n_bytes, seg_cap, c->n_sm), nc = (n_bytes + cb - 1) / cb;
     const int64_t max_pk = seg_cap + 1;
     const int64_t n_blk = (max_pk + 1023) / 1024;
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };

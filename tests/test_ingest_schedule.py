@@ -50,29 +50,33 @@ extern "C" int frame(const uint8_t* stream, int64_t n_bytes, int64_t chunk_bytes
     }
     return emu::mixed;
 }
+extern "C" int64_t chunk_bytes(int64_t n, int64_t seg_cap, int n_sm) { return rta::ingest_chunk_bytes(n, seg_cap, n_sm); }
 """
 
 
 @pytest.fixture(scope="module")
-def frame(tmp_path_factory):
+def lib(tmp_path_factory):
     text = open(os.path.join(_build.CSRC, "k_ingest.cu")).read()
     cut = text.index("// ---------------------------------------------------------------- per-packet checks")
+    rule = text.index("int64_t ingest_chunk_bytes(")
+    rules = text[rule:text.index("cudaError_t launch_ingest(")]
     d = tmp_path_factory.mktemp("emu")
     src = d / "frame.cpp"
-    src.write_text('#include "emu.h"\n' + text[:cut] + "}  // namespace rta\n" + HARNESS)
-    lib = str(d / "frame.so")
+    src.write_text('#include "emu.h"\n' + text[:cut] + rules + "}  // namespace rta\n" + HARNESS)
+    out = str(d / "frame.so")
     cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
     subprocess.run(["g++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", f"-I{os.path.join(HERE, 'cuda_host')}",
-                    f"-I{_build.INCLUDE}", f"-I{_build.CSRC}", f"-I{cuda}", str(src), "-o", lib], check=True)
-    fn = ctypes.CDLL(lib).frame
+                    f"-I{_build.INCLUDE}", f"-I{_build.CSRC}", f"-I{cuda}", str(src), "-o", out], check=True)
+    lib = ctypes.CDLL(out)
     P, i64, i32 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int
-    fn.argtypes = [P, i64, i64, P, i32, P, i32, i64, P]
-    return fn
+    lib.frame.argtypes = [P, i64, i64, P, i32, P, i32, i64, P]
+    lib.chunk_bytes.argtypes, lib.chunk_bytes.restype = [i64, i64, i32], i64
+    return lib
 
 
 @pytest.mark.parametrize("order", [0, 1, 2, 3])
 @pytest.mark.parametrize("seg,chunk", [(None, 128 << 10), ({1: 40, 2: 48, 3: 64}, 64 << 10)])
-def test_every_order_of_a_blocks_threads_frames_the_stream(frame, seg, chunk, order):
+def test_every_order_of_a_blocks_threads_frames_the_stream(lib, seg, chunk, order):
     wl = synth.make_workload(2, 6)
     buf, plan = synth.encode_stream(wl, seg_pixels=seg)
     buf = np.ascontiguousarray(buf)
@@ -91,8 +95,8 @@ def test_every_order_of_a_blocks_threads_frames_the_stream(frame, seg, chunk, or
     data = data[-data.ctypes.data % 16:][: len(buf)]
     data[:] = buf
     out = np.zeros(2 + 3 * n_chunks, np.int64)
-    mixed = frame(data.ctypes.data, len(buf), chunk, tel_cam.ctypes.data, len(tel_cam), ps.ctypes.data, order,
-                  len(start), out.ctypes.data)
+    mixed = lib.frame(data.ctypes.data, len(buf), chunk, tel_cam.ctypes.data, len(tel_cam), ps.ctypes.data, order,
+                      len(start), out.ctypes.data)
     assert mixed == 0, f"{mixed} barriers reached from two places"
     assert (out[0], out[1]) == (len(start), 0)
     count = np.bincount(start // chunk, minlength=n_chunks)
@@ -100,3 +104,15 @@ def test_every_order_of_a_blocks_threads_frames_the_stream(frame, seg, chunk, or
     np.testing.assert_array_equal(out[4::3], np.cumsum(count) - count)
     first = np.array([start[start >= b * chunk].min() if count[b] else -1 for b in range(n_chunks)])
     np.testing.assert_array_equal(out[2::3][count > 0], first[count > 0])
+
+
+@pytest.mark.parametrize("packet,largest", [(64, 1), (3000, 1), (11600, 1), (26000, 2), (51468, 4), (65536, 4)])
+def test_pieces_of_long_streams_are_bounded_by_the_packets_expected(lib, packet, largest):
+    """Pieces grow with the stream to 1 MiB, and beyond only where the capacity expects few enough
+    packets in one for the single thread that walks them."""
+    for n in np.logspace(5, 10.5, 60).astype(np.int64):
+        c = lib.chunk_bytes(int(n), int(n // packet) + 1, 152)
+        assert 128 << 10 <= c <= largest << 20
+        assert c == 128 << 10 or (c // 2) * 152 * 8 < n             # no larger than the stream asks for
+        assert c >= min(1 << 20, n // (152 * 8) // 2)               # and no more pieces than that up to 1 MiB
+    assert c == largest << 20
