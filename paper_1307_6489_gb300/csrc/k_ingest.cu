@@ -679,6 +679,13 @@ int64_t ingest_chunk_bytes(int64_t n_bytes, int64_t seg_cap, int n_sm) {
     return c;
 }
 
+// The most pieces that a stream of up to n_bytes comes to, whatever its packets: the workspace is
+// sized by it, so that it never grows for a shorter stream (which may come to more pieces).
+int64_t ingest_max_chunks(int64_t n_bytes, int n_sm) {
+    const int64_t kib128 = (n_bytes + (int64_t(128) << 10) - 1) >> 17, mib = (n_bytes + (int64_t(1) << 20) - 1) >> 20;
+    return std::min<int64_t>(kib128, std::max<int64_t>(mib, int64_t(n_sm) * 8));
+}
+
 cudaError_t launch_ingest(const IngestArgs& a, int verify_crc, int n_sm, cudaStream_t s) {
     const int64_t nc = a.n_chunks;
     const int64_t max_pk = a.seg_cap + 1;

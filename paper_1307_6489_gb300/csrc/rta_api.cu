@@ -1321,16 +1321,17 @@ int rta_ingest(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, int verify_
         return RTA_OK;
     }
     const int64_t cb = rta::ingest_chunk_bytes(n_bytes, seg_cap, c->n_sm), nc = (n_bytes + cb - 1) / cb;
+    const int64_t nc_max = rta::ingest_max_chunks(n_bytes, c->n_sm);
     const int64_t max_pk = seg_cap + 1;
     const int64_t n_blk = (max_pk + 1023) / 1024;
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
-    const size_t b_chunks = up(sizeof(rta::IngChunk) * size_t(nc));
+    const size_t b_chunks = up(sizeof(rta::IngChunk) * size_t(nc_max));
     const size_t b_hdr = up(sizeof(rta::IngHdr));
     const size_t b_off = up(sizeof(int64_t) * size_t(max_pk));
     const size_t b_err = up(sizeof(int) * size_t(max_pk));
     const size_t b_scan = up(sizeof(unsigned long long) * size_t(max_pk));
     const size_t b_blk = up(sizeof(unsigned long long) * size_t(n_blk));
-    const size_t b_pos = up(sizeof(long long) * rta::ING_SLOTS * size_t(nc));
+    const size_t b_pos = up(sizeof(long long) * rta::ING_SLOTS * size_t(nc_max));
     const size_t need = b_chunks + b_hdr + b_off + 3 * b_err + b_scan + b_blk + b_pos;
     if (need > c->ingest_bytes) {
         CUDA_TRY(cudaStreamSynchronize(s));

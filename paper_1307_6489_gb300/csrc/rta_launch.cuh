@@ -210,6 +210,7 @@ struct IngestArgs {
     unsigned int* status;
 };
 int64_t ingest_chunk_bytes(int64_t n_bytes, int64_t seg_cap, int n_sm);
+int64_t ingest_max_chunks(int64_t n_bytes, int n_sm);
 cudaError_t launch_ingest(const IngestArgs& a, int verify_crc, int n_sm, cudaStream_t s);
 
 // Lookup-table reconstruction and its training sums (k_lut.cu).

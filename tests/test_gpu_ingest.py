@@ -316,3 +316,35 @@ def test_stream_autotune_keeps_the_rows_and_tunes_only_the_stream_path():
                                 rta.RTA_WINDOW_NEIGHBOUR, start, W, t_hi, t_lo, core_nb, ht.data_ptr(), reps=1)
     assert e.value.code == rta.RTA_E_INVALID
     ctx.close()
+
+
+def test_a_shorter_stream_needs_no_larger_workspace(sset):
+    """After a stream just above the length at which pieces double, one just below it (twice as many
+    pieces) is decoded under capture, where the workspace cannot grow."""
+    wl, ctx0 = sset
+    buf, plan = synth.encode_stream(wl)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    edge = (128 << 10) * 8 * n_sm
+    one = dev_bytes(buf)[: len(buf)]
+    k = edge // len(buf)                       # copies that stay below the edge
+    db = one.repeat(k + 1)
+    assert k >= 1 and db.data_ptr() % 16 == 0 and len(buf) % 16 == 0
+    ctx = make_ctx(wl)                         # a context without a workspace yet
+    d = GpuDir(len(plan["img"]) * (k + 1), wl.n_img * (k + 1), wl.n_evt * (k + 1))
+    assert d.ingest(ctx, db, len(buf) * (k + 1))["error"] == 0
+    n = len(buf) * k
+    want = d.ingest(ctx0, db, n)
+    d.counts.fill_(-7)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        rta.rta_ingest(ctx.handle, db.data_ptr(), n, True, d.seg.data_ptr(), d.seg_cap, d.img_seg.data_ptr(),
+                       d.img_tel.data_ptr(), d.img_cap, d.evt_off.data_ptr(), d.evt_number.data_ptr(),
+                       d.evt_time.data_ptr(), d.evt_cap, d.counts.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    g.replay()
+    torch.cuda.synchronize()
+    assert ctx.check() == 0
+    c = d.counts.cpu().numpy()
+    assert (int(c[0]), int(c[1]), int(c[2]), int(c[4])) == (len(want["seg"]), len(want["img_tel"]),
+                                                            len(want["evt_number"]), 0)
+    ctx.close()

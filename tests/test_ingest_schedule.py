@@ -51,6 +51,7 @@ extern "C" int frame(const uint8_t* stream, int64_t n_bytes, int64_t chunk_bytes
     return emu::mixed;
 }
 extern "C" int64_t chunk_bytes(int64_t n, int64_t seg_cap, int n_sm) { return rta::ingest_chunk_bytes(n, seg_cap, n_sm); }
+extern "C" int64_t max_chunks(int64_t n, int n_sm) { return rta::ingest_max_chunks(n, n_sm); }
 """
 
 
@@ -71,6 +72,7 @@ def lib(tmp_path_factory):
     P, i64, i32 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int
     lib.frame.argtypes = [P, i64, i64, P, i32, P, i32, i64, P]
     lib.chunk_bytes.argtypes, lib.chunk_bytes.restype = [i64, i64, i32], i64
+    lib.max_chunks.argtypes, lib.max_chunks.restype = [i64, i32], i64
     return lib
 
 
@@ -116,3 +118,18 @@ def test_pieces_of_long_streams_are_bounded_by_the_packets_expected(lib, packet,
         assert c == 128 << 10 or (c // 2) * 152 * 8 < n             # no larger than the stream asks for
         assert c >= min(1 << 20, n // (152 * 8) // 2)               # and no more pieces than that up to 1 MiB
     assert c == largest << 20
+
+
+def test_the_workspace_of_a_stream_holds_every_shorter_one(lib):
+    """The pieces that the workspace is sized for cover the stream's, and never fall with its length
+    (pieces of twice the size come to half as many)."""
+    before = 0
+    sizes = {int(x) for x in np.logspace(0, 11, 400)} | {(c * 1216 << 17) + d for c in (1, 2, 4, 8, 16, 32)
+                                                         for d in (-1, 0, 1, 1 << 17)}
+    for n in sorted(sizes):
+        most = lib.max_chunks(n, 152)
+        assert most >= before
+        before = most
+        for seg_cap in (0, 1, n // 60000 + 1, n // 12000 + 1, n // 64 + 1):
+            c = lib.chunk_bytes(n, seg_cap, 152)
+            assert -(-n // c) <= most
