@@ -308,7 +308,8 @@ cudaError_t launch_n(const GemmArgs& g, int n_sm, cudaStream_t s) {
     constexpr size_t smem = tc_smem(KC, N);
     const Tiling w = tile(g, N, KC, 1);
     auto kern = k_gemm_tc<KC, N>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    static std::atomic<uint64_t> opted_in{0};
+    const cudaError_t e = smem_opt_in(kern, opted_in);
     if (e != cudaSuccess) return e;
     // resident CTAs per SM: shared memory and the 512 TMEM columns
     constexpr size_t per_sm = std::max<size_t>(1, std::min<size_t>(size_t(200) * 1024 / smem, 512 / (N < 32 ? 32 : N)));
@@ -320,7 +321,8 @@ template <int KC>
 cudaError_t launch_backward(const GemmArgs& gw, int splits, float* bias, const GemmArgs* gx, int n_sm, cudaStream_t s) {
     const Tiling tw = tile(gw, TC_BN, KC, splits), tx = gx ? tile(*gx, TC_BN, TC_KC, 1) : Tiling{};
     const size_t smem = std::max(std::max(tc_smem(KC, TC_BN), gx ? tc_smem(TC_KC, TC_BN) : 0), size_t(COL_SMEM));
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_backward<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    static std::atomic<uint64_t> opted_in{0};
+    const cudaError_t e = smem_opt_in(k_gemm_backward<KC>, opted_in);
     if (e != cudaSuccess) return e;
     // one CTA per SM: the weight gradient's long items take half of the SMs at most, the bias
     // gradient the SMs its columns need, the input gradient's short items the rest of one wave

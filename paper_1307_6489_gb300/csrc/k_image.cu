@@ -2,7 +2,7 @@
 // launchers of the fused image kernel; the kernels themselves live in
 // k_image_chain.cuh, whose neighbour-peak and byte-stream instantiations are
 // compiled in k_image_nb.cu and k_image_stream.cu.
-#include "k_image_chain.cuh"
+#include "k_image_launch.cuh"
 
 namespace rta {
 
@@ -210,53 +210,22 @@ int chain_chunk_pixels(int v, int stage_wave_bytes, int S) {
     return chunk_pixels(kVariants[v].iw * 32 * kVariants[v].ppt, stage_wave_bytes, S);
 }
 
-template <int IW, int PPT, int MB, int OUT, bool ANY>
-static cudaError_t launch_t(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
-                            int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, false, false, 2, OUT, ANY>;
-    // the dynamic shared-memory opt-in is per device; remember the largest size set
-    static size_t attr_bytes[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || attr_bytes[dev] < smem) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_bytes[dev] = smem;
-    }
-    if (occupancy_only) {
-        *occ = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, chain_block(IW, 1), smem);
-    }
-    kern<<<grid, chain_block(IW, 1), smem, s>>>(a);
-    return cudaGetLastError();
-}
-
-template <int OUT, bool ANY>
-static cudaError_t dispatch(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
-                            int* occ) {
-    switch (v) {
-    case 0: return launch_t<8, 1, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
-    case 1: return launch_t<4, 2, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
-    case 2: return launch_t<8, 2, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
-    case 3: return launch_t<4, 1, 2, OUT, ANY>(a, grid, smem, s, occ_only, occ);
-    case 4: return launch_t<8, 1, 3, OUT, ANY>(a, grid, smem, s, occ_only, occ);   // registers for three CTAs per SM
-    default: return cudaErrorInvalidValue;
-    }
+// The integrate-only call, and rows with masks; the digital filter as the call says.
+template <bool ANY>
+static cudaError_t dispatch_pixels(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
+    return a.integrate_only ? dispatch_chain<false, false, 2, OUT_CHARGES, ANY>(v, a, grid, smem, s)
+                            : dispatch_chain<false, false, 2, OUT_MASKS, ANY>(v, a, grid, smem, s);
 }
 
 cudaError_t launch_image_chain(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
     // the image chain's rows on a contiguous bundle; then byte streams, and the per-pixel outputs
     // (integrate-only charges and times, cleaning masks)
     if (!a.smeta && !a.integrate_only && !a.mask_out)
-        return a.any_window ? dispatch_image_chain_any(v, a, grid, smem, s, false, nullptr)
-                            : dispatch_image_chain_lean(v, a, grid, smem, s, false, nullptr);
+        return a.any_window ? dispatch_image_chain_any(v, a, grid, smem, s)
+                            : dispatch_image_chain_lean(v, a, grid, smem, s);
     if (a.pp.nbpeak) return dispatch_image_chain_nb(v, a, grid, smem, s, false, nullptr);
     if (a.smeta) return dispatch_image_chain_stream(v, a, grid, smem, s, false, nullptr);
-    if (a.integrate_only)
-        return a.any_window ? dispatch<OUT_CHARGES, true>(v, a, grid, smem, s, false, nullptr)
-                            : dispatch<OUT_CHARGES, false>(v, a, grid, smem, s, false, nullptr);
-    return a.any_window ? dispatch<OUT_MASKS, true>(v, a, grid, smem, s, false, nullptr)
-                        : dispatch<OUT_MASKS, false>(v, a, grid, smem, s, false, nullptr);
+    return a.any_window ? dispatch_pixels<true>(v, a, grid, smem, s) : dispatch_pixels<false>(v, a, grid, smem, s);
 }
 
 int chain_occupancy(int v, size_t smem, int kind) {
@@ -264,7 +233,7 @@ int chain_occupancy(int v, size_t smem, int kind) {
     ChainArgs dummy = {};
     const cudaError_t e = kind == CHAIN_NB       ? dispatch_image_chain_nb(v, dummy, 0, smem, nullptr, true, &n)
                           : kind == CHAIN_STREAM ? dispatch_image_chain_stream(v, dummy, 0, smem, nullptr, true, &n)
-                                                 : dispatch<OUT_MASKS, false>(v, dummy, 0, smem, nullptr, true, &n);
+                                                 : dispatch_chain<false, false, 2, OUT_MASKS, false>(v, dummy, 0, smem, nullptr, true, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -280,10 +249,9 @@ cudaError_t launch_clean(const CleanArgs& a, int grid, cudaStream_t s) {
 
 cudaError_t launch_hillas(const HillasArgs& a, int grid, cudaStream_t s) {
     const size_t smem = size_t(a.arr.max_P) * 16 + size_t(4) * ((a.arr.max_P + 31) / 32) + 16;
-    if (smem > size_t(48) * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_hillas, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-    }
+    static std::atomic<uint64_t> opted_in{0};
+    const cudaError_t e = smem_opt_in(k_hillas, opted_in);
+    if (e != cudaSuccess) return e;
     k_hillas<<<grid, UNF_WARPS * 32, smem, s>>>(a);
     return cudaGetLastError();
 }

@@ -1,79 +1,15 @@
 // The image chain on contiguous bundles (as k_image_lean.cu) for launches with a
 // camera whose sample count or window has no specialised search (ANY = true).
-#include <algorithm>
-
-#include "k_image_chain.cuh"
+#include "k_image_launch.cuh"
 
 namespace rta {
 
-constexpr size_t SMEM_PER_SM = size_t(227) * 1024;
-
-// FILTER 1: the form with the digital filter.
-template <int IW, int PPT, int MB, bool NB, int FILTER = 0, int TAILS = 1>
-static cudaError_t launch_any(const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occupancy_only,
-                               int* occ) {
-    auto kern = k_image_chain<IW, PPT, MB, NB, false, FILTER, OUT_ROWS, true, TAILS>;
-    // the dynamic shared-memory opt-in is per device; remember the largest size set
-    static size_t attr_bytes[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || attr_bytes[dev] < smem) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_bytes[dev] = smem;
-    }
-    if (occupancy_only) {
-        *occ = 0;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, chain_block(IW, TAILS), smem);
-    }
-    kern<<<grid, chain_block(IW, TAILS), smem, s>>>(a);
-    return cudaGetLastError();
-}
-
-// The same tile variants as the other window modes (kVariants in k_image.cu).
-cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
-                                      bool occ_only, int* occ) {
+cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
     // variant 4 is variant 0's tile in the 64 registers that let three CTAs share an SM; where
     // shared memory holds fewer, variant 0's registers (90) are there to be used: 1,000 images of
     // 4096 pixels x 128 samples, W = 16, 360 us and 370 in 64; 3,000 of 1600 x 100, W = 6, 267 and 276 (rows split)
-    if (v == 4 && 3 * smem > SMEM_PER_SM && (a.arr.max_P > SMALL_PIX || a.max_S >= 64)) v = 0;
-    if (a.pp.nbpeak) {
-        switch (v) {
-        case 0: return launch_any<8, 1, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_any<4, 2, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_any<8, 2, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_any<4, 1, 2, true>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_any<8, 1, 3, true>(a, grid, smem, s, occ_only, occ);
-        default: return cudaErrorInvalidValue;
-        }
-    }
-    if (a.pp.filter) {
-        switch (v) {
-        case 0: return launch_any<8, 1, 2, false, 1>(a, grid, smem, s, occ_only, occ);
-        case 1: return launch_any<4, 2, 2, false, 1>(a, grid, smem, s, occ_only, occ);
-        case 2: return launch_any<8, 2, 2, false, 1>(a, grid, smem, s, occ_only, occ);
-        case 3: return launch_any<4, 1, 2, false, 1>(a, grid, smem, s, occ_only, occ);
-        case 4: return launch_any<8, 1, 3, false, 1>(a, grid, smem, s, occ_only, occ);
-        default: return cudaErrorInvalidValue;
-        }
-    }
-    // small cameras: variant 4's tile with a tail warp for each of eight slots, two CTAs an SM (an
-    // image of 256 pixels is integrated in a fraction of the time its cleaning and moments take:
-    // 2,000 of them 21.4 us, 35.5 with one tail warp for two slots); with rows of 64 samples and more
-    // the search sets the pace again (303 of 208 x 100: 30.3 us so, 28.9 with three CTAs an SM)
-    if (v == 4 && a.arr.max_P <= SMALL_PIX && a.max_S < 64 && !occ_only) {
-        const size_t sm8 = chain_smem_bytes(4, a.nstage, a.stage_wave_bytes, a.arr.max_P, 0, 0, SMALL_TAILS);
-        const int g8 = int(std::min<int64_t>(a.n_img, 2 * int64_t(a.n_sm)));
-        if (sm8 <= size_t(227) * 1024) return launch_any<8, 1, 2, false, 0, SMALL_TAILS>(a, g8, sm8, s, false, nullptr);
-    }
-    switch (v) {
-    case 0: return launch_any<8, 1, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 1: return launch_any<4, 2, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 2: return launch_any<8, 2, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 3: return launch_any<4, 1, 2, false>(a, grid, smem, s, occ_only, occ);
-    case 4: return launch_any<8, 1, 3, false>(a, grid, smem, s, occ_only, occ);   // registers for three CTAs per SM
-    default: return cudaErrorInvalidValue;
-    }
+    if (v == 4 && 3 * smem > SMEM_PER_CTA && (a.arr.max_P > SMALL_PIX || a.max_S >= 64)) v = 0;
+    return dispatch_rows<true>(v, a, grid, smem, s);
 }
 
 }  // namespace rta

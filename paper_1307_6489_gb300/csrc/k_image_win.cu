@@ -2,16 +2,16 @@
 // samples: the packed searches of 40, 30 and 25 samples (and the 16-sample camera's window of 5)
 // compiled for those widths. The search for any width is slower: 6,000 images of
 // 1855 pixels x 40 samples, W = 8, 410 us, here 168 us.
-#include "k_image_rows.cuh"
+#include "k_image_launch.cuh"
 
 namespace rta {
 
 cudaError_t dispatch_image_chain_win(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
     switch (a.pp.W) {
-    case 4: return dispatch_rows<4>(v, a, grid, smem, s, false, nullptr);
-    case 5: return dispatch_rows<5>(v, a, grid, smem, s, false, nullptr);
-    case 7: return dispatch_rows<7>(v, a, grid, smem, s, false, nullptr);
-    case 8: return dispatch_rows<8>(v, a, grid, smem, s, false, nullptr);
+    case 4: return dispatch_flat_rows<false, 4>(v, a, grid, smem, s);
+    case 5: return dispatch_flat_rows<false, 5>(v, a, grid, smem, s);
+    case 7: return dispatch_flat_rows<false, 7>(v, a, grid, smem, s);
+    case 8: return dispatch_flat_rows<false, 8>(v, a, grid, smem, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -895,7 +895,8 @@ cudaError_t launch_pack_tc(const __nv_bfloat16* pb, __nv_bfloat16* pk, cudaStrea
 
 cudaError_t launch_infer(const InferArgs& a, int n_sm, cudaStream_t s) {
     if (a.f.n_evt <= 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_deepsets_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S_TOTAL));
+    static std::atomic<uint64_t> opted_in{0};
+    const cudaError_t e = smem_opt_in(k_deepsets_infer, opted_in);
     if (e != cudaSuccess) return e;
     // one CTA per SM, with at least 16 events each on average
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_sm, a.f.n_evt / 16));

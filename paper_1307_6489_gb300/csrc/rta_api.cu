@@ -311,7 +311,7 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
         const int full = rta::chain_stage_wave_bytes(cfg.variant, c->max_S);
         for (int k = 8; k > 2; --k) {
             const size_t sm = rta::chain_smem_bytes(cfg.variant, k, full, c->max_P);
-            if (sm > size_t(227) * 1024) continue;
+            if (sm > rta::SMEM_PER_CTA) continue;
             cfg.nstage = k;
             swb = full;
             smem = sm;

@@ -1,6 +1,8 @@
 // Launch-argument blocks of the librta kernels and their host-side launchers.
 #pragma once
 
+#include <atomic>
+
 #include "rta_device.cuh"
 
 namespace rta {
@@ -122,11 +124,9 @@ int chain_occupancy(int v, size_t smem, int kind = CHAIN_PLAIN);
 // and the byte-stream ones (k_image_stream.cu)
 cudaError_t dispatch_image_chain_nb(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
                                     int* occ);
-cudaError_t dispatch_image_chain_lean(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
-                                      bool occ_only, int* occ);
+cudaError_t dispatch_image_chain_lean(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t dispatch_image_chain_win(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
-cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
-                                     bool occ_only, int* occ);
+cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                         bool occ_only, int* occ);
 int chain_variant_min_blocks(int v);
@@ -284,6 +284,27 @@ int serve_infer(rta_model* md, const rta_hillas_t* d_h, const int32_t* d_img_tel
 // telescope registered. RTA_OK or RTA_E_INVALID / RTA_E_ALIGN with the message set.
 int check_bundle_images(rta_ctx* c, const int64_t* h_wave_off, const int32_t* h_img_tel, int64_t n_img,
                         int64_t n_wave);
+// ------------------------------------------------------------------ launches
+constexpr size_t SMEM_PER_CTA = size_t(227) * 1024;     // the most a CTA can have, and an SM's CTAs together
+
+// Opts a kernel in to the most dynamic shared memory, once on each device. The limit is the same
+// for every launch: one sized for a launch of its own could be lowered by another thread before
+// that launch.
+template <class K>
+cudaError_t smem_opt_in(K* kern, std::atomic<uint64_t>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = uint64_t(1) << (dev & 63);
+    if (dev < 64 && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(SMEM_PER_CTA - fa.sharedSizeBytes));
+    if (e == cudaSuccess && dev < 64) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
 // The kernels of a training step, and those of an ingest, are launched as programmatic dependents
 // of one another: each signals at once, and waits (grid_dependency_wait) before it reads anything.
 template <class... P, class... A>

@@ -475,3 +475,61 @@ def test_bounded_device_wait_times_out_and_the_context_survives(arr):
     ctx.image_chain(dev.wave, dev.wave_off, dev.img_tel, mode, start, W, t_hi, t_lo, core_nb, out)
     assert ctx.check() == 0
     assert (hillas_rows(out, wl.n_img)["n_pix"] > 0).any()
+
+
+def test_threads_with_cameras_of_different_sizes_do_not_disturb_each_other():
+    """Two threads, each with a context, a stream and a camera size of its own, launch the stage kernels
+    and the image chain side by side: no launch loses its shared memory to the other's, and every
+    row is the one of the thread alone."""
+    import threading
+
+    rng = np.random.default_rng(11)
+    jobs = []
+    for kind, P, S in (("square", 4096, 16), ("hex", 3504, 24)):
+        n_img, W = 3, 5
+        xy, nb = synth.lattice(kind, P, 0.1)
+        ctx = rta.Context(0)
+        ctx.register_camera(5, xy, nb, S)
+        ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                           np.full(P, 1 / 128, np.float32))
+        wave = torch.from_numpy(rng.integers(380, 480, n_img * P * S).astype(np.int16)).cuda()
+        off = torch.arange(n_img, device="cuda") * (P * S)
+        pix = torch.arange(n_img, device="cuda") * P
+        tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+        q, t = torch.zeros(n_img * P, device="cuda"), torch.zeros(n_img * P, device="cuda")
+        mask = torch.zeros(n_img * P, dtype=torch.uint8, device="cuda")
+        h, hc = torch.zeros(n_img * 16, device="cuda"), torch.zeros(n_img * 16, device="cuda")
+        stream = torch.cuda.Stream()
+
+        def work(ctx=ctx, a=(wave, off, tel, pix, q, t, mask, h, hc), s=stream.cuda_stream, W=W, keep=stream):
+            wave, off, tel, pix, q, t, mask, h, hc = a
+            ctx.calibrate_integrate(wave, off, tel, pix, rta.RTA_WINDOW_SLIDING, 0, W, q, t, stream=s)
+            ctx.clean(q, tel, pix, 3.0, 1.5, 1, mask, stream=s)
+            ctx.hillas(q, t, mask, tel, pix, h, stream=s)
+            ctx.image_chain(wave, off, tel, rta.RTA_WINDOW_SLIDING, 0, W, 3.0, 1.5, 1, hc, stream=s)
+            keep.synchronize()
+            return h.cpu(), hc.cpu()
+
+        torch.cuda.synchronize()
+        jobs.append((ctx, work, work()))
+    failed = []
+
+    def loop(work, want):
+        try:
+            for _ in range(300):
+                got = work()
+                if not all(torch.equal(g.view(torch.int32), w.view(torch.int32)) for g, w in zip(got, want)):
+                    failed.append("rows differ")
+                    return
+        except rta.RtaError as e:
+            failed.append(str(e))
+
+    threads = [threading.Thread(target=loop, args=(work, want)) for _, work, want in jobs]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed
+    for ctx, _, want in jobs:
+        assert ctx.check() == 0 and int(want[0].view(torch.int32).view(-1, 16)[:, 10].min()) > 0
+        ctx.close()
