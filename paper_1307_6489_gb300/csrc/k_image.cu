@@ -211,21 +211,22 @@ int chain_chunk_pixels(int v, int stage_wave_bytes, int S) {
 }
 
 // The integrate-only call, and rows with masks; the digital filter as the call says.
-template <bool ANY>
+template <int SEARCH>
 static cudaError_t dispatch_pixels(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
-    return a.integrate_only ? dispatch_chain<false, false, 2, OUT_CHARGES, ANY>(v, a, grid, smem, s)
-                            : dispatch_chain<false, false, 2, OUT_MASKS, ANY>(v, a, grid, smem, s);
+    return a.integrate_only ? dispatch_chain<false, false, 2, OUT_CHARGES, SEARCH>(v, a, grid, smem, s)
+                            : dispatch_chain<false, false, 2, OUT_MASKS, SEARCH>(v, a, grid, smem, s);
 }
 
 cudaError_t launch_image_chain(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
     // the image chain's rows on a contiguous bundle; then byte streams, and the per-pixel outputs
     // (integrate-only charges and times, cleaning masks)
     if (!a.smeta && !a.integrate_only && !a.mask_out)
-        return a.any_window ? dispatch_image_chain_any(v, a, grid, smem, s)
-                            : dispatch_image_chain_lean(v, a, grid, smem, s);
+        return a.search == SEARCH_PACKED   ? dispatch_image_chain_any(v, a, grid, smem, s)
+               : a.search == SEARCH_SERIAL ? dispatch_image_chain_serial(v, a, grid, smem, s)
+                                           : dispatch_image_chain_lean(v, a, grid, smem, s);
     if (a.pp.nbpeak) return dispatch_image_chain_nb(v, a, grid, smem, s, false, nullptr);
     if (a.smeta) return dispatch_image_chain_stream(v, a, grid, smem, s, false, nullptr);
-    return a.any_window ? dispatch_pixels<true>(v, a, grid, smem, s) : dispatch_pixels<false>(v, a, grid, smem, s);
+    return a.search == SEARCH_PACKED ? dispatch_pixels<SEARCH_PACKED>(v, a, grid, smem, s) : dispatch_pixels<SEARCH_SERIAL>(v, a, grid, smem, s);
 }
 
 int chain_occupancy(int v, size_t smem, int kind) {
@@ -233,7 +234,7 @@ int chain_occupancy(int v, size_t smem, int kind) {
     ChainArgs dummy = {};
     const cudaError_t e = kind == CHAIN_NB       ? dispatch_image_chain_nb(v, dummy, 0, smem, nullptr, true, &n)
                           : kind == CHAIN_STREAM ? dispatch_image_chain_stream(v, dummy, 0, smem, nullptr, true, &n)
-                                                 : dispatch_chain<false, false, 2, OUT_MASKS, false>(v, dummy, 0, smem, nullptr, true, &n);
+                                                 : dispatch_chain<false, false, 2, OUT_MASKS, SEARCH_SERIAL>(v, dummy, 0, smem, nullptr, true, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;

@@ -252,8 +252,8 @@ __device__ __forceinline__ uint32_t spread_even(uint32_t v) {
     return v;
 }
 
-// The search for any sample count and any window of up to 16 samples (the cameras and windows
-// without a specialised one), eight words of a row at a time. As in max_window_packed, samples
+// The search for any sample count and any window of up to 16 samples (of the cameras and windows
+// without a specialised one, those that window_search names), eight words of a row at a time. As in max_window_packed, samples
 // must be below 4096 (checked: sums of 16 stay below 2^16, so plain 32-bit adds carry nothing
 // from one half of a word into the other), and rows that start on an odd 16-bit position are
 // read from the word below.
@@ -390,11 +390,11 @@ __device__ __forceinline__ int best_key_generic(const uint16_t* row, int S, int 
 // (shared memory), for the cameras without a specialised search. A search is part of every
 // kernel: a caller's own capture of a launch stays with the kernel it was captured with when
 // a camera is registered again with a sample count that has no compiled search there.
-template <bool ANY>
+template <int SEARCH>
 __device__ __forceinline__ void window_sum(const uint16_t* row, int S, const ProcParams& pp, int& sum, int& st) {
     const int W = pp.W;
     if (pp.sliding) {
-        const int key = ANY ? best_key_serial(row, S, W) : best_key_rolled(row, S, W);
+        const int key = SEARCH == SEARCH_OWN ? best_key_rolled(row, S, W) : best_key_serial(row, S, W);
         sum = key >> 7;
         st = 127 - (key & 127);
     } else {
@@ -738,8 +738,8 @@ struct NbShared {
     int* n_cand;          // candidates so far in this image
 };
 
-// ANY: the generic path (S == 0) has the packed search for any window, else the rolled one.
-template <int S, int W, int IT, int PPT, bool INTEG, bool ANY = false>
+// SEARCH: what the generic path (S == 0) searches with.
+template <int S, int W, int IT, int PPT, bool INTEG, int SEARCH = SEARCH_OWN>
 __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
                                               const unsigned char* buf, const int32_t* cp16, const float* cscale,
                                               const NbShared& nb, const SlotView& v, int ct, int lane) {
@@ -768,7 +768,8 @@ __device__ __forceinline__ void nb_keys_chunk(const ChainArgs& a, const ProcPara
                 int key;
                 if constexpr (S != 0 && !INTEG && W == 6) key = best_key_serial(row, S, W);
                 else if constexpr (S != 0) key = best_key_T<S, W>(row, pp.one, pp.k128);
-                else if constexpr (ANY) key = best_key_generic(row, Sr, Wr);
+                else if constexpr (SEARCH == SEARCH_PACKED) key = best_key_generic(row, Sr, Wr);
+                else if constexpr (SEARCH == SEARCH_SERIAL) key = best_key_serial(row, Sr, Wr);
                 else key = best_key_rolled(row, Sr, Wr);
                 q0 = charge(key >> 7, Wr, cp16[c], cscale[c], num);
                 st = 127 - (key & 127);
@@ -846,10 +847,9 @@ __device__ __forceinline__ void nb_pixel(const ChainArgs& a, const ProcParams& p
 // compile-time for the specialised sliding-window cameras (the camera is the
 // same for the whole chunk, so the dispatch happens once per chunk); S == 0 is
 // the generic path with run-time S and W.
-// ANY: the generic path (S == 0) has the packed search for any sliding window; without it the
-// fixed window and the rolled search. SKEW: chunks of skewed_rows cameras are laid out in SKEW_BLOCKS runs, and
+// SEARCH: what the generic path (S == 0) searches sliding windows with. SKEW: chunks of skewed_rows cameras are laid out in SKEW_BLOCKS runs, and
 // split_rows cameras take two threads a pixel.
-template <int S, int W, int IT, int PPT, bool INTEG, int FILTER, bool ANY = false, bool SKEW = false>
+template <int S, int W, int IT, int PPT, bool INTEG, int FILTER, int SEARCH = SEARCH_OWN, bool SKEW = false>
 __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcParams& pp, const StageHdr& h,
                                                 const unsigned char* buf, const int32_t* cp16, const float* cscale,
                                                 const SlotView& v, int ct, int lane, const int* wts) {
@@ -956,7 +956,7 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                     wst = 127 - (key & 127);
                 } else {
                     bool found = false;
-                    if (ANY && pp.sliding) {
+                    if (SEARCH == SEARCH_PACKED && pp.sliding) {
                         // as above: below t_lo the maximum alone is the pixel's result
                         const PackedRow pr(row, h.S, Wr);
                         int b0 = 0, b1 = pr.blocks(), blk;
@@ -989,7 +989,7 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                             if (!done) wst = pr.start_in(blk, sum);
                         }
                     }
-                    if (!done && !found) window_sum<ANY>(row, h.S, pp, sum, wst);
+                    if (!done && !found) window_sum<SEARCH>(row, h.S, pp, sum, wst);
                 }
                 if (!done) emit(c, sum, wst, row, hi, lo);
             }
@@ -1057,23 +1057,23 @@ static __device__ __forceinline__ int stream_chunk_copy(const ChainArgs& a, cons
 // combination is a separate instantiation, so that every kernel carries only the
 // code of the calls it serves (branches left in, even untaken, cost the hot loop
 // instruction-cache misses and scheduling).
-// ANY: the packed search that takes any sample count and window width; without it the kernel has
-// the specialised ones and the fixed window, for launches all of whose cameras have one (its code and
-// registers, left in, cost those launches 11 % on the 10,000-event bundle, 926 against 834 us),
-// and a rolled serial search for a camera that gets another sample count after a capture (0.7 % of
+// SEARCH: beside the specialised searches and the fixed window, SEARCH_PACKED carries the packed
+// search (its code and registers, left in, cost launches that do not need it 11 % on the 10,000-event
+// bundle, 926 against 834 us), SEARCH_SERIAL the serial one, and SEARCH_OWN a rolled one for a
+// camera that gets another sample count after a capture (0.7 % of
 // 2,000 events with the neighbour-peak window, 1 % of 2,000 images of 256 pixels, else nothing).
 // OUT: what a launch writes -- Hillas rows, charges and times only (the integrate-only call), or
 // rows and cleaning masks.
 enum { OUT_ROWS = 0, OUT_CHARGES = 1, OUT_MASKS = 2 };
 // WIN: the width of the sliding window that has specialised searches for 40, 30 and 25 samples (a
 // launch has one width; the kernels of 4, 5, 7 and 8 samples serve flat windows, rows only).
-template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, bool ANY, int TAILS = 1, int WIN = 6>
+template <int IW, int PPT, int MB, bool NB, bool STREAM, int FILTER, int OUT, int SEARCH, int TAILS = 1, int WIN = 6>
 __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(const ChainArgs a) {
     // flat windows of 6 for the rows alone: the 16-sample camera's window of 5 is the WIN = 5 kernel's
-    constexpr bool ROWS6 = WIN == 6 && OUT == OUT_ROWS && FILTER == 0 && !STREAM && !ANY;
+    constexpr bool ROWS6 = WIN == 6 && OUT == OUT_ROWS && FILTER == 0 && !STREAM && SEARCH == SEARCH_OWN;
     static_assert(!(NB && FILTER) && !(STREAM && OUT != OUT_ROWS), "the calls there are");
     constexpr bool integ = OUT == OUT_CHARGES;
-    constexpr bool SKEW = ANY && !NB && !STREAM;
+    constexpr bool SKEW = SEARCH == SEARCH_PACKED && !NB && !STREAM;
     constexpr int IT = IW * 32;          // integrator threads
     constexpr int CHUNK = IT * PPT;      // largest chunk in pixels
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1396,7 +1396,7 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
             else if (pp.W == 6 && h.S == 25)
                 nb_keys_chunk<25, 6, IT, PPT, integ>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             else
-                nb_keys_chunk<0, 0, IT, PPT, integ, ANY>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
+                nb_keys_chunk<0, 0, IT, PPT, integ, SEARCH>(a, pp, h, buf, cp16, cscale, nb, v, ct, lane);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
             if (++stage == NST) { stage = 0; phase ^= 1u; }
@@ -1428,7 +1428,7 @@ __global__ void __launch_bounds__(chain_block(IW, TAILS), MB) k_image_chain(cons
             else if ((WIN == 5 || !ROWS6) && pp.sliding && pp.W == 5 && h.S == 16)
                 integrate_chunk<16, 5, IT, PPT, integ, FILTER>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             else
-                integrate_chunk<0, 0, IT, PPT, integ, FILTER, ANY, SKEW>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
+                integrate_chunk<0, 0, IT, PPT, integ, FILTER, SEARCH, SKEW>(a, pp, h, buf, cp16, cscale, v, ct, lane, sm.wts);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.empty[stage]);
             if (++stage == NST) { stage = 0; phase ^= 1u; }

@@ -5,18 +5,18 @@
 
 namespace rta {
 
-template <bool ANY>
+template <int SEARCH>
 static cudaError_t dispatch_nb(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
                                int* occ) {
-    if (a.smeta) return dispatch_chain<true, true, 0, OUT_ROWS, ANY>(v, a, grid, smem, s, occ_only, occ);
-    if (a.integrate_only) return dispatch_chain<true, false, 0, OUT_CHARGES, ANY>(v, a, grid, smem, s, occ_only, occ);
-    return dispatch_chain<true, false, 0, OUT_MASKS, ANY>(v, a, grid, smem, s, occ_only, occ);
+    if (a.smeta) return dispatch_chain<true, true, 0, OUT_ROWS, SEARCH>(v, a, grid, smem, s, occ_only, occ);
+    if (a.integrate_only) return dispatch_chain<true, false, 0, OUT_CHARGES, SEARCH>(v, a, grid, smem, s, occ_only, occ);
+    return dispatch_chain<true, false, 0, OUT_MASKS, SEARCH>(v, a, grid, smem, s, occ_only, occ);
 }
 
 cudaError_t dispatch_image_chain_nb(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
                                     int* occ) {
-    return a.any_window ? dispatch_nb<true>(v, a, grid, smem, s, occ_only, occ)
-                        : dispatch_nb<false>(v, a, grid, smem, s, occ_only, occ);
+    return a.search == SEARCH_PACKED ? dispatch_nb<SEARCH_PACKED>(v, a, grid, smem, s, occ_only, occ)
+                        : dispatch_nb<SEARCH_SERIAL>(v, a, grid, smem, s, occ_only, occ);
 }
 
 }  // namespace rta

@@ -5,17 +5,17 @@
 
 namespace rta {
 
-template <bool ANY>
+template <int SEARCH>
 static cudaError_t dispatch_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s, bool occ_only,
                                    int* occ) {
-    return a.pp.filter || occ_only ? dispatch_chain<false, true, 1, OUT_ROWS, ANY>(v, a, grid, smem, s, occ_only, occ)
-                                   : dispatch_chain<false, true, 0, OUT_ROWS, ANY>(v, a, grid, smem, s, occ_only, occ);
+    return a.pp.filter || occ_only ? dispatch_chain<false, true, 1, OUT_ROWS, SEARCH>(v, a, grid, smem, s, occ_only, occ)
+                                   : dispatch_chain<false, true, 0, OUT_ROWS, SEARCH>(v, a, grid, smem, s, occ_only, occ);
 }
 
 cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                         bool occ_only, int* occ) {
-    return a.any_window ? dispatch_stream<true>(v, a, grid, smem, s, occ_only, occ)
-                        : dispatch_stream<false>(v, a, grid, smem, s, occ_only, occ);
+    return a.search == SEARCH_PACKED ? dispatch_stream<SEARCH_PACKED>(v, a, grid, smem, s, occ_only, occ)
+                        : dispatch_stream<SEARCH_SERIAL>(v, a, grid, smem, s, occ_only, occ);
 }
 
 }  // namespace rta

@@ -8,10 +8,10 @@ namespace rta {
 
 cudaError_t dispatch_image_chain_win(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
     switch (a.pp.W) {
-    case 4: return dispatch_flat_rows<false, 4>(v, a, grid, smem, s);
-    case 5: return dispatch_flat_rows<false, 5>(v, a, grid, smem, s);
-    case 7: return dispatch_flat_rows<false, 7>(v, a, grid, smem, s);
-    case 8: return dispatch_flat_rows<false, 8>(v, a, grid, smem, s);
+    case 4: return dispatch_flat_rows<SEARCH_OWN, 4>(v, a, grid, smem, s);
+    case 5: return dispatch_flat_rows<SEARCH_OWN, 5>(v, a, grid, smem, s);
+    case 7: return dispatch_flat_rows<SEARCH_OWN, 7>(v, a, grid, smem, s);
+    case 8: return dispatch_flat_rows<SEARCH_OWN, 8>(v, a, grid, smem, s);
     default: return cudaErrorInvalidValue;
     }
 }

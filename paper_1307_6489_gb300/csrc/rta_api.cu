@@ -286,10 +286,11 @@ int chain_launch_config(rta_ctx* c, int64_t n_img, int* grid, size_t* smem, int*
     return config_launch(c, cfg_of(c, kind), n_img, grid, smem, swb, kind);
 }
 
-int needs_any_window(const rta_ctx* c, const rta::ProcParams& pp, bool rows) {
+int launch_search(const rta_ctx* c, const rta::ProcParams& pp, bool rows) {
+    int search = rta::SEARCH_OWN;
     for (int t = 0; t < c->n_tel; ++t)
-        if (!rta::window_specialised(pp, c->cams[c->tel_cam[t]].S, rows)) return 1;
-    return 0;
+        search = rta::search_of_both(search, rta::window_search(pp, c->cams[c->tel_cam[t]].S, rows));
+    return search;
 }
 
 int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t* d_wave_off, const int32_t* d_img_tel,
@@ -339,7 +340,7 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
     a.max_S = c->max_S;
     a.nstage = std::max(2, std::min(cfg.nstage, 8));
     a.integrate_only = integrate_only;
-    a.any_window = needs_any_window(c, pp, !integrate_only && !d_mask && !d_smeta);
+    a.search = launch_search(c, pp, !integrate_only && !d_mask && !d_smeta);
     a.n_sm = c->n_sm;
     a.n_img_dev = d_n_img;
     a.seg = d_seg;

@@ -30,7 +30,7 @@ struct ChainArgs {
     int max_S;               // longest rows of the array's cameras
     int integrate_only;
     int n_sm;                // of the device
-    int any_window;          // some camera has no specialised window search (window_specialised)
+    int search;              // SEARCH_*: what some camera without a specialised window search needs
     // a byte-stream bundle (rta_ingest's directory): wave is the stream, wave_off unused;
     // smeta: one prepared record per image (k_stream_meta)
     const rta_segment_t* seg;
@@ -39,17 +39,37 @@ struct ChainArgs {
     const struct StreamImg* smeta;
 };
 
-// Whether launches with S samples and windows of W run the instantiations that carry a search
-// compiled for them, and no other (all cameras of a launch have to). rows: flat windows of a
-// contiguous bundle, rows only. A fixed window needs no search, but rows of a multiple of 32
-// samples put a warp's 16-bit loads on two banks or one, and the kernels for any window lay such
-// chunks out in padded runs: 1,000 images of 4096 pixels x 128 samples, W = 16, 247 us, 329 with
-// plain rows; 10,000 of 1000 x 32, W = 8, 185 us, 249. On four banks the plain rows are faster
-// (5,000 of 2000 x 48, W = 3: 154 us, 175 with padded runs).
-inline bool window_specialised(const ProcParams& pp, int S, bool rows) {
-    if (!pp.sliding) return !(rows && !pp.filter && S % 32 == 0);
+// The search for windows of W in a camera of S samples: SEARCH_OWN, a kernel that has one compiled
+// for them; SEARCH_SERIAL, two 16-bit loads per window start; SEARCH_PACKED (PackedRow), which
+// works on 16 samples at a time and can lay chunks out in padded runs. rows: flat windows of a
+// contiguous bundle, rows only.
+//
+// The serial search is bound by its shared loads, and those by the banks that a warp's rows share:
+// two rows a bank when S % 8 is 2, 4 or 6, four when it is 0 and S / 8 is odd, else more. With one
+// or two it is the faster one, for every output: on 0.2 GB of 1000-pixel images, W = 4, packed and
+// serial 1.41 times apart at 20 samples, 1.27 at 31, 1.18 at 50, 1.13 at 60, 1.20 at 100, 1.11 at
+// 127 (charges alone 1.8 to 1.13); with four, 1.05 at 24 samples (with the filter 0.94), 0.83 at 56
+// and 0.73 at 104; with more, 0.85 at 16, 0.51 at 48, 0.12 at 128. Windows of one sample are
+// cheaper packed in long rows (0.91 at 65 and 100 samples).
+//
+// A fixed window needs no search, but rows of a multiple of 32 samples put a warp's loads on two
+// banks or one, and the packed kernels' padded runs spread them: 8 samples of 1000 pixels x 32
+// 0.79 of the time, x 64 0.73, x 128 0.83. For up to three samples the runs' copies cost more than
+// they save (1.12, 1.20 and 1.01 for one sample). On four banks plain rows are faster
+// (5,000 of 2000 x 48, W = 3: 154 us, 175 in padded runs).
+enum { SEARCH_OWN = 0, SEARCH_PACKED = 1, SEARCH_SERIAL = 2 };
+inline int window_search(const ProcParams& pp, int S, bool rows) {
+    if (!pp.sliding) return rows && !pp.filter && S % 32 == 0 && pp.W > 3 ? SEARCH_PACKED : SEARCH_OWN;
     const bool width = pp.W == 6 || (rows && !pp.nbpeak && !pp.filter && pp.W >= 4 && pp.W <= 8);
-    return (width && (S == 40 || S == 30 || S == 25)) || (pp.W == 5 && S == 16 && !pp.nbpeak);
+    if ((width && (S == 40 || S == 30 || S == 25)) || (pp.W == 5 && S == 16 && !pp.nbpeak)) return SEARCH_OWN;
+    if (pp.W == 1 && S >= 64) return SEARCH_PACKED;
+    return S % 8 != 0 || (S % 16 == 8 && S <= 24 && !pp.filter) ? SEARCH_SERIAL : SEARCH_PACKED;
+}
+
+// The search of a launch with cameras of both: the serial search loses far more on the other's rows
+// than the packed one on its own.
+inline int search_of_both(int a, int b) {
+    return a == SEARCH_PACKED || b == SEARCH_PACKED ? SEARCH_PACKED : a > b ? a : b;
 }
 
 // One image of a byte stream as the image kernel's producer needs it: checked
@@ -126,6 +146,7 @@ cudaError_t dispatch_image_chain_nb(int v, const ChainArgs& a, int grid, size_t 
                                     int* occ);
 cudaError_t dispatch_image_chain_lean(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t dispatch_image_chain_win(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
+cudaError_t dispatch_image_chain_serial(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t dispatch_image_chain_any(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s);
 cudaError_t dispatch_image_chain_stream(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s,
                                         bool occ_only, int* occ);

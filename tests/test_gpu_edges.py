@@ -234,6 +234,64 @@ def test_any_camera_and_window(kind, P, S, W):
     ctx.close()
 
 
+@pytest.mark.parametrize("S,W", [(9, 9), (17, 16), (20, 3), (25, 12), (30, 3), (31, 8), (50, 2), (63, 9), (65, 6),
+                                 (100, 12), (127, 16), (40, 6), (104, 4)])
+@pytest.mark.parametrize("mode", [rta.RTA_WINDOW_SLIDING, rta.RTA_WINDOW_FILTER, rta.RTA_WINDOW_NEIGHBOUR])
+def test_rows_do_not_depend_on_the_search_that_the_array_takes(mode, S, W):
+    """A camera alone in its array, and beside another whose rows share banks (48 samples: the packed
+    search for the whole launch): the same rows, masks, charges and times bit for bit, for rows of
+    every alignment and several images per block, samples up to full scale among them."""
+    P, P2, S2, n_img = 264, 72, 48, 700
+    if (P * S) % 8:
+        P += 8 - P % 8
+    rng = np.random.default_rng(31 * S + W)
+    cams = [synth.lattice("hex", P, 0.1), synth.lattice("hex", P2, 0.1)]
+    wave = rng.integers(380, 430, (40, P, S)).astype(np.uint16)
+    for i in range(40):
+        d = ((cams[0][0] - cams[0][0][rng.integers(P)]) ** 2).sum(1)
+        k0 = rng.integers(0, S)
+        wave[i, :, k0] += (200 * (1 + i % 5) * np.exp(-d / 0.03)).astype(np.uint16)
+    wave[3, P // 2] = 65535
+    wave[5, 7, S // 2:] = 4096
+    wave[6] = 400
+    wave2 = rng.integers(380, 430, (40, P2, S2)).astype(np.uint16)
+    wave2[:, :9, 20] += 700
+    flat = torch.from_numpy(np.concatenate([wave.reshape(-1), wave2.reshape(-1)]).view(np.int16)).cuda()
+    kind = np.arange(n_img) % 3 == 2                      # the other camera's images in between
+    at = np.where(kind, 40 * P * S + np.arange(n_img) % 40 * (P2 * S2), np.arange(n_img) % 40 * (P * S))
+    pixels = np.where(kind, P2, P)
+    first = np.cumsum(pixels) - pixels
+    got = []
+    for both in (False, True):
+        ctx = rta.Context(0)
+        for c, (xy, nb) in enumerate(cams):
+            ctx.register_camera(c, xy, nb, (S, S2)[c])
+        n_tel = 2 if both else 1
+        ctx.register_array(np.arange(n_tel, dtype=np.int32), np.zeros((n_tel, 2), np.float32),
+                           np.full(P + both * P2, 6400, np.int32), np.full(P + both * P2, 1 / 128, np.float32))
+        if mode == rta.RTA_WINDOW_FILTER:
+            rta.rta_set_filter_weights(ctx.handle, [1 + k % 4 for k in range(W)])
+        use = np.arange(n_img) if both else np.flatnonzero(~kind)
+        off, pix = (torch.from_numpy(np.ascontiguousarray(a[use]).astype(np.int64)).cuda() for a in (at, first))
+        tel = torch.from_numpy(kind[use].astype(np.int32)).cuda()
+        q = torch.full((int(pixels.sum()),), float("nan"), device="cuda")
+        t, mask = torch.full_like(q, float("nan")), torch.full(q.shape, 7, dtype=torch.uint8, device="cuda")
+        h, hm = torch.zeros(len(use) * 16, device="cuda"), torch.zeros(len(use) * 16, device="cuda")
+        ctx.calibrate_integrate(flat, off, tel, pix, mode, 0, W, q, t)
+        ctx.image_chain(flat, off, tel, mode, 0, W, 4.0, 2.0, 1, h)
+        ctx.image_chain_masks(flat, off, tel, pix, mode, 0, W, 4.0, 2.0, 1, mask, hm)
+        assert ctx.check() == 0
+        ctx.close()
+        h, hm = h.cpu().numpy().view(np.uint32).reshape(-1, 16), hm.cpu().numpy().view(np.uint32).reshape(-1, 16)
+        np.testing.assert_array_equal(h, hm)
+        mine = np.repeat(~kind, pixels)
+        got.append((h[~kind[use]], q.cpu().numpy().view(np.uint32)[mine], t.cpu().numpy().view(np.uint32)[mine],
+                    mask.cpu().numpy()[mine]))
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
+    assert (got[0][0][:, 10] > 0).mean() > 0.3
+
+
 @pytest.mark.parametrize("kind,P,S,start,W", [
     ("hex", 331, 32, 20, 12), ("square", 1030, 32, 0, 1), ("hex", 1000, 64, 17, 16), ("square", 257, 96, 95, 1),
     ("square", 2049, 128, 112, 16), ("hex", 130, 128, 0, 7), ("square", 1600, 100, 9, 6), ("hex", 1000, 48, 40, 8)])
