@@ -9,42 +9,24 @@ namespace rta {
 // ------------------------------------------------------------------ unfused stage kernels
 
 // One block per image, a warp per 32-pixel word and a lane per pixel. What an image's pixels need
-// from memory -- values straight into ballots, then the neighbours, or the charges, times and
-// positions, of the pixels that count -- is loaded side by side, one latency for all of them (a
-// thread per bitmap word met one per set bit). 501 events, 2,320 images: k_hillas 38 -> 26 us,
-// k_clean 20.5 -> 22 alone but the two, back to back with the integration, 116 -> 108.
-constexpr int UNF_WARPS = 8;
-constexpr int UNF_WORDS = 8;      // words a warp takes at a time
-constexpr int UNF_STEP = UNF_WARPS * UNF_WORDS;
+// from memory -- values straight into ballots, or the charges, times and positions of the pixels
+// that count -- is loaded side by side, one latency for all of them (a thread per bitmap word met
+// one per set bit). Both kernels are bound by such chains (telescope, camera, pixels, barriers), so
+// their time is that of an image times the rounds that the resident blocks make.
 
-// w0[w] = {v >= t0}, w1[w] = {v >= t1} of the image's values q (global memory).
-__device__ __forceinline__ void threshold_words(const float* q, int P, float t0, float t1, uint32_t* w0, uint32_t* w1) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = words_of(P);
-    for (int wb = 0; wb < nw; wb += UNF_STEP) {
-        float v[UNF_WORDS];
-#pragma unroll
-        for (int k = 0; k < UNF_WORDS; ++k) {
-            const int p = 32 * (wb + warp + UNF_WARPS * k) + lane;
-            v[k] = p < P ? __ldg(q + p) : __int_as_float(0x7fc00000);      // NaN: neither
-        }
-#pragma unroll
-        for (int k = 0; k < UNF_WORDS; ++k) {
-            const int w = wb + warp + UNF_WARPS * k;
-            if (w >= nw) break;
-            const uint32_t b0 = __ballot_sync(0xffffffffu, v[k] >= t0);
-            const uint32_t b1 = __ballot_sync(0xffffffffu, v[k] >= t1);
-            if (lane == 0) {
-                w0[w] = b0;
-                w1[w] = b1;
-            }
-        }
-    }
-}
+// k_clean: a warp takes the same words of an image in every pass and holds its lanes' bits of them, so only what neighbours ask for, the hi and the core bits, is shared: two barriers an
+// image, and the next image's hi bits may be written while this one's core bits are still read.
+// The neighbours' lists are loaded for the words that have such pixels alone, one after another:
+// held for all of a warp's words they took the registers of half the resident blocks. 500, 4,224 and
+// 28,160 images of the three presets 9.0, 27.1 and 142 us; 8.4, 35.6 and 220 with the lists
+// held, 10.5, 27.5 and 187 with a thread per bitmap word.
+constexpr int CLEAN_WARPS = 8;
+constexpr int CLEAN_WORDS = RTA_MAX_PIX / 32 / CLEAN_WARPS;      // words a warp has at most
+static_assert(CLEAN_WORDS <= 32, "a bit per word");
 
-__global__ void __launch_bounds__(UNF_WARPS * 32) k_clean(const CleanArgs a) {
+__global__ void __launch_bounds__(CLEAN_WARPS * 32, 8) k_clean(const CleanArgs a) {
     extern __shared__ __align__(16) uint32_t words[];
-    const int maxw = words_of(a.arr.max_P);
-    uint32_t *hi = words, *lo = hi + maxw, *core = lo + maxw, *mask = core + maxw;
+    uint32_t *hi = words, *core = words + words_of(a.arr.max_P);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t img = blockIdx.x; img < a.n_img; img += gridDim.x) {
         const int tel = a.img_tel[img];
@@ -58,60 +40,64 @@ __global__ void __launch_bounds__(UNF_WARPS * 32) k_clean(const CleanArgs a) {
             if (threadIdx.x == 0) atomicOr(a.status, RTA_DEV_BAD_IMAGE);
             continue;
         }
-        threshold_words(a.q + off, C.P, a.pp.t_hi, a.pp.t_lo, hi, lo);
-        __syncthreads();
-        // core = hi, with a hi neighbour if asked; mask = core, and lo with a core neighbour. The
-        // neighbours of the pixels in lo (hi is part of it) are loaded once for both
         const int nw = words_of(C.P);
-        int4 nbr[UNF_WORDS];
-        auto fetch = [&](int w0) {
+        const float* q = a.q + off + 32 * warp + lane;
+        // bit k of this lane: its pixel of the warp's word k (warp + 8 k); of the warp: any pixel of it
+        unsigned is_hi = 0, is_lo = 0, any_hi = 0, any_lo = 0;
 #pragma unroll
-            for (int k = 0; k < UNF_WORDS; ++k) {
-                const int w = w0 + warp + UNF_WARPS * k;
-                if (w < nw && ((lo[w] >> lane) & 1u)) nbr[k] = __ldg(C.nb + (32 * w + lane));
+        for (int k0 = 0; k0 < CLEAN_WORDS; k0 += 8) {
+            if (warp + CLEAN_WARPS * k0 >= nw) break;
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int at = 32 * CLEAN_WARPS * (k0 + k);
+                v[k] = at + 32 * warp + lane < C.P ? __ldg(q + at) : __int_as_float(0x7fc00000);   // NaN: neither
             }
-        };
-        for (int w0 = 0; w0 < nw; w0 += UNF_STEP) {
-            fetch(w0);
 #pragma unroll
-            for (int k = 0; k < UNF_WORDS; ++k) {
-                const int w = w0 + warp + UNF_WARPS * k;
+            for (int k = 0; k < 8; ++k) {
+                const int w = warp + CLEAN_WARPS * (k0 + k);
                 if (w >= nw) break;
-                bool on = (hi[w] >> lane) & 1u;
-                if (on && a.pp.core_nb) on = any_neighbour(nbr[k], C.K, C.P, hi);
-                const uint32_t b = __ballot_sync(0xffffffffu, on);
-                if (lane == 0) core[w] = b;
+                const bool h = v[k] >= a.pp.t_hi, l = v[k] >= a.pp.t_lo;
+                const uint32_t bh = __ballot_sync(0xffffffffu, h);
+                is_hi |= unsigned(h) << (k0 + k);
+                is_lo |= unsigned(l) << (k0 + k);
+                any_hi |= unsigned(bh != 0) << (k0 + k);
+                any_lo |= unsigned(__any_sync(0xffffffffu, l)) << (k0 + k);
+                if (lane == 0) hi[w] = bh;
             }
         }
         __syncthreads();
-        for (int w0 = 0; w0 < nw; w0 += UNF_STEP) {
-            if (nw > UNF_STEP) fetch(w0);                // else they are still there
-#pragma unroll
-            for (int k = 0; k < UNF_WORDS; ++k) {
-                const int w = w0 + warp + UNF_WARPS * k;
-                if (w >= nw) break;
-                bool on = (core[w] >> lane) & 1u;
-                if (!on && ((lo[w] >> lane) & 1u)) on = any_neighbour(nbr[k], C.K, C.P, core);
-                const uint32_t b = __ballot_sync(0xffffffffu, on);
-                if (lane == 0) mask[w] = b;
-            }
+        // core = hi, with a hi neighbour if asked
+        const int mine = warp + CLEAN_WARPS * lane;
+        if (lane < CLEAN_WORDS && mine < nw && !((any_hi >> lane) & 1u)) core[mine] = 0u;
+        unsigned is_mask = 0;
+        for (unsigned m = any_hi; m; m &= m - 1) {
+            const int k = __ffs(m) - 1, w = warp + CLEAN_WARPS * k;
+            bool on = (is_hi >> k) & 1u;
+            if (on && a.pp.core_nb) on = any_neighbour(__ldg(C.nb + (32 * w + lane)), C.K, C.P, hi);
+            is_mask |= unsigned(on) << k;
+            const uint32_t b = __ballot_sync(0xffffffffu, on);
+            if (lane == 0) core[w] = b;
         }
         __syncthreads();
-        uint8_t* out = a.mask + off;
-        const int quads = C.P >> 2;
-        if ((reinterpret_cast<uintptr_t>(out) & 3u) == 0) {
-            // four pixels a thread: bits 0..3 spread to the bytes
-            for (int g = threadIdx.x; g < quads; g += blockDim.x) {
-                const uint32_t b = (mask[g >> 3] >> (4 * (g & 7))) & 15u;
-                reinterpret_cast<uint32_t*>(out)[g] = (b * 0x00204081u) & 0x01010101u;
-            }
-            for (int p = 4 * quads + threadIdx.x; p < C.P; p += blockDim.x) out[p] = bit_of(mask, p) ? 1 : 0;
-        } else {
-            for (int p = threadIdx.x; p < C.P; p += blockDim.x) out[p] = bit_of(mask, p) ? 1 : 0;
+        // mask = core, and lo with a core neighbour
+        for (unsigned m = any_lo; m; m &= m - 1) {
+            const int k = __ffs(m) - 1, w = warp + CLEAN_WARPS * k;
+            if ((is_lo & ~is_mask) >> k & 1u)
+                is_mask |= unsigned(any_neighbour(__ldg(C.nb + (32 * w + lane)), C.K, C.P, core)) << k;
         }
-        __syncthreads();
+        uint8_t* out = a.mask + off + 32 * warp + lane;
+        for (int k = 0; warp + CLEAN_WARPS * k < nw; ++k)
+            if (32 * (warp + CLEAN_WARPS * k) + lane < C.P) out[32 * CLEAN_WARPS * k] = (is_mask >> k) & 1u;
     }
 }
+
+// k_hillas: four warps, so that an SM holds eight images. 500, 4,224 and 28,160 images of the three
+// presets 10.5, 32.9 and 200 us, 7,800 of 256 pixels 48 us; 11.3, 40.3, 224 and 90 with eight warps,
+// 12.9, 48.5, 400 and 84 with a thread per bitmap word.
+constexpr int UNF_WARPS = 4;
+constexpr int UNF_WORDS = 8;      // words a warp takes at a time
+constexpr int UNF_STEP = UNF_WARPS * UNF_WORDS;
 
 __global__ void __launch_bounds__(UNF_WARPS * 32) k_hillas(const HillasArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -243,8 +229,8 @@ int chain_occupancy(int v, size_t smem, int kind) {
 }
 
 cudaError_t launch_clean(const CleanArgs& a, int grid, cudaStream_t s) {
-    const size_t smem = size_t(16) * ((a.arr.max_P + 31) / 32) + 16;
-    k_clean<<<grid, UNF_WARPS * 32, smem, s>>>(a);
+    const size_t smem = size_t(8) * ((a.arr.max_P + 31) / 32);
+    k_clean<<<grid, CLEAN_WARPS * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 

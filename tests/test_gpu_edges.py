@@ -591,3 +591,48 @@ def test_threads_with_cameras_of_different_sizes_do_not_disturb_each_other():
     for ctx, _, want in jobs:
         assert ctx.check() == 0 and int(want[0].view(torch.int32).view(-1, 16)[:, 10].min()) > 0
         ctx.close()
+
+
+@pytest.mark.parametrize("core_nb", [0, 1])
+@pytest.mark.parametrize("P", [8, 31, 33, 256, 257, 1023, 1025, 2049, 4096])
+def test_stage_calls_on_more_images_than_fit_at_once(P, core_nb):
+    """rta_clean and rta_hillas on charges of every density, NaN and values at the thresholds among
+    them, several images per block and rows at odd offsets: masks as the oracle's pixel by pixel,
+    rows within the usual rules and the same for every copy of an image."""
+    rng = np.random.default_rng(P)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    kinds, n_img, hi, lo = 9, 17 * n_sm + 5, 10.0, 5.0
+    xy, nb = synth.lattice("hex", P, 0.1)
+    q = rng.normal(0, 2, (kinds, P)).astype(np.float32)
+    for i in range(1, kinds):                        # none to nearly all pixels above the thresholds
+        pick = rng.random(P) < [0, 0.01, 0.05, 0.2, 0.5, 0.9, 1, 0.1, 0.3][i]
+        q[i, pick] = rng.uniform(3, 60, int(pick.sum())).astype(np.float32)
+    q[7, ::5], q[7, 1::5], q[7, 2::5] = hi, lo, np.nextafter(np.float32(lo), np.float32(0))
+    q[8, ::11] = np.nan
+    t = rng.uniform(0, 20, (kinds, P)).astype(np.float32)
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, 8)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                       np.full(P, 1 / 128, np.float32))
+    step = P + 3
+    dq = torch.full((n_img, step), 1e9, dtype=torch.float32, device="cuda")     # (must not be read)
+    dt = torch.zeros_like(dq)
+    which = torch.arange(n_img, device="cuda") % kinds
+    dq[:, :P], dt[:, :P] = torch.from_numpy(q).cuda()[which], torch.from_numpy(t).cuda()[which]
+    dq, dt = dq.view(-1), dt.view(-1)
+    pix = torch.arange(n_img, dtype=torch.int64, device="cuda") * step
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    mask = torch.full(dq.shape, 7, dtype=torch.uint8, device="cuda")
+    ctx.clean(dq, tel, pix, hi, lo, core_nb, mask)
+    out = torch.zeros(n_img * 16, dtype=torch.float32, device="cuda")
+    ctx.hillas(dq, dt, mask, tel, pix, out)
+    assert ctx.check() == 0
+    m = mask.cpu().numpy().reshape(n_img, step)
+    assert (m[:, P:] == 7).all()
+    ref = [oracle.clean(q[i], nb, hi, lo, core_nb) for i in range(kinds)]
+    np.testing.assert_array_equal(m[:, :P], np.array(ref)[np.arange(n_img) % kinds])
+    raw = out.cpu().numpy().view(np.uint32).reshape(n_img, 16)
+    np.testing.assert_array_equal(raw, raw[:kinds][np.arange(n_img) % kinds])
+    rows = np.array([oracle.hillas(xy, q[i], t[i], ref[i]) for i in range(kinds)])
+    compare_hillas(hillas_rows(out[: kinds * 16], kinds), rows, f"stages {P}")
+    ctx.close()
