@@ -17,8 +17,9 @@
 // instruction holds its sub-partition's pipe for a long time whatever the
 // number of active lanes. Four neighbouring threads therefore take one event,
 // a sum and a quotient each: an image costs a warp one addition for eight
-// events instead of four for the events of a thread each (10,000 events
-// 12.3 us; 18.6 with a thread per event).
+// events instead of four for the events of a thread each (10,000 events of the
+// array 12.3 us; 18.6 with a thread per event). Many events of few images are an
+// exception (lut_threads_per_event).
 //
 // k_lut_train: one thread per training event, FP64 atomic sums per cell.
 // k_lut_finalize, k_lut_prepare: one thread per cell.
@@ -30,9 +31,7 @@ namespace rta {
 
 namespace {
 
-constexpr int LUT_THREADS = 512;
-constexpr int LUT_MAX_EPB = 128;    // events per group at most (four threads each)
-static_assert(LUT_THREADS == 4 * LUT_MAX_EPB, "four threads an event");
+constexpr int LUT_MAX_EPB = 128;    // events per group at most
 constexpr int LUT_PIECE = 1024;     // per-image terms staged per pass
 
 // The lookup form of one cell (RTA_LUT_LOOKUP_BYTES = 64 bytes).
@@ -109,9 +108,9 @@ __device__ __forceinline__ int64_t cell_index(const LutArgs& a, int cam, int iu,
 // issues each stage's loads for all of them before using any, so the chain
 // image row -> telescope -> cell costs three memory latencies per batch
 // instead of three per image.
-constexpr int LUT_ILP = 2;
-
+template <int TPE>
 __device__ __forceinline__ void stage_terms(const LutArgs& a, LutSmem& sm, int epb, long long p0, long long p1) {
+    constexpr int LUT_THREADS = TPE * LUT_MAX_EPB, LUT_ILP = TPE == 4 ? 2 : 4;
     for (long long base = p0 + threadIdx.x; base < p1; base += LUT_THREADS * LUT_ILP) {
         int64_t img[LUT_ILP];
         int slot[LUT_ILP];
@@ -202,11 +201,14 @@ __device__ __forceinline__ void stage_terms(const LutArgs& a, LutSmem& sm, int e
     }
 }
 
-__global__ void __launch_bounds__(LUT_THREADS) k_lut_events(const LutArgs a) {
+// TPE: threads an event, four or one.
+template <int TPE>
+__global__ void __launch_bounds__(TPE * LUT_MAX_EPB) k_lut_events(const LutArgs a) {
+    constexpr int LUT_THREADS = TPE * LUT_MAX_EPB, PARTS = 4 / TPE;
     __shared__ LutSmem sm;
     grid_dependency_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int slot = tid >> 2, part = tid & 3;         // this thread's event in the group and its sum
+    const int slot = tid / TPE, part0 = tid % TPE;     // this thread's event in the group and its first sum
     for (int k = tid; k <= a.n_size; k += LUT_THREADS) sm.se[k] = a.size_edges[k];
     for (int k = tid; k <= a.n_dist; k += LUT_THREADS) sm.de[k] = a.dist_edges[k];
     const int epb = a.events_per_block;
@@ -263,46 +265,58 @@ __global__ void __launch_bounds__(LUT_THREADS) k_lut_events(const LutArgs a) {
         __syncthreads();
         const long long total = sm.pre[epb];
         const long long my0 = slot < epb ? sm.pre[slot] : 0, my1 = slot < epb ? sm.pre[slot + 1] : 0;
-        double sum = 0.0;                    // of the scaled widths, scaled lengths, w_e or w_e mean_e
+        double sum[PARTS] = {};              // of the scaled widths, scaled lengths, w_e, w_e mean_e
         int n = 0;
         for (long long p0 = 0; p0 < total; p0 += LUT_PIECE) {
             const long long p1 = min(total, p0 + LUT_PIECE);
-            stage_terms(a, sm, epb, p0, p1);
+            stage_terms<TPE>(a, sm, epb, p0, p1);
             __syncthreads();
             const long long j0 = max(my0, p0), j1 = min(my1, p1);
-            const double* term = sm.term[part];
+            const double* term = sm.term[part0];
             for (long long j = j0; j < j1; ++j) {
                 const int k = int(j - p0);
                 if (sm.tu[k]) {
                     ++n;
-                    sum = __dadd_rn(sum, term[k]);
+                    sum[0] = __dadd_rn(sum[0], term[k]);
+#pragma unroll
+                    for (int q = 1; q < PARTS; ++q) sum[q] = __dadd_rn(sum[q], term[q * LUT_PIECE + k]);
                 }
             }
             __syncthreads();
         }
         // mscw, mscl = sums / n; log E = sum(w_e mean_e) / sum(w_e); sigma = sqrt(1 / sum(w_e)): one
-        // quotient per thread (thread 2 forms sigma, thread 3 log E)
-        const double sd = __shfl_sync(0xffffffffu, sum, (lane & ~3) + 2);
+        // quotient per sum (the third thread's, or sum's, is the one under the root)
+        const double sd = TPE == 1 ? sum[2 % PARTS] : __shfl_sync(0xffffffffu, sum[0], (lane & ~3) + 2);
         const int state = slot < epb ? sm.state[slot] : 3;
         const bool fold = state == 0 && n > 0;
-        const double top = part == 2 ? 1.0 : sum, under = part < 2 ? double(n) : sd;
-        double v = 0.0;
-        if (fold) v = __ddiv_rn(top, under);
-        if (fold && part == 2) v = __dsqrt_rn(v);
-        const bool in = fold && part < 2 && (part == 0 ? cw_lo <= v && v <= cw_hi : cl_lo <= v && v <= cl_hi);
-        const unsigned inside = __ballot_sync(0xffffffffu, in);
+        double v[PARTS];
+        bool in = fold;                      // those of mscw and mscl that this thread has are within the cuts
+#pragma unroll
+        for (int q = 0; q < PARTS; ++q) {
+            const int part = part0 + q;
+            const double top = part == 2 ? 1.0 : sum[q], under = part < 2 ? double(n) : sd;
+            v[q] = 0.0;
+            if (fold) v[q] = __ddiv_rn(top, under);
+            if (fold && part == 2) v[q] = __dsqrt_rn(v[q]);
+            if (part < 2) in = in && (part == 0 ? cw_lo : cl_lo) <= v[q] && v[q] <= (part == 0 ? cw_hi : cl_hi);
+        }
+        if (TPE == 4) in = ((__ballot_sync(0xffffffffu, in) >> (lane & ~3)) & 3u) == 3u;
         if (state != 3) {
             // the row: log E, sigma, mscw, mscl, n_used, flags, two reserved
             float* row = reinterpret_cast<float*>(a.out + e0 + slot);
-            row[part == 0 ? 2 : part == 1 ? 3 : part == 2 ? 1 : 0] = __double2float_rn(v);
             uint32_t flags = 0;
             if (state == 1) flags = RTA_LF_MALFORMED;
             else if (state == 2) flags = RTA_LF_NO_CORE;
             else if (n == 0) flags = RTA_LF_NO_IMAGE;
-            else if (((inside >> (lane & ~3)) & 3u) == 3u) flags = RTA_LF_GAMMA;
-            row[4 + part] = part == 0   ? __int_as_float(state == 1 ? -1 : state == 0 ? n : 0)
-                            : part == 1 ? __uint_as_float(flags)
-                                        : 0.f;
+            else if (in) flags = RTA_LF_GAMMA;
+#pragma unroll
+            for (int q = 0; q < PARTS; ++q) {
+                const int part = part0 + q;
+                row[part == 0 ? 2 : part == 1 ? 3 : part == 2 ? 1 : 0] = __double2float_rn(v[q]);
+                row[4 + part] = part == 0   ? __int_as_float(state == 1 ? -1 : state == 0 ? n : 0)
+                                : part == 1 ? __uint_as_float(flags)
+                                            : 0.f;
+            }
         }
         __syncthreads();   // the next group reuses the shared arrays
     }
@@ -388,19 +402,19 @@ int lut_events_per_block(int64_t n_evt, int n_sm) {
     return int(std::min<int64_t>(LUT_MAX_EPB, std::max<int64_t>(16, epb)));
 }
 
+// With a full group of events for every SM and few images each, an SM's registers hold more events
+// with a thread each than with four, and the sums are too short to share: 50,000 events of 1, 2, 3
+// and 5 images 12.8, 15.0, 17.5 and 23.0 us, 18.6, 20.0, 21.4 and 22.7 with four threads; 10,000 of 3
+// images 10.9 and 9.1.
+int lut_threads_per_event(int64_t n_evt, int64_t n_img, int n_sm) {
+    return n_evt >= int64_t(n_sm) * LUT_MAX_EPB && n_img <= 3 * n_evt ? 1 : 4;
+}
+
 cudaError_t launch_lut_reconstruct(const LutArgs& a, int grid, cudaStream_t s) {
     // a programmatic dependent: its blocks start while the kernel before (the stereo kernel, as a
     // rule) ends, and wait for it before they read anything
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid));
-    cfg.blockDim = dim3(LUT_THREADS);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_lut_events, a);
+    return a.threads_per_event == 1 ? launch_dependent(k_lut_events<1>, unsigned(grid), LUT_MAX_EPB, 0, s, a)
+                                    : launch_dependent(k_lut_events<4>, unsigned(grid), 4 * LUT_MAX_EPB, 0, s, a);
 }
 
 cudaError_t launch_lut_accumulate(const LutArgs& a, int grid, cudaStream_t s) {

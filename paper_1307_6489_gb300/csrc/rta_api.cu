@@ -1292,6 +1292,7 @@ int rta_lut_reconstruct(rta_ctx* c, const rta_hillas_t* d_hillas, const int32_t*
     a.cut[3] = mscl_hi;
     a.out = d_out;
     a.events_per_block = rta::lut_events_per_block(n_evt, c->n_sm);
+    a.threads_per_event = rta::lut_threads_per_event(n_evt, n_img, c->n_sm);
     const int64_t g = std::min<int64_t>((n_evt + a.events_per_block - 1) / a.events_per_block, int64_t(c->n_sm) * 16);
     CUDA_TRY(rta::launch_lut_reconstruct(a, int(g), (cudaStream_t)stream));
     return RTA_OK;

@@ -255,9 +255,10 @@ struct LutArgs {
     float cut[4];                   // mscw_lo, mscw_hi, mscl_lo, mscl_hi
     rta_lut_event_t* out;
     unsigned int* status;
-    int events_per_block;
+    int events_per_block, threads_per_event;
 };
 int lut_events_per_block(int64_t n_evt, int n_sm);
+int lut_threads_per_event(int64_t n_evt, int64_t n_img, int n_sm);
 cudaError_t launch_lut_reconstruct(const LutArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_lut_accumulate(const LutArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_lut_finalize(const double* acc, int64_t n_cells, int min_count, rta_lut_cell_t* cells, int grid,

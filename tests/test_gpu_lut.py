@@ -247,6 +247,36 @@ def test_full_bundle_matches_the_oracle(ctx_of):
     assert (g["n_used"] > 0).sum() > 5000
 
 
+@pytest.mark.parametrize("extra", [-1, 0, 129])
+def test_many_events_of_few_images_match_the_oracle(training, ctx_of, extra):
+    """Around a full group of events for every SM, from where an event of few images has a thread to
+    itself: zero to six images each, one of 3000 (several staging pieces), malformed ranges,
+    unknown telescopes, events without a core."""
+    wl, hbuf, sbuf = training
+    rng = np.random.default_rng(12)
+    n_evt = 128 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    ref_cells, _ = oracle_build(wl, hbuf, (wl.truth[:, 5] == 0), 5)
+    cells = oracle_cells_as_struct(ref_cells)
+    sizes = rng.integers(0, 6, n_evt)
+    sizes[n_evt // 2] = 3000
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    n_img = int(off[-1])
+    assert n_img <= 3 * n_evt
+    pick = rng.integers(0, len(hbuf), n_img)
+    hb, tel = hbuf[pick], wl.img_tel[pick].copy()
+    tel[::501] = 10 ** 6
+    hb[::997, 4] = np.nan
+    st = sbuf[rng.integers(0, len(sbuf), n_evt)].copy()
+    st.view(np.int32)[::50, 5] |= oracle.FLAG_STEREO_INVALID
+    st.view(np.int32)[n_evt // 2, 5] &= ~oracle.FLAG_STEREO_INVALID
+    off[77], off[1001] = -5, off[1002] + 1
+    g = gpu_reconstruct(ctx_of, hb, tel, off, n_img, st, cells, expect_bits=rta.RTA_DEV_BAD_IMAGE)
+    ref = lut.lut_reconstruct(f32_rows_as_oracle(hb), tel, off, n_img, wl.tel_cam, wl.tel_xy,
+                              f32_stereo_as_oracle(st), ref_cells, SIZE_EDGES, DIST_EDGES, CUTS)
+    compare_events(g, ref)
+    assert g["n_used"][n_evt // 2] > 100 and (g["flags"] & rta.RTA_LF_MALFORMED).any()
+
+
 def test_bad_arguments_are_refused(training, ctx_of):
     wl, hbuf, sbuf = training
     h = dev(hbuf.reshape(-1))
