@@ -196,16 +196,19 @@ int rta_selftest_wait_timeout(rta_ctx* ctx, int timeout_ms, uint64_t* waited_ns,
  * fit). Sets the configuration of every window mode, the neighbour-peak
  * window's included (whose kernel runs with as many of the CTAs as fit), and
  * of the byte-stream path (rta_reconstruct_stream), undoing what
- * rta_autotune_stream tuned. Returns RTA_E_INVALID if the combination does not fit in shared memory for
+ * rta_autotune_stream tuned. Every launch then runs as set; until then, those of
+ * at most one image per SM use more stages than the default two. In flat-window
+ * launches that write rows alone, for cameras of at most 512 pixels and fewer than
+ * 64 samples, variant 4 with up to two CTAs per SM (0: two) has eight image slots
+ * instead of two. Returns RTA_E_INVALID if the combination does not fit in shared memory for
  * the registered cameras. Results do not depend on the configuration. */
 int rta_set_chain_config(rta_ctx* ctx, int variant, int n_stages, int ctas_per_sm);
 
 /* The configuration a launch outside the neighbour-peak mode would use now (the
  * byte-stream path too, unless rta_autotune_stream has tuned its own):
  * variant, stages, CTAs per SM, grid size and dynamic shared memory per CTA in
- * bytes (NULL outputs are skipped). Launches of at most one image per SM use more
- * stages than the default configuration's two, and small cameras (at most 512
- * pixels) more image slots; results do not depend on it. */
+ * bytes of rta_image_chain on a large bundle in the flat window (NULL outputs are
+ * skipped). */
 int rta_get_chain_config(rta_ctx* ctx, int* variant, int* n_stages, int* ctas_per_sm, int* grid,
                          size_t* smem_bytes);
 
@@ -238,7 +241,9 @@ typedef struct rta_tune_entry_t {
  * *n_entries = number measured). The neighbour-peak window
  * (RTA_WINDOW_NEIGHBOUR) has a configuration of its own, which a call in that
  * mode tunes; a call in any other mode tunes the configuration all other modes
- * share. d_out receives the (configuration-independent) Hillas rows.
+ * share. Launches of at most one image per SM run as the tuned configuration says
+ * if the bundle was such a launch, else with more stages where it has two. d_out
+ * receives the (configuration-independent) Hillas rows.
  * Synchronises `stream`. */
 int rta_autotune(rta_ctx* ctx, const uint16_t* d_wave, int64_t n_wave, const int64_t* d_wave_off,
                  const int32_t* d_img_tel, int64_t n_img, int window_mode, int start, int W, float t_hi,

@@ -648,8 +648,6 @@ __device__ __forceinline__ void write_bad_row(rta_hillas_t* out) {
 // parameterise than to integrate) as many as there are slots, one each.
 __host__ __device__ constexpr int chain_slots(int tails) { return tails > 2 ? tails : 2; }
 __host__ __device__ constexpr int chain_block(int iw, int tails) { return iw * 32 + 32 + 32 * tails; }
-constexpr int SMALL_TAILS = 8;
-constexpr int SMALL_PIX = 512;      // pixels of the largest camera that counts as small
 enum { SLOT_END = 1 };
 
 struct SlotHdr {

@@ -1,8 +1,6 @@
 // Launches of the image chain's kernels (k_image_chain.cuh), compiled in several files so that the
 // builds run in parallel.
 #pragma once
-#include <algorithm>
-
 #include "k_image_chain.cuh"
 
 namespace rta {
@@ -41,16 +39,7 @@ cudaError_t dispatch_chain(int v, const ChainArgs& a, int grid, size_t smem, cud
 // Contiguous bundles, rows only, the flat window (of WIN samples in the specialised searches).
 template <int SEARCH, int WIN = 6>
 cudaError_t dispatch_flat_rows(int v, const ChainArgs& a, int grid, size_t smem, cudaStream_t s) {
-    // small cameras: variant 4's tile with a tail warp for each of eight slots, two CTAs an SM (an
-    // image of 256 pixels is integrated in a fraction of the time its cleaning and moments take:
-    // 2,000 of them 21.4 us, 35.5 with one tail warp for two slots); with rows of 64 samples and more
-    // the search sets the pace again (303 of 208 x 100: 30.3 us so, 28.9 with three CTAs an SM)
-    if (v == 4 && a.arr.max_P <= SMALL_PIX && a.max_S < 64) {
-        const size_t sm8 = chain_smem_bytes(4, a.nstage, a.stage_wave_bytes, a.arr.max_P, 0, 0, SMALL_TAILS);
-        const int g8 = int(std::min<int64_t>(a.n_img, 2 * int64_t(a.n_sm)));
-        if (sm8 <= SMEM_PER_CTA)
-            return launch_chain<8, 1, 2, false, false, 0, OUT_ROWS, SEARCH, SMALL_TAILS, WIN>(a, g8, sm8, s, false, nullptr);
-    }
+    if (a.small) return launch_chain<8, 1, 2, false, false, 0, OUT_ROWS, SEARCH, SMALL_TAILS, WIN>(a, grid, smem, s, false, nullptr);
     return dispatch_chain<false, false, 0, OUT_ROWS, SEARCH, WIN>(v, a, grid, smem, s);
 }
 

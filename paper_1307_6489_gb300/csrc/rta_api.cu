@@ -100,6 +100,7 @@ struct rta_ctx {
     int variant = 4;      // tile shape, see chain_variant_* (the fastest on GB300 for the array cameras)
     int nstage = 2;
     int ctas_per_sm = 0;  // 0 = the variant's target, shrinking the stages to fit, else as many as fit
+    bool exact_config = false;   // set by the caller: every launch runs as it says
     // the neighbour-peak kernel's own configuration (more shared memory per CTA,
     // a per-image barrier: its fastest shape differs)
     int nb_variant = 0;
@@ -229,9 +230,20 @@ struct ChainCfg {
     int variant, nstage, ctas_per_sm;
 };
 
-// kind: which instantiation (rta::CHAIN_*); the neighbour-peak one also needs its keys in shared memory
-int config_launch(rta_ctx* c, const ChainCfg& k, int64_t n_img, int* grid, size_t* smem, int* swb,
-                  int kind = rta::CHAIN_PLAIN) {
+// What a launch runs with.
+struct ChainLaunch {
+    int nstage, swb, grid;
+    size_t smem;
+    int small;     // the form for small cameras (dispatch_flat_rows)
+};
+
+// kind: which instantiation (rta::CHAIN_*); the neighbour-peak one also needs its keys in shared memory.
+// flat_rows: rows of the flat window alone. deep: launches of an image per SM at most may take more
+// stages than the configuration's two.
+int config_launch(rta_ctx* c, const ChainCfg& k, int64_t n_img, ChainLaunch* out, int kind = rta::CHAIN_PLAIN,
+                  bool flat_rows = false, bool deep = false) {
+    int* const swb = &out->swb;
+    size_t* const smem = &out->smem;
     const int nb = kind == rta::CHAIN_NB;
     // the stream kernel keeps two per-image records (the neighbour-peak one too: it may run on a stream)
     const int st = kind == rta::CHAIN_STREAM || kind == rta::CHAIN_NB;
@@ -285,9 +297,37 @@ int config_launch(rta_ctx* c, const ChainCfg& k, int64_t n_img, int* grid, size_
             return fail(RTA_E_INVALID, "%d CTAs/SM do not fit (%d do)", k.ctas_per_sm, occ);
         occ = std::min(occ, k.ctas_per_sm);
     }
-    int64_t g = int64_t(c->n_sm) * occ;
-    g = std::min<int64_t>(g, std::max<int64_t>(n_img, 1));
-    *grid = int(g);
+    out->nstage = nst;
+    if (deep && kind == rta::CHAIN_PLAIN && k.variant == 4 && nst == 2 && n_img <= c->n_sm) {
+        // an image per SM at most (an alert): no other CTA of the launch shares the SM, so the stages
+        // that would make room for two more hold the image's next chunks instead. A reconstruction of 8
+        // events (37 to 43 images) takes 17.3 us with this and without the counter's reset, 20.7 before.
+        // (Such launches on several streams at once share fewer SMs than with two stages.)
+        const int full = rta::chain_stage_wave_bytes(k.variant, c->max_S);
+        for (int n = 8; n > 2; --n) {
+            const size_t sm = rta::chain_smem_bytes(k.variant, n, full, c->max_P);
+            if (sm > rta::SMEM_PER_CTA) continue;
+            out->nstage = n;
+            *swb = full;
+            *smem = sm;
+            break;
+        }
+    }
+    out->small = 0;
+    if (flat_rows && kind == rta::CHAIN_PLAIN && k.variant == 4 && k.ctas_per_sm <= 2 && c->max_P <= rta::SMALL_PIX &&
+        c->max_S < 64) {
+        // small cameras: variant 4's tile with a tail warp for each of eight slots, two CTAs an SM (an
+        // image of 256 pixels is integrated in a fraction of the time its cleaning and moments take:
+        // 2,000 of them 21.4 us, 35.5 with one tail warp for two slots); with rows of 64 samples and more
+        // the search sets the pace again (303 of 208 x 100: 30.3 us so, 28.9 with three CTAs an SM)
+        const size_t sm8 = rta::chain_smem_bytes(4, out->nstage, *swb, c->max_P, 0, 0, rta::SMALL_TAILS);
+        if (sm8 <= rta::SMEM_PER_CTA) {
+            out->small = 1;
+            *smem = sm8;
+            occ = std::min(k.ctas_per_sm > 0 ? k.ctas_per_sm : 2, rta::SMEM_PER_CTA + 1024 >= 2 * (sm8 + 1024) ? 2 : 1);
+        }
+    }
+    out->grid = int(std::min<int64_t>(int64_t(c->n_sm) * occ, std::max<int64_t>(n_img, 1)));
     return RTA_OK;
 }
 
@@ -297,10 +337,6 @@ ChainCfg cfg_of(const rta_ctx* c, int kind) {
     if (kind == rta::CHAIN_NB) return ChainCfg{c->nb_variant, c->nb_nstage, c->nb_ctas_per_sm};
     if (kind == rta::CHAIN_STREAM && c->st_variant >= 0) return ChainCfg{c->st_variant, c->st_nstage, c->st_ctas_per_sm};
     return ChainCfg{c->variant, c->nstage, c->ctas_per_sm};
-}
-
-int chain_launch_config(rta_ctx* c, int64_t n_img, int* grid, size_t* smem, int* swb, int kind = rta::CHAIN_PLAIN) {
-    return config_launch(c, cfg_of(c, kind), n_img, grid, smem, swb, kind);
 }
 
 int launch_search(const rta_ctx* c, const rta::ProcParams& pp, bool rows) {
@@ -316,26 +352,12 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
               const int64_t* d_n_img = nullptr, const rta_segment_t* d_seg = nullptr,
               const int32_t* d_img_seg = nullptr, int64_t n_seg = 0, rta::StreamImg* d_smeta = nullptr,
               uint8_t* d_mask = nullptr) {
-    int grid, swb;
-    size_t smem;
     const int kind = pp.nbpeak ? rta::CHAIN_NB : d_smeta ? rta::CHAIN_STREAM : rta::CHAIN_PLAIN;
-    int rc = chain_launch_config(c, n_img, &grid, &smem, &swb, kind);
+    const bool rows = !integrate_only && !d_mask && !d_smeta;
+    const ChainCfg cfg = cfg_of(c, kind);
+    ChainLaunch l;
+    int rc = config_launch(c, cfg, n_img, &l, kind, rows && !pp.filter, !c->exact_config);
     if (rc) return rc;
-    ChainCfg cfg = cfg_of(c, kind);
-    if (kind == rta::CHAIN_PLAIN && cfg.variant == 4 && cfg.nstage == 2 && n_img <= c->n_sm) {
-        // an image per SM at most (an alert): nothing shares the SM, so the stages that would make
-        // room for two more CTAs hold the image's next chunks instead. A reconstruction of 8 events
-        // (37 to 43 images) takes 17.3 us with this and without the counter's reset, 20.7 before.
-        const int full = rta::chain_stage_wave_bytes(cfg.variant, c->max_S);
-        for (int k = 8; k > 2; --k) {
-            const size_t sm = rta::chain_smem_bytes(cfg.variant, k, full, c->max_P);
-            if (sm > rta::SMEM_PER_CTA) continue;
-            cfg.nstage = k;
-            swb = full;
-            smem = sm;
-            break;
-        }
-    }
     rta::ChainArgs a{};
     a.arr = dev_array(c);
     a.pp = pp;
@@ -353,22 +375,21 @@ int run_chain(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64_t*
     a.mask_out = d_mask;
     a.counter = counter ? counter : take_counter(c);
     a.status = c->d_status;
-    a.stage_wave_bytes = swb;
+    a.stage_wave_bytes = l.swb;
     a.max_S = c->max_S;
-    a.nstage = std::max(2, std::min(cfg.nstage, 8));
+    a.nstage = l.nstage;
+    a.small = l.small;
     a.integrate_only = integrate_only;
-    a.search = launch_search(c, pp, !integrate_only && !d_mask && !d_smeta);
-    a.n_sm = c->n_sm;
+    a.search = launch_search(c, pp, rows);
     a.n_img_dev = d_n_img;
     a.seg = d_seg;
     a.img_seg = d_img_seg;
     a.n_seg = n_seg;
     a.smeta = d_smeta;
     if (d_smeta) CUDA_TRY(rta::launch_stream_meta(a, d_smeta, n_img, c->n_sm, s));
-    // with an image for every block at most, whatever the counter holds ends the launch (small
-    // cameras run with two blocks an SM)
-    if (n_img > std::min<int64_t>(grid, 2 * int64_t(c->n_sm))) CUDA_TRY(cudaMemsetAsync(a.counter, 0, sizeof(unsigned int), s));
-    CUDA_TRY(rta::launch_image_chain(cfg.variant, a, grid, smem, s));
+    // with an image for every block at most, whatever the counter holds ends the launch
+    if (n_img > l.grid) CUDA_TRY(cudaMemsetAsync(a.counter, 0, sizeof(unsigned int), s));
+    CUDA_TRY(rta::launch_image_chain(cfg.variant, a, l.grid, l.smem, s));
     return RTA_OK;
 }
 
@@ -632,13 +653,13 @@ int rta_set_chain_config(rta_ctx* c, int variant, int n_stages, int ctas_per_sm)
     if (rc) return rc;
     if (n_stages < 2 || n_stages > 8) return fail(RTA_E_INVALID, "n_stages %d outside 2..8", n_stages);
     if (ctas_per_sm < 0 || ctas_per_sm > 8) return fail(RTA_E_INVALID, "ctas_per_sm %d outside 0..8", ctas_per_sm);
-    int g, swb;
-    size_t sm;
-    if ((rc = config_launch(c, ChainCfg{variant, n_stages, ctas_per_sm}, int64_t(1) << 30, &g, &sm, &swb))) return rc;
+    ChainLaunch l;
+    if ((rc = config_launch(c, ChainCfg{variant, n_stages, ctas_per_sm}, int64_t(1) << 30, &l))) return rc;
     c->variant = c->nb_variant = variant;
     c->nstage = c->nb_nstage = n_stages;
     c->ctas_per_sm = c->nb_ctas_per_sm = ctas_per_sm;
     c->st_variant = -1;
+    c->exact_config = true;
     return RTA_OK;
 }
 
@@ -660,15 +681,13 @@ int rta_set_filter_weights(rta_ctx* c, const int32_t* w, int W) {
 int rta_get_chain_config(rta_ctx* c, int* variant, int* n_stages, int* ctas_per_sm, int* grid, size_t* smem_bytes) {
     int rc = check_ctx(c);
     if (rc) return rc;
-    int g, swb;
-    size_t sm;
-    rc = chain_launch_config(c, int64_t(1) << 30, &g, &sm, &swb);
-    if (rc) return rc;
+    ChainLaunch l;
+    if ((rc = config_launch(c, cfg_of(c, rta::CHAIN_PLAIN), int64_t(1) << 30, &l, rta::CHAIN_PLAIN, true))) return rc;
     if (variant) *variant = c->variant;
     if (n_stages) *n_stages = c->nstage;
-    if (ctas_per_sm) *ctas_per_sm = g / c->n_sm;
-    if (grid) *grid = g;
-    if (smem_bytes) *smem_bytes = sm;
+    if (ctas_per_sm) *ctas_per_sm = l.grid / c->n_sm;
+    if (grid) *grid = l.grid;
+    if (smem_bytes) *smem_bytes = l.smem;
     return RTA_OK;
 }
 
@@ -686,9 +705,11 @@ namespace {
 // Every configuration that fits (variant x 2..6 stages x 1..4 CTAs/SM) of the kernel of `kind`:
 // *cv, *cn, *cc (the context's fields for that kind) are set to it, `run` launches the kernel once
 // (one warm-up, then `reps` timed launches between CUDA events); the fastest is kept, or the
-// previous configuration if a launch failed.
+// previous configuration if a launch failed. flat_rows as in config_launch. The plain kernel's
+// launches run as each configuration says, and do so afterwards too if it was tuned on an image per
+// SM at most (else such launches take the deeper pipeline, which the sweep did not see).
 template <class Run>
-int tune_sweep(rta_ctx* c, int kind, int64_t n_img, int reps, cudaStream_t s, int* cv, int* cn, int* cc, Run run,
+int tune_sweep(rta_ctx* c, int kind, bool flat_rows, int64_t n_img, int reps, cudaStream_t s, int* cv, int* cn, int* cc, Run run,
                rta_tune_entry_t* h_entries, int max_entries, int* n_entries) {
     const ChainCfg saved{*cv, *cn, *cc};
     cudaEvent_t e0, e1;
@@ -697,15 +718,16 @@ int tune_sweep(rta_ctx* c, int kind, int64_t n_img, int reps, cudaStream_t s, in
         cudaEventDestroy(e0);
         return fail(RTA_E_CUDA, "cudaEventCreate failed");
     }
+    const bool exact_before = c->exact_config;
+    c->exact_config = true;
     ChainCfg best = saved;
     float best_ms = 1e30f;
     int n = 0, rc = RTA_OK;
     for (int v = 0; v < RTA_CHAIN_VARIANTS && !rc; ++v)
         for (int nst = 2; nst <= 6 && !rc; ++nst)
             for (int cps = 1; cps <= 4; ++cps) {
-                int g, swb;
-                size_t sm;
-                if (config_launch(c, ChainCfg{v, nst, cps}, n_img, &g, &sm, &swb, kind) != RTA_OK) continue;
+                ChainLaunch l;
+                if (config_launch(c, ChainCfg{v, nst, cps}, n_img, &l, kind, flat_rows) != RTA_OK) continue;
                 *cv = v;
                 *cn = nst;
                 *cc = cps;
@@ -718,12 +740,13 @@ int tune_sweep(rta_ctx* c, int kind, int64_t n_img, int reps, cudaStream_t s, in
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, e0, e1);
                 ms /= reps;
-                if (h_entries && n < max_entries) h_entries[n] = rta_tune_entry_t{v, nst, cps, g, ms};
+                if (h_entries && n < max_entries) h_entries[n] = rta_tune_entry_t{v, nst, cps, l.grid, ms};
                 ++n;
                 if (ms < best_ms) { best_ms = ms; best = ChainCfg{v, nst, cps}; }
             }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    c->exact_config = rc || kind != rta::CHAIN_PLAIN ? exact_before : n_img <= c->n_sm;
     const ChainCfg keep = rc ? saved : best;
     *cv = keep.variant;
     *cn = keep.nstage;
@@ -770,7 +793,7 @@ int rta_autotune(rta_ctx* c, const uint16_t* d_wave, int64_t n_wave, const int64
         return run_chain(c, d_wave, n_wave, d_wave_off, d_img_tel, nullptr, n_img, pp, nullptr, nullptr, 0, d_out, 0, s,
                          nullptr);
     };
-    return tune_sweep(c, kind, n_img, reps, s, cv, cn, cc, run, h_entries, max_entries, n_entries);
+    return tune_sweep(c, kind, !pp.filter, n_img, reps, s, cv, cn, cc, run, h_entries, max_entries, n_entries);
 }
 
 int rta_autotune_stream(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, const rta_segment_t* d_seg,
@@ -804,7 +827,7 @@ int rta_autotune_stream(rta_ctx* c, const uint8_t* d_stream, int64_t n_bytes, co
                          max_img, pp, nullptr, nullptr, 0, d_hillas, 0, s, nullptr, d_counts + 1, d_seg, d_img_seg,
                          max_seg, static_cast<rta::StreamImg*>(c->d_smeta));
     };
-    rc = tune_sweep(c, rta::CHAIN_STREAM, max_img, reps, s, &c->st_variant, &c->st_nstage, &c->st_ctas_per_sm, run,
+    rc = tune_sweep(c, rta::CHAIN_STREAM, false, max_img, reps, s, &c->st_variant, &c->st_nstage, &c->st_ctas_per_sm, run,
                     h_entries, max_entries, n_entries);
     if (rc && st_before < 0) c->st_variant = -1;
     return rc;

@@ -7,6 +7,9 @@
 
 namespace rta {
 
+constexpr int SMALL_TAILS = 8;
+constexpr int SMALL_PIX = 512;      // pixels of the largest camera that counts as small
+
 struct ChainArgs {
     DevArray arr;
     ProcParams pp;
@@ -29,7 +32,7 @@ struct ChainArgs {
     int nstage;
     int max_S;               // longest rows of the array's cameras
     int integrate_only;
-    int n_sm;                // of the device
+    int small;               // the form for small cameras, of SMALL_TAILS slots and tail warps
     int search;              // SEARCH_*: what some camera without a specialised window search needs
     // a byte-stream bundle (rta_ingest's directory): wave is the stream, wave_off unused;
     // smeta: one prepared record per image (k_stream_meta)

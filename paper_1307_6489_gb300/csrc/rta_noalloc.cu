@@ -190,7 +190,6 @@ extern "C" int rta_image_chain_noalloc(const rta_camera_desc_t* h_cams, int n_ca
     a.max_S = max_S;
     a.nstage = nstage;
     a.integrate_only = 0;
-    a.n_sm = n_sm;
     for (int t = 0; t < n_tel; ++t)
         a.search = rta::search_of_both(a.search, rta::window_search(a.pp, cams[h_tel_cam[t]].S, true));
     NA_TRY(rta::launch_image_chain(variant, a, int(grid), smem, s));

@@ -636,3 +636,65 @@ def test_stage_calls_on_more_images_than_fit_at_once(P, core_nb):
     rows = np.array([oracle.hillas(xy, q[i], t[i], ref[i]) for i in range(kinds)])
     compare_hillas(hillas_rows(out[: kinds * 16], kinds), rows, f"stages {P}")
     ctx.close()
+
+
+def test_small_cameras_run_with_the_ctas_that_the_configuration_names():
+    """Up to two CTAs per SM, and by default two, variant 4 keeps eight image slots for cameras of at
+    most 512 pixels; the configuration reports what is launched, and the rows do not depend on it."""
+    P, S, W = 256, 16, 5
+    rng = np.random.default_rng(5)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    xy, nb = synth.lattice("square", P, 0.1)
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                       np.full(P, 1 / 128, np.float32))
+    n = 4 * n_sm
+    wave = torch.from_numpy(rng.integers(380, 480, n * P * S).astype(np.int16)).cuda()
+    off = torch.arange(n, dtype=torch.int64, device="cuda") * (P * S)
+    tel = torch.zeros(n, dtype=torch.int32, device="cuda")
+    seen, rows = {}, {}
+    for config in (None, (4, 2, 0), (4, 2, 1), (4, 2, 2), (4, 2, 3), (0, 3, 2)):
+        if config:
+            ctx.set_chain_config(*config)
+        seen[config] = ctx.chain_config()
+        for n_img in (7, n_sm, 2 * n_sm + 1, n):
+            out = torch.full((n_img * 16,), -1.0, device="cuda")
+            ctx.image_chain(wave, off[:n_img], tel[:n_img], rta.RTA_WINDOW_SLIDING, 0, W, 3.0, 1.5, 1, out)
+            assert ctx.check() == 0
+            want = rows.setdefault(n_img, out)
+            assert torch.equal(out.view(torch.int32), want.view(torch.int32)), (config, n_img)
+    for config, ctas in ((None, 2), ((4, 2, 0), 2), ((4, 2, 1), 1), ((4, 2, 2), 2), ((4, 2, 3), 3), ((0, 3, 2), 2)):
+        assert seen[config]["ctas_per_sm"] == ctas and seen[config]["grid"] == ctas * n_sm, config
+    assert seen[(4, 2, 1)]["smem_bytes"] == seen[None]["smem_bytes"] > seen[(4, 2, 3)]["smem_bytes"]
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_img_of_sm", [0.25, 3])
+def test_autotuning_a_small_bundle_measures_what_it_records(n_img_of_sm):
+    """Tuned on an image per SM at most, the launches that were measured are the ones made afterwards
+    (no deeper pipeline in their place); the rows are the untuned ones, there and on more images."""
+    P, S, W = 1000, 40, 6
+    rng = np.random.default_rng(6)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    xy, nb = synth.lattice("hex", P, 0.1)
+    n_img = int(n_img_of_sm * n_sm)
+    wave = torch.from_numpy(rng.integers(380, 480, n_img * P * S).astype(np.int16)).cuda()
+    off = torch.arange(n_img, dtype=torch.int64, device="cuda") * (P * S)
+    tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
+    ctx = rta.Context(0)
+    ctx.register_camera(5, xy, nb, S)
+    ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
+                       np.full(P, 1 / 128, np.float32))
+    args = (rta.RTA_WINDOW_SLIDING, 0, W, 3.0, 1.5, 1)
+    ref, out = torch.zeros(n_img * 16, device="cuda"), torch.zeros(n_img * 16, device="cuda")
+    ctx.image_chain(wave, off, tel, *args, ref)
+    table = ctx.autotune(wave, off, tel, *args, out, reps=1)
+    assert torch.equal(out.view(torch.int32), ref.view(torch.int32))
+    for e in table:
+        assert e["grid"] == min(n_img, e["ctas_per_sm"] * n_sm)
+    out.zero_()
+    ctx.image_chain(wave, off, tel, *args, out)
+    assert ctx.check() == 0
+    assert torch.equal(out.view(torch.int32), ref.view(torch.int32))
+    ctx.close()
