@@ -297,8 +297,8 @@ def test_rows_do_not_depend_on_the_search_that_the_array_takes(mode, S, W):
     ("square", 2049, 128, 112, 16), ("hex", 130, 128, 0, 7), ("square", 1600, 100, 9, 6), ("hex", 1000, 48, 40, 8)])
 def test_fixed_window_of_long_rows(kind, P, S, start, W):
     """The fixed window on rows of a multiple of 32 samples (chunks in padded runs, from 64 samples
-    two threads a row) and on their neighbours: decisions exact, rows within the usual rules, the
-    same through every tile shape and with one CTA an SM, samples up to full scale."""
+    two threads a row; four samples and more) and on their neighbours: decisions exact, rows within
+    the usual rules, the same through every tile shape, samples up to full scale."""
     rng = np.random.default_rng(100 * S + start)
     xy, nb = synth.lattice(kind, P, 0.1)
     n_img = 7
@@ -338,35 +338,53 @@ def test_fixed_window_of_long_rows(kind, P, S, start, W):
     ctx.close()
 
 
-@pytest.mark.parametrize("P,S,W", [(256, 16, 5), (331, 40, 6), (1855, 40, 6), (1600, 100, 6)])
-def test_rows_do_not_depend_on_the_launch_size(P, S, W):
+@pytest.mark.parametrize("P,S,W,start", [
+    (256, 16, 5, -1), (331, 40, 6, -1), (1855, 40, 6, -1), (1600, 100, 6, -1),
+    # chunks in padded runs, one thread a row and two: sliding, and the fixed window from `start`
+    (331, 32, 6, -1), (264, 48, 16, -1), (1000, 64, 5, -1), (2049, 128, 16, -1), (130, 112, 9, -1),
+    (331, 32, 4, 13), (512, 32, 16, 16), (1000, 64, 8, 28), (257, 96, 5, 40), (2049, 128, 16, 56)])
+def test_rows_do_not_depend_on_the_launch_size(P, S, W, start):
     """Launches of up to an image per SM (a deeper pipeline), up to the resident CTAs (no counter
-    reset) and beyond: each image's row is the one it has alone, call after call."""
-    rng = np.random.default_rng(P)
-    kind = "square" if P == 256 else "hex"
+    reset) and beyond, images of different brightness in turn (a slot's bitmaps are left zero by
+    one for the next, and its stages reused): each image's row is the one it has alone, call after call."""
+    rng = np.random.default_rng(P + S)
+    kind = "square" if P in (256, 512) else "hex"
     xy, nb = synth.lattice(kind, P, 0.1)
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
     kinds = 5                                        # distinct images, repeated
     wave = rng.integers(380, 421, (kinds, P, S)).astype(np.uint16)
     for i in range(kinds):
         d = ((xy - xy[rng.integers(P)]) ** 2).sum(1)
-        wave[i, :, S // 2] += (300 * (i + 1) * np.exp(-d / 0.03)).astype(np.uint16)
+        wave[i, :, S // 2 if start < 0 else start + W // 2] += (300 * (i + 1) * np.exp(
+            -d / (0.03 + 0.1 * (i % 2)))).astype(np.uint16)
+    wave[2] = rng.integers(380, 390, (P, S))         # one with nothing to clean away
     ctx = rta.Context(0)
     ctx.register_camera(5, xy, nb, S)
     ctx.register_array(np.array([5], np.int32), np.zeros((1, 2), np.float32), np.full(P, 6400, np.int32),
                        np.full(P, 1 / 128, np.float32))
     d_wave = torch.from_numpy(wave.reshape(-1).view(np.int16)).cuda()
-    single = None
-    for n_img in (kinds, n_sm - 1, n_sm, n_sm + 1, 2 * n_sm, 2 * n_sm + 1, 3 * n_sm, 3 * n_sm + 1, 5 * n_sm, 3, n_sm):
-        off = (torch.arange(n_img, dtype=torch.int64, device="cuda") % kinds) * (P * S)
-        tel = torch.zeros(n_img, dtype=torch.int32, device="cuda")
-        out = torch.full((n_img * 16,), -1.0, dtype=torch.float32, device="cuda")
-        ctx.image_chain(d_wave, off, tel, rta.RTA_WINDOW_SLIDING, 0, W, 10.0, 5.0, 1, out)
+    mode = (rta.RTA_WINDOW_SLIDING, 0) if start < 0 else (rta.RTA_WINDOW_FIXED, start)
+
+    def rows(order):
+        off = torch.from_numpy(np.asarray(order, np.int64) * (P * S)).cuda()
+        tel = torch.zeros(len(off), dtype=torch.int32, device="cuda")
+        out = torch.full((len(off) * 16,), -1.0, dtype=torch.float32, device="cuda")
+        ctx.image_chain(d_wave, off, tel, *mode, W, 10.0, 5.0, 1, out)
         assert ctx.check() == 0
-        raw = out.cpu().numpy().view(np.uint32).reshape(n_img, 16)
-        if single is None:
-            single = raw
-        np.testing.assert_array_equal(raw, single[np.arange(n_img) % kinds])
+        return out.cpu().numpy().view(np.uint32).reshape(-1, 16)
+
+    single = np.concatenate([rows([i]) for i in range(kinds)])
+    assert (single[:, 10] > 0).sum() >= 3 and single[2, 10] == 0
+    for n_img in (kinds, n_sm - 1, n_sm, n_sm + 1, 2 * n_sm, 2 * n_sm + 1, 3 * n_sm, 3 * n_sm + 1, 5 * n_sm, 3, n_sm):
+        order = np.arange(n_img) % kinds if n_img % 2 else rng.integers(0, kinds, n_img)
+        np.testing.assert_array_equal(rows(order), single[order])
+    for config in ((4, 2, 1), (0, 2, 1), (1, 2, 1), (3, 3, 1)):      # one CTA an SM: every slot many times over
+        try:
+            ctx.set_chain_config(*config)
+        except rta.RtaError:
+            continue                                 # no room for this camera
+        order = rng.integers(0, kinds, 9 * n_sm)
+        np.testing.assert_array_equal(rows(order), single[order])
     ctx.close()
 
 
