@@ -145,3 +145,41 @@ def f32_rows_as_oracle(buf):
     ref[:, H["n_pix"]] = ib[:, 10]
     ref[:, H["flags"]] = ib[:, 11]
     return ref
+
+
+def custom_workload(cameras, W, mode="sliding", n_evt=60, seed=1):
+    """Events of one image per telescope, a telescope per camera of [(kind, P, S), ...]: pedestal noise, a
+    bright blob in most images, samples to full scale in some. mode: sliding, filter or nbpeak."""
+    import synth
+    rng = np.random.default_rng(seed)
+    cams = {}
+    for c, (kind, P, S) in enumerate(cameras):
+        xy, nb = synth.lattice(kind, P, 0.1)
+        cams[c] = synth.Camera(c, P, S, nb.shape[1], 0.1, 0.01, 100.0, xy, nb)
+    n_tel = len(cams)
+    tel = np.tile(np.arange(n_tel, dtype=np.int32), n_evt)
+    pix = np.array([cams[int(t)].n_pix for t in tel], np.int64)
+    samples = pix * [cams[int(t)].n_samples for t in tel]
+    wave = []
+    for i, t in enumerate(tel):
+        cam = cams[int(t)]
+        w = rng.integers(385, 416, (cam.n_pix, cam.n_samples))
+        if i % 5:
+            d = ((cam.xy - cam.xy[rng.integers(cam.n_pix)]) ** 2).sum(1)
+            k0 = rng.integers(0, cam.n_samples, cam.n_pix) if i % 3 == 0 else rng.integers(0, cam.n_samples)
+            w[np.arange(cam.n_pix), k0] += (rng.uniform(100, 2000) * np.exp(-d / 0.05)).astype(np.int64)
+        if i % 11 == 0:
+            w[rng.integers(cam.n_pix), rng.integers(cam.n_samples)] = [4095, 4096, 65535][i % 3]
+        wave.append(w.astype(np.uint16).reshape(-1))
+    rows = sum(c.n_pix for c in cams.values())
+    weights = tuple(int(k) for k in 1 + np.arange(W) % 4) if mode == "filter" else None
+    proc = synth.Processing(True, 0, W, 6.0, 3.0, True, weights, mode == "nbpeak")
+    zero = np.zeros
+    return synth.Workload(
+        -1, seed, proc, cams, np.arange(n_tel, dtype=np.int32), rng.uniform(-100, 100, (n_tel, 2)).astype(np.float32),
+        np.concatenate([[0], np.cumsum([c.n_pix for c in cams.values()])]).astype(np.int64), zero(rows), zero(rows),
+        rng.integers(16 * 399, 16 * 401, rows).astype(np.int32),
+        (rng.uniform(0.9, 1.1, rows) / (128 if mode != "filter" else 320)).astype(np.float32),
+        (np.arange(n_evt + 1) * n_tel).astype(np.int32), tel, np.repeat(np.arange(n_evt, dtype=np.int32), n_tel),
+        (np.cumsum(samples) - samples).astype(np.int64), np.concatenate([[0], np.cumsum(pix)]).astype(np.int64),
+        zero((len(tel), 3, 6), np.float32), zero(len(tel), np.int32), zero((n_evt, 8)), np.concatenate(wave))

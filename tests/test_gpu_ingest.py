@@ -12,7 +12,7 @@ import synth
 import paper_1307_6489_gb300 as rta
 from oracle import ingest
 
-from gpu_helpers import Dev, compare_hillas, hillas_rows, make_ctx, proc_args
+from gpu_helpers import T_ABS, Dev, compare_hillas, custom_workload, hillas_rows, make_ctx, proc_args
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -347,4 +347,36 @@ def test_a_shorter_stream_needs_no_larger_workspace(sset):
     c = d.counts.cpu().numpy()
     assert (int(c[0]), int(c[1]), int(c[2]), int(c[4])) == (len(want["seg"]), len(want["img_tel"]),
                                                             len(want["evt_number"]), 0)
+    ctx.close()
+
+
+@pytest.mark.parametrize("cameras,W", [
+    ([("hex", 264, 50)], 3), ([("hex", 200, 31), ("square", 520, 100)], 12),             # the serial search
+    ([("hex", 264, 48)], 5), ([("square", 520, 128), ("hex", 136, 17)], 16),             # the packed one
+    ([("hex", 1856, 40), ("hex", 264, 104), ("square", 1032, 25)], 8)])
+@pytest.mark.parametrize("mode", ["sliding", "filter", "nbpeak"])
+def test_cameras_without_a_compiled_search_like_the_oracle(cameras, W, mode):
+    """Every window mode on cameras that take the packed search or the serial one: charges and masks bit
+    for bit and rows within the usual rules against the oracle, contiguous and as a byte stream (the
+    same rows), with segments that end inside the chunks."""
+    wl = custom_workload(cameras, W, mode)
+    ref = oracle.reconstruct(wl, per_pixel=True, do_stereo=False)
+    ctx = make_ctx(wl)
+    dev = Dev(wl)
+    m, start, W, t_hi, t_lo, core_nb = proc_args(wl)
+    q = torch.full((dev.n_pix,), np.nan, dtype=torch.float32, device="cuda")
+    t = torch.full_like(q, np.nan)
+    ctx.calibrate_integrate(dev.wave, dev.wave_off, dev.img_tel, dev.pix_off, m, start, W, q, t)
+    mask = torch.full((dev.n_pix,), 7, dtype=torch.uint8, device="cuda")
+    hm = dev.hillas_buf()
+    ctx.image_chain_masks(dev.wave, dev.wave_off, dev.img_tel, dev.pix_off, m, start, W, t_hi, t_lo, core_nb, mask, hm)
+    assert ctx.check() == 0
+    np.testing.assert_array_equal(q.cpu().numpy().view(np.uint32), ref["q"].view(np.uint32))
+    assert np.max(np.abs(t.cpu().numpy() - ref["t"])) <= T_ABS
+    np.testing.assert_array_equal(mask.cpu().numpy(), ref["mask"])
+    segments = {c: 8 * max(1, cam.n_pix // 48) for c, cam in wl.cams.items()}
+    h0, s0, h1, s1, _, _ = reconstruct_both(wl, ctx, segments)
+    assert torch.equal(h0, h1) and torch.equal(s0, s1) and torch.equal(h0, hm)
+    compare_hillas(hillas_rows(h0, wl.n_img), ref["hillas"], f"{cameras} {mode}")
+    assert (ref["hillas"][:, oracle.H["n_pix"]] > 0).mean() > 0.3
     ctx.close()
