@@ -24,7 +24,6 @@
 namespace rta {
 
 constexpr int NCW = 8;             // warps of the block-wide (unfused) kernels
-constexpr int NCT = NCW * 32;
 constexpr int MAX_STAGES = 8;
 
 enum { HDR_LAST = 1, HDR_BAD = 2, HDR_END = 4 };
@@ -437,9 +436,6 @@ __device__ __forceinline__ float peak_time(const uint16_t* row, int st, int W, i
 // integration. Thread w owns word w and visits its bits in increasing order, and
 // partial sums are combined by a fixed tree: the summation order depends only on
 // the camera, never on the data or on the rest of the batch.
-struct NamedBar {
-    __device__ __forceinline__ void operator()() const { named_bar_sync(1, NCT); }
-};
 struct BlockBar {
     __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };

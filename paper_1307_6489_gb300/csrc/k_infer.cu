@@ -900,17 +900,7 @@ cudaError_t launch_infer(const InferArgs& a, int n_sm, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     // one CTA per SM, with at least 16 events each on average
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_sm, a.f.n_evt / 16));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(grid));
-    cfg.blockDim = dim3(NT);
-    cfg.dynamicSmemBytes = S_TOTAL;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_deepsets_infer, a);
+    return launch_dependent(k_deepsets_infer, unsigned(grid), NT, S_TOTAL, s, a);
 }
 
 }  // namespace rta

@@ -161,17 +161,7 @@ cudaError_t launch_stereo(StereoArgs a, int n_sm, cudaStream_t s) {
     const int64_t wave = int64_t(n_sm) * ST_CTAS;
     a.per_cta = int(std::max<int64_t>(1, std::min<int64_t>(ST_MAX_E, (a.n_evt + wave - 1) / wave)));
     const int64_t grid = std::min<int64_t>((a.n_evt + a.per_cta - 1) / a.per_cta, int64_t(n_sm) * 16);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(std::max<int64_t>(grid, 1)));
-    cfg.blockDim = dim3(ST_NT);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_stereo, a);
+    return launch_dependent(k_stereo, unsigned(std::max<int64_t>(grid, 1)), ST_NT, 0, s, a);
 }
 
 }  // namespace rta

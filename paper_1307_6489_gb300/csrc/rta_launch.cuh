@@ -330,8 +330,9 @@ cudaError_t smem_opt_in(K* kern, std::atomic<uint64_t>& done) {
     return e;
 }
 
-// The kernels of a training step, and those of an ingest, are launched as programmatic dependents
-// of one another: each signals at once, and waits (grid_dependency_wait) before it reads anything.
+// A launch as a programmatic dependent of the kernel before it on the stream: a training step's
+// kernels after its first, those of an ingest, the stereo, lookup and inference kernels. Each waits
+// (grid_dependency_wait) before it reads what that kernel writes.
 template <class... P, class... A>
 cudaError_t launch_dependent(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};

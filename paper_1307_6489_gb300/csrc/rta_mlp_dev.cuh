@@ -7,28 +7,10 @@
 
 namespace rta {
 
-// D = A B + D on the tensor cores: one m16n8k16 tile, BF16 operands, FP32 accumulators.
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
 __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi) {
     return uint32_t(__bfloat16_as_ushort(lo)) | (uint32_t(__bfloat16_as_ushort(hi)) << 16);
-}
-
-// B fragment of the output layer (256 x 4, BF16, row-major) for k-step ks,
-// widened to n = 8 with zero columns.
-__device__ __forceinline__ void head_b_fragment(const __nv_bfloat16* __restrict__ V2b, int ks, int gq, int tq,
-                                                uint32_t (&b)[2]) {
-    const int k = 16 * ks + 2 * tq;
-    b[0] = gq < 4 ? pack_bf16(V2b[k * 4 + gq], V2b[(k + 1) * 4 + gq]) : 0u;
-    b[1] = gq < 4 ? pack_bf16(V2b[(k + 8) * 4 + gq], V2b[(k + 9) * 4 + gq]) : 0u;
 }
 
 // An image takes part in the network when cleaning kept at least three pixels.
