@@ -205,7 +205,8 @@ __device__ __forceinline__ void best_key_pair(const uint16_t* row0, int one, int
 // out of the instruction caches. U starts at a time: their loads are under way together, of up to U
 // samples past the row's end (a stage has them; a window that reaches there is never the first).
 // With 2 % of the pixels above t_lo, 4,000 images of 1855 x 40 127 us, 138 one start at a time (167
-// and 185 with the neighbour-peak window); with 0.2 % 103 and 104.
+// and 185 with the neighbour-peak window); with 0.2 % 103 and 104. (One at a time in the kernels
+// with per-pixel outputs, whose code is larger: masks of 4,000 images of 1855 x 40, W = 10, 232 us, 254.)
 template <int U>
 __device__ __forceinline__ int first_start(const uint16_t* row, int S, int W, int sum, int st = 0) {
     int s = 0;
@@ -955,7 +956,7 @@ __device__ __forceinline__ void integrate_chunk(const ChainArgs& a, const ProcPa
                     if (!done) {
                         if (!integ && !filt && m > 0) {
                             sum = m;
-                            wst = first_start<4>(row, S, W, m);
+                            wst = first_start<FILTER == 2 ? 1 : 4>(row, S, W, m);
                         } else {
                             int key;
                             if constexpr (!INTEG && FILTER == 0) key = best_key_serial(row, S, W);

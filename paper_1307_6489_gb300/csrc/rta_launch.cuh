@@ -49,11 +49,14 @@ struct ChainArgs {
 //
 // The serial search is bound by its shared loads, and those by the banks that a warp's rows share:
 // two rows a bank when S % 8 is 2, 4 or 6, four when it is 0 and S / 8 is odd, else more. With one
-// or two it is the faster one, for every output: on 0.2 GB of 1000-pixel images, W = 4, packed and
-// serial 1.41 times apart at 20 samples, 1.27 at 31, 1.18 at 50, 1.13 at 60, 1.20 at 100, 1.11 at
-// 127 (charges alone 1.8 to 1.13); with four, 1.05 at 24 samples (with the filter 0.94), 0.83 at 56
-// and 0.73 at 104; with more, 0.85 at 16, 0.51 at 48, 0.12 at 128. Windows of one sample are
-// cheaper packed in long rows (0.91 at 65 and 100 samples).
+// or two it is the faster one as a rule, for every output and whatever the images: 0.2 GB of
+// 1000-pixel images, W = 4, 1 % of the pixels above t_lo (in brackets nearly all), the packed
+// search's time over the serial one's 1.60 (1.41) at 20 samples, 1.38 (1.27) at 31, 1.34 (1.18) at 50,
+// 1.06 (1.13) at 60, 1.03 (1.20) at 100, 0.95 (1.11) at 127. With four, 0.94 (1.05) at 24 samples,
+// 0.62 (0.83) at 56 and 0.55 (0.73) at 104; with more, 0.70 (0.85) at 16, 0.34 (0.51) at 48, 0.08
+// (0.12) at 128. The neighbour peak forms 64-bit keys beside it and gains less from the packed
+// search: 1.05 at 24 samples, 1.04 at 16, with W = 16 1.20 at 40 and 1.09 at 56. Windows of one sample are cheaper packed in long rows
+// (0.93 at 65 samples, 0.90 at 100).
 //
 // A fixed window needs no search, but rows of a multiple of 32 samples put a warp's loads on two
 // banks or one, and the packed kernels' padded runs spread them: 8 samples of 1000 pixels x 32
@@ -66,7 +69,8 @@ inline int window_search(const ProcParams& pp, int S, bool rows) {
     const bool width = pp.W == 6 || (rows && !pp.nbpeak && !pp.filter && pp.W >= 4 && pp.W <= 8);
     if ((width && (S == 40 || S == 30 || S == 25)) || (pp.W == 5 && S == 16 && !pp.nbpeak)) return SEARCH_OWN;
     if (pp.W == 1 && S >= 64) return SEARCH_PACKED;
-    return S % 8 != 0 || (S % 16 == 8 && S <= 24 && !pp.filter) ? SEARCH_SERIAL : SEARCH_PACKED;
+    if (pp.nbpeak && (S <= 24 || (S % 16 == 8 && 4 * pp.W >= S))) return SEARCH_SERIAL;
+    return S % 8 != 0 ? SEARCH_SERIAL : SEARCH_PACKED;
 }
 
 // The search of a launch with cameras of both: the serial search loses far more on the other's rows
